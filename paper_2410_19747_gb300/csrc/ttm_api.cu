@@ -1125,9 +1125,7 @@ ttm_status ttm_gemm(ttm_handle* h, ttm_precision prec, int64_t M, int64_t N, int
     RawGemmFn f{t, (int)M, (int)N, (int)K, A, (long)lda, B, (long)ldb, C, (long)ldc};
     cudaStream_t st = h->s.stream;
     if (prec == TTM_PREC_FP64) {
-      dim3 grid((unsigned)((N + GT - 1) / GT), (unsigned)((M + GT - 1) / GT), 1);
-      dgemm_kernel<RawGemmFn><<<grid, 256, 0, st>>>(f, 1);
-      TTM_CUDA(cudaGetLastError());
+      TTM_CUDA(launch_dgemm(st, f, 1, 1, (int)M, (int)N, (int)K, h->s.num_sms));
     } else {
       const int S = h->s.opt.split_digits > 0 ? h->s.opt.split_digits : kOzMaxS;
       const size_t need = tc_ws_bytes(1, (int)M, (int)N, (int)K, S) + 256;

@@ -206,9 +206,8 @@ class Engine {
           throw Error(TTM_ERR_CUDA, std::string("tensor-core GEMM, ") + tc_failed_step() + ": " + cudaGetErrorString(e));
         launches_ += 6;
       } else {
-        dim3 grid(cdiv(N_ub, GT), cdiv(M_ub, GT), (unsigned)(Z_ * nbatch));
-        dgemm_kernel<F><<<grid, 256, 0, hs_.stream>>>(f, nbatch, d_stat_ + ST_GFLOPS, tab_.ns);
-        TTM_CUDA(cudaGetLastError());
+        TTM_CUDA(launch_dgemm(hs_.stream, f, Z_ * nbatch, nbatch, M_ub, N_ub, K_ub, hs_.num_sms, d_stat_ + ST_GFLOPS,
+                              tab_.ns));
         ++launches_;
       }
     });

@@ -66,9 +66,7 @@ struct EnvRunner {
     for (long b0 = 0; b0 < nb; b0 += 65535) {
       const int cnt = (int)std::min<long>(65535, nb - b0);
       GenFn f{M, N, K, nb2, (int)b0, A, B, C, alpha, beta};
-      dim3 grid((N + GT - 1) / GT, (M + GT - 1) / GT, cnt);
-      dgemm_kernel<GenFn><<<grid, 256, 0, hs.stream>>>(f, cnt);
-      TTM_CUDA(cudaGetLastError());
+      TTM_CUDA(launch_dgemm(hs.stream, f, cnt, cnt, M, N, K, hs.num_sms));
       ++launches;
     }
   }
@@ -89,17 +87,29 @@ struct TTv {
   View at_t(int k) const { return View{c[k], D[k + 1], D[k], 1, (long)D[k + 1], (long)d * D[k + 1]}; }  // l <-> r
 };
 
+// The last contraction of a step sums over (l, s) of one core. In both kinds of view these two
+// legs lie at one stride (l outer, s inner of a core; s outer, l inner of its transpose), so the
+// sum is one GEMM with K = d Dl when the other operand holds its rows in the same order: row
+// (l, s) at l * lo + s * so rows.
+struct Fold {
+  long k;       // stride of the joint index in the core
+  long lo, so;  // row offsets of l and s in the other operand
+};
+static Fold fold(const View& v, int d) {
+  if (v.cl == (long)d * v.cs) return Fold{v.cs, d, 1};
+  return Fold{v.cl, 1, v.Dl};  // v.cs == Dl * v.cl
+}
+
 // ---------------------------------------------------------------- two layers
 
 // E'[x', y'] = sum_{x, y, s} E[x, y] X[x, s, x'] Y[y, s, y'].  T: Dx * d * Dy'.
 static void env2_step(EnvRunner& r, int d, const double* E, View X, View Y, double* T, double* En) {
-  // T[s][x][y'] = sum_y E[x, y] Y[y, s, y']              (batch s)
+  const Fold f = fold(X, d);
+  // T[(x, s)][y'] = sum_y E[x, y] Y[y, s, y']             (batch s; rows in the order of X's legs)
   r.gemm(X.Dl, Y.Dr, Y.Dl, 1, d, op(E, Y.Dl, 1), op(Y.p, Y.cl, Y.cr, 0, Y.cs),
-         out(T, Y.Dr, 1, 0, (long)X.Dl * Y.Dr));
-  // E'[x', y'] = sum_s sum_x X[x, s, x'] T[s][x][y']
-  for (int s = 0; s < d; ++s)
-    r.gemm(X.Dr, Y.Dr, X.Dl, 1, 1, op(X.p + s * X.cs, X.cr, X.cl), op(T + (long)s * X.Dl * Y.Dr, Y.Dr, 1),
-           out(En, Y.Dr, 1), 1.0, s == 0 ? 0.0 : 1.0);
+         out(T, f.lo * Y.Dr, 1, 0, f.so * Y.Dr));
+  // E'[x', y'] = sum_(x, s) X[x, s, x'] T[(x, s)][y']
+  r.gemm(X.Dr, Y.Dr, d * X.Dl, 1, 1, op(X.p, X.cr, f.k), op(T, Y.Dr, 1), out(En, Y.Dr, 1));
 }
 
 // ---------------------------------------------------------------- three layers (W, A, B)
@@ -111,15 +121,13 @@ static void env3_step(EnvRunner& r, int d, const double* E, View W, View A, View
   // T1[s][(w, a)][b'] = sum_b E[(w, a), b] B[b, s, b']    (batch s)
   r.gemm(W.Dl * A.Dl, B.Dr, B.Dl, 1, d, op(E, B.Dl, 1), op(B.p, B.cl, B.cr, 0, B.cs),
          out(T1, B.Dr, 1, 0, (long)W.Dl * A.Dl * B.Dr));
-  // T2[s][w][a'][b'] = sum_a A[a, s, a'] T1[s][w][a][b']  (batch (s, w))
+  const Fold f = fold(W, d);
+  const long q = (long)A.Dr * B.Dr;
+  // T2[(w, s)][a'][b'] = sum_a A[a, s, a'] T1[s][w][a][b'] (batch (s, w); rows in the order of W's legs)
   r.gemm(A.Dr, B.Dr, A.Dl, d, W.Dl, op(A.p, A.cr, A.cl, A.cs, 0),
-         op(T1, B.Dr, 1, (long)W.Dl * A.Dl * B.Dr, (long)A.Dl * B.Dr),
-         out(T2, B.Dr, 1, (long)W.Dl * A.Dr * B.Dr, (long)A.Dr * B.Dr));
-  // E'[w'][(a', b')] = sum_s sum_w W[w, s, w'] T2[s][w][(a', b')]
-  for (int s = 0; s < d; ++s)
-    r.gemm(W.Dr, A.Dr * B.Dr, W.Dl, 1, 1, op(W.p + s * W.cs, W.cr, W.cl),
-           op(T2 + (long)s * W.Dl * A.Dr * B.Dr, (long)A.Dr * B.Dr, 1), out(En, (long)A.Dr * B.Dr, 1), 1.0,
-           s == 0 ? 0.0 : 1.0);
+         op(T1, B.Dr, 1, (long)W.Dl * A.Dl * B.Dr, (long)A.Dl * B.Dr), out(T2, B.Dr, 1, f.so * q, f.lo * q));
+  // E'[w'][(a', b')] = sum_(w, s) W[w, s, w'] T2[(w, s)][(a', b')]
+  r.gemm(W.Dr, (int)q, d * W.Dl, 1, 1, op(W.p, W.cr, f.k), op(T2, q, 1), out(En, q, 1));
 }
 
 // G[a, s, a'] (+)= alpha * sum E[w, a, b] W[w, s, w'] B[b, s, b'] R[w', a', b'] for the core A_k
@@ -151,14 +159,13 @@ static void env4_step(EnvRunner& r, int d, const double* E, View A, View B, doub
   // S2[s][(a, x)][b'][y'] = sum_b B[b, s, b'] S1[s][(a, x)][b][y']    (batch (s, (a, x)))
   r.gemm(Dbp, Dbp, Db, d, (int)ab, op(B.p, B.cr, B.cl, B.cs, 0), op(T1, Dbp, 1, ab * Db * Dbp, (long)Db * Dbp),
          out(T2, Dbp, 1, ab * Dbp * Dbp, (long)Dbp * Dbp));
-  // S3[s][a][x'][(b', y')] = sum_x A[x, s, x'] S2[s][a][x][(b', y')] (batch (s, a))
+  const Fold f = fold(A, d);
+  // S3[(a, s)][x'][(b', y')] = sum_x A[x, s, x'] S2[s][a][x][(b', y')] (batch (s, a); rows in A's order)
   const long q = (long)Dbp * Dbp;
   r.gemm(Dap, (int)q, Da, d, Da, op(A.p, A.cr, A.cl, A.cs, 0), op(T2, q, 1, ab * q, (long)Da * q),
-         out(T1, q, 1, (long)Da * Dap * q, (long)Dap * q));
-  // E'[a'][(x', b', y')] = sum_s sum_a A[a, s, a'] S3[s][a][(x', b', y')]
-  for (int s = 0; s < d; ++s)
-    r.gemm(Dap, (int)(Dap * q), Da, 1, 1, op(A.p + s * A.cs, A.cr, A.cl),
-           op(T1 + (long)s * Da * Dap * q, (long)Dap * q, 1), out(En, (long)Dap * q, 1), 1.0, s == 0 ? 0.0 : 1.0);
+         out(T1, q, 1, f.so * Dap * q, f.lo * Dap * q));
+  // E'[a'][(x', b', y')] = sum_(a, s) A[a, s, a'] S3[(a, s)][(x', b', y')]
+  r.gemm(Dap, (int)(Dap * q), d * Da, 1, 1, op(A.p, A.cr, f.k), op(T1, (long)Dap * q, 1), out(En, (long)Dap * q, 1));
 }
 
 // G[x, s, x'] (+)= alpha * sum E[a, x, b, y] A[a, s, a'] B[b, s, b'] B[y, s, y'] R[a', x', b', y']:
@@ -175,10 +182,10 @@ static void adjoint4(EnvRunner& r, int d, const double* E, const double* R, View
   // S3[s][x][a'][(b', y')] = sum_a A[a, s, a'] S2[s][a][x][(b', y')]  (batch (s, x))
   r.gemm(Dap, (int)q, Da, d, Da, op(A.p, A.cr, A.cl, A.cs, 0), op(T2, (long)Da * q, 1, ab * q, q),
          out(T1, q, 1, (long)Da * Dap * q, (long)Dap * q));
-  // G[x, s, x'] = sum_a' sum_(b', y') S3[s][x][a'][(b', y')] R[a'][x'][(b', y')]   (batch s)
-  for (int a = 0; a < Dap; ++a)
-    r.gemm(Da, Dap, (int)q, 1, d, op(T1 + (long)a * q, (long)Dap * q, 1, 0, (long)Da * Dap * q),
-           op(R + (long)a * Dap * q, 1, q), out(G, (long)d * Dap, 1, 0, Dap), alpha, a == 0 ? beta : 1.0);
+  // G[x, s, x'] = sum_(a', b', y') S3[s][x][(a', b', y')] R[x'][(a', b', y')]   (batch s; R is
+  // symmetric in its two A layers, so its x' rows hold (a', b', y') contiguously)
+  const int kq = (int)(Dap * q);
+  r.gemm(Da, Dap, kq, 1, d, op(T1, kq, 1, 0, (long)Da * kq), op(R, 1, kq), out(G, (long)d * Dap, 1, 0, Dap), alpha, beta);
 }
 
 // ---------------------------------------------------------------- drivers

@@ -7,11 +7,21 @@
 // is ever materialised. A functor F maps (z, b) to the problem, reading the bond
 // table, so sizes are the realised ones.
 //
-// Tile: 64 x 64 outputs per CTA, K panels of 16, 256 threads with a 4 x 4 register
-// micro-tile each. On this part float64 runs on a narrow pipe (about 1.1 TFLOP/s
-// for the whole GPU), so the kernel is bound by DFMA issue, not by memory.
+// Bound: the float64 pipe (2 DFMA per clock and SM, about 1.1 TFLOP/s for the whole GPU), not
+// memory; one 64 x 64 x 256 tile is 0.26 ms of one SM's pipe, so what decides the time of the
+// sweep's GEMMs (16 .. 1024 on a side) is over how many SMs the work is spread. Tiles of 16 x 16
+// or 32 x 32 outputs, K panels of 32 prefetched into registers, 256 threads in four groups that
+// split the panel's K (so one CTA alone fills the four sub-partitions), and, where the tiles are
+// fewer than the SMs can hold, up to 8 CTAs of a cluster that split K and add their partial tiles
+// through distributed shared memory in a fixed order. Measured against 64 x 64 tiles without a
+// split (GB300): the GEMMs of a 256 x 256 Swap 133 -> 19 us each, the overlap of two L = 30 trains
+// of bonds 512 and 300 22.6 -> 6.2 ms (1.07 TFLOP/s), a gradient at L = 20, d = 4, chi = 64
+// 172 -> 33 ms; 2048 x 2048 x 1024 runs at 1.23 TFLOP/s.
 #pragma once
+#include <cooperative_groups.h>
 #include "ttm_common.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace ttm {
 
@@ -31,7 +41,9 @@ struct GemmDesc {
   int upper;  // 1: only the output tiles that meet the upper triangle (symmetric results)
 };
 
-constexpr int GT = 64, GK = 16;
+constexpr int kDgK = 32;        // K panel
+constexpr int kDgThreads = 256;
+constexpr int kDgMaxSplit = 8;  // CTAs of a cluster that split K
 
 // Realised flops of one problem (2 M N K; M (M + 1) K for a symmetric Gram whose upper
 // triangle is formed), added by one thread of the problem's first tile when fl is set: a
@@ -49,72 +61,140 @@ struct GemmShape {
   int sym;  // 1: symmetric result, only the upper triangle is counted
 };
 
-template <class F>
-__global__ void __launch_bounds__(256) dgemm_kernel(F f, int nbatch, double* fl = nullptr, int fl_stride = 0) {
+// Grid: x = (M tile * n_tiles + N tile) * split + K part (the parts of a tile are one cluster),
+// z = problems.
+template <class F, int DT>
+__global__ void __launch_bounds__(kDgThreads) dgemm_kernel(F f, int nbatch, int n_tiles, int split, double* fl,
+                                                           int fl_stride) {
   const int z = blockIdx.z / nbatch, bi = blockIdx.z % nbatch;
   const GemmDesc g = f(z, bi);
-  const int m0 = blockIdx.y * GT, n0 = blockIdx.x * GT;
-  if (g.M <= 0 || g.N <= 0 || m0 >= g.M || n0 >= g.N) return;
-  if (m0 == 0 && n0 == 0 && threadIdx.x == 0) gemm_count_flops(fl, fl_stride, z, g);
+  const int rank = blockIdx.x % split, tile = blockIdx.x / split;
+  const int m0 = tile / n_tiles * DT, n0 = tile % n_tiles * DT;
+  if (g.M <= 0 || g.N <= 0 || m0 >= g.M || n0 >= g.N) return;  // uniform over the cluster
+  if (m0 == 0 && n0 == 0 && rank == 0 && threadIdx.x == 0) gemm_count_flops(fl, fl_stride, z, g);
   if (g.upper && m0 > n0) return;
-  __shared__ double As[GK][GT + 1];
-  __shared__ double Bs[GK][GT + 1];
+  constexpr int MI = DT / 8;                 // rows and columns per thread
+  constexpr int LD = DT + 1;
+  constexpr int PER = DT * kDgK / kDgThreads;  // panel elements per thread and operand
+  constexpr int OUT = DT * DT / kDgThreads;    // outputs per thread in the final sum
+  constexpr int kPanels = 2 * kDgK * LD, kPart = 4 * DT * DT;
+  __shared__ double sm[kPanels > kPart ? kPanels : kPart];
+  double* As = sm;                // [kDgK][LD]
+  double* Bs = sm + kDgK * LD;    // [kDgK][LD]
   const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
-  double acc[4][4];
+  const int grp = tid >> 6, tx = tid & 7, ty = (tid >> 3) & 7;
+  // consecutive threads follow the unit stride of the operand when it has one
+  const bool a_kfast = (g.A.cs == 1), b_kfast = (g.B.cs != 1);
+  int per = (g.K + split - 1) / split;
+  per = (per + kDgK - 1) / kDgK * kDgK;
+  const int kbeg = rank * per, kend = min(g.K, kbeg + per);
+  double ra[PER], rb[PER];
+  auto fetch = [&](int k0) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+    for (int u = 0; u < PER; ++u) {
+      const int e = tid + u * kDgThreads;
+      const int mm = a_kfast ? e / kDgK : e % DT, ka = k0 + (a_kfast ? e % kDgK : e / DT);
+      const int nn = b_kfast ? e / kDgK : e % DT, kb = k0 + (b_kfast ? e % kDgK : e / DT);
+      ra[u] = (m0 + mm < g.M && ka < kend) ? g.A.p[(long)(m0 + mm) * g.A.rs + (long)ka * g.A.cs] : 0.0;
+      rb[u] = (n0 + nn < g.N && kb < kend) ? g.B.p[(long)kb * g.B.rs + (long)(n0 + nn) * g.B.cs] : 0.0;
+    }
+  };
+  double acc[MI][MI];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+  for (int i = 0; i < MI; ++i)
+#pragma unroll
+    for (int j = 0; j < MI; ++j) acc[i][j] = 0.0;
+  if (kbeg < kend) fetch(kbeg);
+  for (int k0 = kbeg; k0 < kend; k0 += kDgK) {
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+      const int e = tid + u * kDgThreads;
+      As[(a_kfast ? e % kDgK : e / DT) * LD + (a_kfast ? e / kDgK : e % DT)] = ra[u];
+      Bs[(b_kfast ? e % kDgK : e / DT) * LD + (b_kfast ? e / kDgK : e % DT)] = rb[u];
+    }
+    __syncthreads();
+    if (k0 + kDgK < kend) fetch(k0 + kDgK);
+#pragma unroll
+    for (int q = 0; q < kDgK / 4; ++q) {
+      const int kk = q * 4 + grp;
+      double a[MI], b[MI];
+#pragma unroll
+      for (int i = 0; i < MI; ++i) a[i] = As[kk * LD + ty + 8 * i];
+#pragma unroll
+      for (int j = 0; j < MI; ++j) b[j] = Bs[kk * LD + tx + 8 * j];
+#pragma unroll
+      for (int i = 0; i < MI; ++i)
+#pragma unroll
+        for (int j = 0; j < MI; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+    }
+  }
+  __syncthreads();
+  double* part = sm;  // [4][DT][DT]
+#pragma unroll
+  for (int i = 0; i < MI; ++i)
+#pragma unroll
+    for (int j = 0; j < MI; ++j) part[grp * DT * DT + (ty + 8 * i) * DT + tx + 8 * j] = acc[i][j];
+  __syncthreads();
+  const bool c_rfast = (g.C.rs == 1);
+  auto put = [&](int e, double v) {  // e = row * DT + column
+    const int gm = m0 + e / DT, gn = n0 + e % DT;
+    if (gm >= g.M || gn >= g.N) return;
+    double* c = g.C.p + (long)gm * g.C.rs + (long)gn * g.C.cs;
+    v *= g.alpha;
+    if (g.beta != 0.0) v = fma(g.beta, *c, v);
+    *c = v;
+  };
+  auto slot = [&](int o) { return c_rfast ? (o % DT) * DT + o / DT : o; };  // writes along C's unit stride
+  if (split == 1) {
+#pragma unroll
+    for (int u = 0; u < OUT; ++u) {
+      const int e = slot(tid + u * kDgThreads);
+      put(e, (part[e] + part[DT * DT + e]) + (part[2 * DT * DT + e] + part[3 * DT * DT + e]));
+    }
+    return;
+  }
+#pragma unroll
+  for (int u = 0; u < OUT; ++u) {
+    const int e = tid + u * kDgThreads;
+    part[e] = (part[e] + part[DT * DT + e]) + (part[2 * DT * DT + e] + part[3 * DT * DT + e]);
+  }
+  cg::cluster_group cl = cg::this_cluster();
+  cl.sync();
+  for (int o = rank * kDgThreads + tid; o < DT * DT; o += split * kDgThreads) {
+    const int e = slot(o);
+    double v = 0.0;
+    for (int q = 0; q < split; ++q) v += cl.map_shared_rank(part, q)[e];
+    put(e, v);
+  }
+  cl.sync();  // the partial tile is read by the other CTAs of the cluster until here
+}
 
-  // Load mapping: pick the loop order so that consecutive threads follow the
-  // unit stride of the operand when it has one.
-  const bool a_kfast = (g.A.cs == 1);
-  const bool b_nfast = (g.B.cs == 1);
-  for (int k0 = 0; k0 < g.K; k0 += GK) {
-#pragma unroll
-    for (int e = tid; e < GT * GK; e += 256) {
-      int mm, kk;
-      if (a_kfast) { kk = e % GK; mm = e / GK; } else { mm = e % GT; kk = e / GT; }
-      const int gm = m0 + mm, gk = k0 + kk;
-      As[kk][mm] = (gm < g.M && gk < g.K) ? g.A.p[(long)gm * g.A.rs + (long)gk * g.A.cs] : 0.0;
-    }
-#pragma unroll
-    for (int e = tid; e < GT * GK; e += 256) {
-      int nn, kk;
-      if (b_nfast) { nn = e % GT; kk = e / GT; } else { kk = e % GK; nn = e / GK; }
-      const int gn = n0 + nn, gk = k0 + kk;
-      Bs[kk][nn] = (gn < g.N && gk < g.K) ? g.B.p[(long)gk * g.B.rs + (long)gn * g.B.cs] : 0.0;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < GK; ++kk) {
-      double a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int gm = m0 + ty + 16 * i;
-    if (gm >= g.M) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int gn = n0 + tx + 16 * j;
-      if (gn >= g.N) continue;
-      double* c = g.C.p + (long)gm * g.C.rs + (long)gn * g.C.cs;
-      double v = g.alpha * acc[i][j];
-      if (g.beta != 0.0) v = fma(g.beta, *c, v);
-      *c = v;
-    }
-  }
+// Launches the float64 product of nprob = (products x batch) problems with these upper bounds.
+template <class F>
+cudaError_t launch_dgemm(cudaStream_t st, const F& f, int nprob, int nbatch, int M_ub, int N_ub, int K_ub, int num_sms,
+                         double* fl = nullptr, int fl_stride = 0) {
+  auto cdiv = [](long a, long b) { return (a + b - 1) / b; };
+  const long t32 = cdiv(M_ub, 32) * cdiv(N_ub, 32) * nprob;
+  const bool big = t32 >= 8L * num_sms;
+  const long DT = big ? 32 : 16;
+  const long tiles = cdiv(M_ub, DT) * cdiv(N_ub, DT);
+  const int n_tiles = (int)cdiv(N_ub, DT);
+  int split = 1;
+  while (split < kDgMaxSplit && tiles * nprob * split * 2 <= 4L * num_sms && K_ub >= 2 * kDgK * split * 2) split *= 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(tiles * split), 1, (unsigned)nprob);
+  cfg.blockDim = dim3(kDgThreads);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)split;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = split > 1 ? 1 : 0;
+  if (big) return cudaLaunchKernelEx(&cfg, dgemm_kernel<F, 32>, f, nbatch, n_tiles, split, fl, fl_stride);
+  return cudaLaunchKernelEx(&cfg, dgemm_kernel<F, 16>, f, nbatch, n_tiles, split, fl, fl_stride);
 }
 
 // ---------------------------------------------------------------------------

@@ -134,12 +134,29 @@ void Engine::qr_move(int c, int& nx, int bl, int& br, int brr) {
   const int out = get_buf();
   note_carriage(bl, nbnd);
   note_carriage(nbnd, brr);
-  if (launch_) {
-    const Dim m{d_, bl}, n{1, br};
+  const Dim m{d_, bl}, n{1, br};
+  QrdArgs qd{};
+  qd.t = tab_;
+  qd.bsrc = c;
+  qd.src_rowmajor = 1;
+  qd.bv = ws(WS_T);
+  qd.btau = ws(WS_TAU);
+  qd.br = ws(WS_R);
+  qd.m = m;
+  qd.n = n;
+  qd.ik = nbnd;
+  bool fast = false;
+  if (qrd_apply_fits(m_ub)) timed_if(launch_, 2, [&] {
+    fast = qrd<double>(qd, m_ub, n_ub);
+    if (fast) qrd_apply(QrdApplyArgs{tab_, ws(WS_T), ws(WS_TAU), m, n, -1, -1, nbnd, c, 1, 0}, m_ub, k_ub);
+  });
+  if (launch_ && !fast) {
     copy2d(RowToColFn{tab_, c, ws(WS_T), m, n}, 1, m_ub, n_ub);
     QRArgs qa{tab_, ws(WS_T), ws(WS_TAU), ws(WS_R), ws(WS_Q), m, n, nbnd, n_ub, k_ub};
     timed(2, [&] { coop((void*)householder_kernel, &qa, 1, (long)Z_ * n_ub); });
     copy2d(ColToRowFn{tab_, ws(WS_Q), c, m, Dim{1, nbnd}}, 1, m_ub, k_ub);
+  }
+  if (launch_) {
     gemm(RMergeFn{tab_, ws(WS_R), nx, out, nbnd, br, brr, d_}, 1, k_ub, d_ * umax(brr), n_ub,
          GemmShape{Dim{1, nbnd}, Dim{d_, brr}, Dim{1, br}, 1, 0});
   }
@@ -586,6 +603,10 @@ void Engine::execute(void* arena, const ttm_options& opt, std::vector<ttm_report
   off = align256(off + (size_t)tc_bytes_);
   svd_log_ = (int*)(base + off);
   off = align256(off + (size_t)Z_ * std::max(1, n_trunc_) * kSvdRec * sizeof(int));
+  for (int q = 0; q < 2; ++q) {
+    ex_[q] = (unsigned long long*)(base + off);
+    off = align256(off + (size_t)Z_ * ex_elems_ * sizeof(unsigned long long));
+  }
 
   std::vector<int> hb((size_t)Z_ * nbd, 0);
   for (int id = 0; id < nbd; ++id)
@@ -599,6 +620,9 @@ void Engine::execute(void* arena, const ttm_options& opt, std::vector<ttm_report
   TTM_CUDA(cudaMemsetAsync(d_istat_, 0, (size_t)Z_ * nis * sizeof(int), st));
   TTM_CUDA(cudaMemsetAsync(counters_, 0, (size_t)n_jac * counter_stride_ * sizeof(int), st));
   TTM_CUDA(cudaMemsetAsync(fro2_, 0, (size_t)n_jac * Z_ * sizeof(double), st));
+  if (ex_elems_ > 0)
+    for (int q = 0; q < 2; ++q)
+      TTM_CUDA(cudaMemsetAsync(ex_[q], 0xff, (size_t)Z_ * ex_elems_ * sizeof(unsigned long long), st));
   TTM_CUDA(cudaMemsetAsync(svd_log_, 0, (size_t)Z_ * std::max(1, n_trunc_) * kSvdRec * sizeof(int), st));
   tab_ = Tables{d_buf_, d_bond_, d_stat_, d_istat_, nb_, nbd, ns, nis, Z_};
 
@@ -639,7 +663,7 @@ void Engine::execute(void* arena, const ttm_options& opt, std::vector<ttm_report
   for (int z = 0; z < Z_; ++z) {
     const int st_z = istat[(size_t)z * nis + IS_STATUS];
     if (st_z == (int)TTM_ERR_TIMEOUT)
-      throw Error(TTM_ERR_TIMEOUT, "a tensor-core pipeline wait hit its time limit");
+      throw Error(TTM_ERR_TIMEOUT, "a bounded wait on the device hit its limit");
     if (st_z == (int)TTM_ERR_NONFINITE)
       throw Error(TTM_ERR_NONFINITE, "product " + std::to_string(z) + ": a Swap met a non-finite value");
   }
@@ -1068,7 +1092,14 @@ ttm_status ttm_multiply_noalloc(const ttm_tt* A, const ttm_tt* B, ttm_tt* out, c
     hs.coop_qr = info.coop_qr;
     Engine e(hs, 1, A, B);
     e.plan();
-    const size_t need = e.bytes_needed();
+    // the limit is on the workspace of the general kernels; they run alone where the array has no
+    // room for what the faster ones add
+    const size_t need = e.base_bytes();
+    const bool room = e.bytes_needed() <= (size_t)TTM_NOALLOC_SCRATCH_BYTES;
+    if (!room) {
+      e.base_only();
+      e.plan();
+    }
     if (need > (size_t)TTM_NOALLOC_SCRATCH_BYTES)
       throw Error(TTM_ERR_WORKSPACE, "the product needs " + std::to_string(need) +
                                          " bytes of workspace; the allocation-free path has " +

@@ -17,6 +17,7 @@
 #include "ttm_copy.cuh"
 #include "ttm_gemm.cuh"
 #include "ttm_qr.cuh"
+#include "ttm_qrd.cuh"
 #include "ttm_svd.cuh"
 #include "ttm_bjac.cuh"
 #include "ttm_newton.cuh"
@@ -41,6 +42,7 @@ class Engine {
   // ------------------------------------------------------------------ planning
   void plan() {
     launch_ = false;
+    ex_elems_ = 0;
     reset_ids();
     run();
     // sizes
@@ -48,7 +50,11 @@ class Engine {
     nb_ = nchain_ + WS_COUNT;
   }
 
-  size_t bytes_needed() const { return per_product_bytes() * Z_ + table_bytes() + (size_t)tc_bytes_ + 256; }
+  // Workspace of the general kernels; the faster variants add extra_bytes().
+  size_t base_bytes() const { return per_product_bytes() * Z_ + table_bytes() + (size_t)tc_bytes_ + 256; }
+  size_t bytes_needed() const { return base_bytes() + extra_bytes(); }
+  // only the general kernels: for a caller whose workspace has no room for extra_bytes()
+  void base_only() { base_only_ = true; }
   // use_graph may capture and replay this plan: only for an arena that persists across calls
   void allow_graph() { graph_ok_ = true; }
 
@@ -104,6 +110,12 @@ class Engine {
   double* d_stat_ = nullptr;
   int* d_istat_ = nullptr;
   std::vector<double*> hbuf_;  // host copy of the buffer table
+  bool base_only_ = false;
+  // exchange buffers of the distributed QR (ttm_qrd.cuh): two per product, used in turn
+  long ex_elems_ = 0;          // elements per product and buffer (planned)
+  unsigned long long* ex_[2] = {nullptr, nullptr};
+  int ex_flip_ = 0;
+  long ex_prev_ = 0;           // extent the previous distributed launch used
 
   void reset_ids() {
     gemm_log_.clear();
@@ -115,6 +127,8 @@ class Engine {
     log_.clear();
     trace_ids_.clear();
     jac_launch_ = 0;
+    ex_flip_ = 0;
+    ex_prev_ = 0;
   }
 
   int umax(int id) const {
@@ -162,6 +176,9 @@ class Engine {
     b += (size_t)std::max(1, jac_launch_) * Z_ * sizeof(double) + 256;
     b += (size_t)Z_ * std::max(1, n_trunc_) * kSvdRec * sizeof(int) + 256;
     return b;
+  }
+  size_t extra_bytes() const {
+    return ex_elems_ > 0 ? 2 * ((size_t)Z_ * ex_elems_ * sizeof(unsigned long long) + 256) : 0;
   }
   // Sweep counters per product and Jacobi launch: room for the sweep limit of any pass.
   // sweep limit of the float64 Jacobi of the fallback (max_sweeps when set)
@@ -328,6 +345,63 @@ class Engine {
     }
     return v;
   }
+  // Distributed Householder QR (ttm_qrd.cuh) of a matrix with these upper bounds. G: a CTA per four
+  // columns (one per sub-partition) as far as the SMs reach: on a 256 x 256 float64 matrix G = 64
+  // takes 770 us, 32 791, 16 1218 and 152 772; on 32 x 32 G = 8 84 us and G = 1 104 (at half the
+  // full clock). 0: the columns do not fit the shared memory.
+  int qrd_ctas(int m_ub, int n_ub, size_t elem, size_t* smem) const {
+    if (m_ub > kQdMaxRows) return 0;
+    int G = std::max(1, (n_ub + 3) / 4);
+    const int sms = std::max(1, hs_.num_sms);
+    for (;; G = (G + 1) / 2) {
+      const size_t need = (size_t)((n_ub + G - 1) / G + 1) * m_ub * elem;
+      if (need > (size_t)kQdSmem) return 0;
+      const long occ = std::max<long>(1, std::min<long>(4, (long)(220 * 1024 / (need + 1024))));
+      *smem = need;
+      if ((long)Z_ * G <= occ * sms || G == 1) return G;
+    }
+  }
+  // Plans or launches it. a: everything but the sizes of the distribution.
+  template <typename T>
+  bool qrd(QrdArgs a, int m_ub, int n_ub) {
+    size_t smem = 0;
+    int G = base_only_ ? 0 : qrd_ctas(m_ub, n_ub, sizeof(T), &smem);
+    if (G == 0) return false;
+    const long extent = (long)m_ub * std::min(m_ub, n_ub);
+    if (!launch_) {
+      if (G > 1) ex_elems_ = std::max(ex_elems_, extent);
+      return true;
+    }
+    a.G = G;
+    a.cols_ub = (n_ub + G - 1) / G;
+    a.ld_ub = m_ub;
+    a.ex_stride = ex_elems_;
+    a.ex = ex_[ex_flip_];
+    a.ex_next = ex_[ex_flip_ ^ 1];
+    a.clear_n = 0;
+    void* fn = (void*)qrd_kernel<T>;
+    void* kargs[] = {&a};
+    TTM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (G > 1) {
+      a.clear_n = ex_prev_;
+      ex_prev_ = extent;
+      ex_flip_ ^= 1;
+      TTM_CUDA(cudaLaunchCooperativeKernel(fn, dim3((unsigned)(Z_ * G)), dim3(kQdThreads), kargs, smem, hs_.stream));
+    } else {
+      TTM_CUDA(cudaLaunchKernel(fn, dim3((unsigned)Z_), dim3(kQdThreads), kargs, smem, hs_.stream));
+    }
+    ++launches_;
+    return true;
+  }
+  void qrd_apply(QrdApplyArgs a, int m_ub, int c_ub) {
+    if (!launch_) return;
+    const size_t smem = (size_t)(kQaStages + 4) * m_ub * sizeof(double);
+    a.ld_ub = m_ub;
+    TTM_CUDA(cudaFuncSetAttribute(qrd_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    qrd_apply_kernel<<<dim3(cdiv(c_ub, 4), (unsigned)Z_), kQaThreads, smem, hs_.stream>>>(a);
+    TTM_CUDA(cudaGetLastError());
+    ++launches_;
+  }
   long launches_ = 0;
   int prof_used_ = 0;
   std::vector<int> prof_kind_;  // per event pair: 0 GEMM, 1 float32 Jacobi pass, 2 Householder QR
@@ -353,6 +427,13 @@ class Engine {
     launch();
     TTM_CUDA(cudaEventRecord(e1, hs_.stream));
   }
+
+  template <class Launch>
+  void timed_if(bool on, int kind, Launch&& launch) {
+    if (on) timed(kind, launch);
+    else launch();
+  }
+  static bool qrd_apply_fits(int m_ub) { return (size_t)(kQaStages + 4) * m_ub * sizeof(double) <= (size_t)kQdSmem; }
 
   // ------------------------------------------------------------------ steps
   void load_core(const ttm_tt* T, int k, int buf);

@@ -1,0 +1,449 @@
+// ttm_qrd.cuh -- Householder QR with the columns resident in shared memory, distributed over the
+// CTAs of a product, and the application of its reflectors.
+//
+// A (M x N) = Q R with k = min(M, N). Reflector j is kept as H = I - tau v v^T with v = x - beta e_j
+// (x: column j from row j down, beta = -sign(x_j) ||x||, tau = 2 / v^T v = 1 / (||x|| (||x|| + |x_j|));
+// Golub & Van Loan, Alg. 5.1.1, without the division by v_j). Serves the gauge moves (a carriage,
+// float64) and the Swap SVD (Theta^T in float64; its triangular factor again in float32).
+//
+// What bounds it: a chain of k dependent steps, and in it the float64 pipe, on which one warp
+// instruction takes 64 clocks of its sub-partition whatever its lanes do (measured; a warp sum is
+// 600 clocks, a division 450, a square root 700). So the chain has one reduction per step and as few
+// float64 instructions as possible:
+//   - column j travels as it is; whoever receives it forms x.x and x.a for its next column in one
+//     joint sum (4 warps, one per sub-partition) and derives beta, tau and v.a = x.a - beta a_j;
+//   - 1 / ||x|| and 1 / (||x|| + |x_j|) come from a float32 seed and one cubic step (12 instructions
+//     instead of a square root and two divisions);
+//   - columns are dealt out cyclically to G CTAs and stay in shared memory; the owner of column
+//     j + 1 updates and publishes it before its other columns. Receivers poll the data itself (the
+//     exchange buffer is filled with a NaN pattern that arithmetic does not produce), so a step
+//     costs one one-way trip through L2 (about 800 clocks) and no flag or grid barrier.
+// The other columns are updated by one warp each, four per pass when there are that many (their
+// sums share a reduce-scatter of 6 instead of 4 x 5 additions). Every wait is bounded.
+#pragma once
+#include "ttm_common.cuh"
+
+namespace ttm {
+
+constexpr int kQdThreads = 256;
+constexpr int kQdMaxRows = 2048;
+constexpr int kQdSmem = 200 * 1024;  // columns of one CTA
+constexpr int kQdPolls = 2 << 20;    // bound of a wait (a second or so)
+constexpr unsigned long long kQdEmpty = ~0ull;  // exchange element not written yet
+
+struct QrdArgs {
+  Tables t;
+  int bsrc;          // A: float64 buffer
+  int src_rowmajor;  // 1: A row-major (ld N); 0: A column-major (ld M)
+  int bv, btau;      // out (bv < 0: none): reflectors, column-major M x k (row j holds v_j), and tau[k]
+  int br;            // out: R, row-major k x N (zero below the diagonal), type T
+  Dim m, n;
+  int ik;            // -1, or bond id that receives k
+  int G;             // CTAs per product
+  int cols_ub, ld_ub;           // columns held per CTA (upper bound) and their leading dimension
+  unsigned long long* ex;       // exchange, ex_stride elements per product, holding kQdEmpty (G > 1)
+  unsigned long long* ex_next;  // the buffer of the next launch: its first clear_n elements are emptied
+  long ex_stride, clear_n;
+  double* absmax;    // [nz] T = double: nullptr or receives max |R|; T = float: nullptr or A is divided by
+                     // the power of two above it
+  float ridge;       // T = float: diagonal entries of R are moved away from zero by this much
+};
+
+template <typename T>
+__device__ __forceinline__ T qd_sum(T v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Sums of four values over a warp: the sum of value q ends in the lanes with lane / 8 == q.
+template <typename T>
+__device__ __forceinline__ T qd_sum4(const T (&s)[4], int lane) {
+  const bool hi = lane & 16, h2 = lane & 8;
+  T a = hi ? s[2] : s[0], b = hi ? s[3] : s[1];
+  a += __shfl_xor_sync(0xffffffffu, hi ? s[0] : s[2], 16);
+  b += __shfl_xor_sync(0xffffffffu, hi ? s[1] : s[3], 16);
+  T c = h2 ? b : a;
+  c += __shfl_xor_sync(0xffffffffu, h2 ? a : b, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+  return c;
+}
+
+// beta, v_j and tau of a column with squared norm g and leading entry alpha. A zero column has
+// tau = 0; a NaN travels on in beta.
+__device__ __forceinline__ void qd_scalars(double g, double alpha, double& beta, double& vj, double& tau) {
+  const int hi = __double2hiint(g), lo = __double2loint(g), ex = (hi >> 20) - 1023;
+  double mu, r;
+  if (ex > -900 && ex < 900) {  // (a negative or NaN g is outside)
+    const int h = ex >> 1;
+    const int gh = hi - ((2 * h) << 20);  // g 2^(-2h) in [1, 4)
+    const double gs = __hiloint2double(gh, lo);
+    const unsigned s = __float_as_uint(rsqrtf(__uint_as_float(((unsigned)(gh - 0x38000000) << 3) | ((unsigned)lo >> 29))));
+    const double r0 = __hiloint2double((int)(s >> 3) + 0x38000000, (int)(s << 29));
+    const double e = fma(-(gs * r0), r0, 1.0);
+    const double rs = fma(r0 * e, fma(e, 0.375, 0.5), r0);
+    const double ms = gs * rs;
+    r = __hiloint2double(__double2hiint(rs) - (h << 20), __double2loint(rs));
+    mu = __hiloint2double(__double2hiint(ms) + (h << 20), __double2loint(ms));
+  } else if (g > 0.0) {
+    mu = sqrt(g);
+    r = 1.0 / mu;
+  } else {
+    beta = g == 0.0 ? alpha : g;
+    vj = 0.0;
+    tau = 0.0;
+    return;
+  }
+  const double y = fabs(alpha) + mu;
+  const int yh = __double2hiint(y), yl = __double2loint(y), ye = (yh >> 20) - 1023;
+  double q;
+  if (ye > -900 && ye < 900) {
+    const int sh = yh - (ye << 20);  // y 2^-ye in [1, 2)
+    const unsigned s =
+        __float_as_uint(__fdividef(1.f, __uint_as_float(((unsigned)(sh - 0x38000000) << 3) | ((unsigned)yl >> 29))));
+    const double q0 = __hiloint2double((int)(s >> 3) + 0x38000000, (int)(s << 29));
+    const double e = fma(-__hiloint2double(sh, yl), q0, 1.0);
+    const double qs = fma(q0 * e, 1.0 + e, q0);
+    q = __hiloint2double(__double2hiint(qs) - (ye << 20), __double2loint(qs));
+  } else {
+    q = 1.0 / y;
+  }
+  tau = r * q;
+  beta = alpha <= 0.0 ? mu : -mu;
+  vj = alpha <= 0.0 ? -y : y;
+}
+__device__ __forceinline__ void qd_scalars(float g, float alpha, float& beta, float& vj, float& tau) {
+  if (g > 0.f) {
+    float r = rsqrtf(g);
+    r = fmaf(r * 0.5f, fmaf(-(g * r), r, 1.f), r);
+    const float mu = g * r, y = fabsf(alpha) + mu;
+    tau = __fdividef(r, y);
+    beta = alpha <= 0.f ? mu : -mu;
+    vj = alpha <= 0.f ? -y : y;
+  } else {
+    beta = g == 0.f ? alpha : g;
+    vj = 0.f;
+    tau = 0.f;
+  }
+}
+
+template <typename T> struct QdBits;
+template <> struct QdBits<double> {
+  static __device__ __forceinline__ unsigned long long to(double x) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    return b == kQdEmpty ? 0x7ff8000000000000ull : b;
+  }
+  static __device__ __forceinline__ double from(unsigned long long b) { return __longlong_as_double((long long)b); }
+};
+template <> struct QdBits<float> {
+  static __device__ __forceinline__ unsigned long long to(float x) { return __float_as_uint(x); }  // high word 0
+  static __device__ __forceinline__ float from(unsigned long long b) { return __uint_as_float((unsigned)b); }
+};
+__device__ __forceinline__ unsigned long long qd_ld(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void qd_st(unsigned long long* p, unsigned long long v) {
+  asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kQdThreads) qrd_kernel(QrdArgs a) {
+  extern __shared__ __align__(16) unsigned char qd_raw[];
+  const int G = a.G, z = blockIdx.x / G, b = blockIdx.x % G;
+  const int M = a.m.eval(a.t, z), N = a.n.eval(a.t, z), k = min(M, N);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int ld = a.ld_ub;
+  T* cols = reinterpret_cast<T*>(qd_raw);          // [cols_ub][ld]
+  T* xs = cols + (long)a.cols_ub * ld;              // [ld] the column received
+  __shared__ T red[2][8];
+  __shared__ T s_sc[3];                             // beta, v_j, tau of the current step
+  __shared__ int s_abort;
+  if (b == 0 && tid == 0 && a.ik >= 0) a.t.bond[z * a.t.nbd + a.ik] = k;
+  for (long e = (long)b * kQdThreads + tid; e < a.clear_n; e += (long)G * kQdThreads)
+    a.ex_next[z * a.ex_stride + e] = kQdEmpty;
+  const int nl = b < N ? (N - b + G - 1) / G : 0;
+  if (nl == 0) return;  // nothing of this product here, and no one waits for this CTA
+  if (tid == 0) s_abort = 0;
+  const double* src = bufp(a.t, z, a.bsrc);
+  double scale = 1.0;
+  if constexpr (sizeof(T) == 4) {
+    if (a.absmax) {
+      const double mx = a.absmax[z];
+      int e = 0;
+      if (mx > 0.0 && mx < 1.7e308) frexp(mx, &e);
+      scale = ldexp(1.0, -max(-1000, min(1000, e)));
+    }
+  }
+  for (int e = tid; e < nl * M; e += kQdThreads) {
+    int l, i;
+    if (G == 1 && a.src_rowmajor) {  // consecutive threads along a row
+      i = e / nl;
+      l = e - i * nl;
+    } else {
+      l = e / M;
+      i = e - l * M;
+    }
+    const int c = b + G * l;
+    const double x = a.src_rowmajor ? src[(long)i * N + c] : src[(long)c * M + i];
+    cols[l * ld + i] = sizeof(T) == 4 ? (T)(x * scale) : (T)x;
+  }
+  unsigned long long* ex = a.ex + z * a.ex_stride;
+  T* R = reinterpret_cast<T*>(bufp(a.t, z, a.br));
+  double* V = a.bv >= 0 ? bufp(a.t, z, a.bv) : nullptr;
+  double* taug = a.bv >= 0 ? bufp(a.t, z, a.btau) : nullptr;
+  __syncthreads();
+  if (G > 1 && b == 0)
+    for (int i = tid; i < M; i += kQdThreads) qd_st(ex + i, QdBits<T>::to(cols[i]));
+
+  int lj = 0, jr = 0;  // j / G and j % G
+  for (int j = 0; j < k; ++j) {
+    if (b + G * (nl - 1) < j) break;  // no column from j on is held here
+    const bool mine = jr == b;
+    const int nxt = j + 1;
+    const int nr = jr + 1 == G ? 0 : jr + 1, nlj = jr + 1 == G ? lj + 1 : lj;
+    const int lc = (nr == b && nxt < N) ? nlj : -1;  // local index of column j + 1, if it is here
+    const T* x = mine ? cols + lj * ld : xs;
+    const int base = j & ~31;
+    T* crit = lc >= 0 ? cols + lc * ld : nullptr;
+    if (warp < 4) {
+      T p0 = T(0), p1 = T(0);
+      if (mine) {
+        for (int i = base + tid; i < M; i += 128) {
+          const T xi = i >= j ? x[i] : T(0);
+          p0 = fma(xi, xi, p0);
+          if (crit) p1 = fma(xi, crit[i], p1);
+        }
+      } else {
+        // all of this thread's rows are requested before any is waited for
+        const unsigned long long* src_x = ex + (long)j * M;
+        constexpr int NB = 8;
+        for (int i0 = base + tid; i0 < M; i0 += 128 * NB) {
+          unsigned long long bits[NB];
+#pragma unroll
+          for (int u = 0; u < NB; ++u) {
+            const int i = i0 + 128 * u;
+            bits[u] = (i >= j && i < M) ? qd_ld(src_x + i) : 0;
+          }
+#pragma unroll
+          for (int u = 0; u < NB; ++u) {
+            const int i = i0 + 128 * u;
+            if (i >= M) break;
+            for (int polls = 0; bits[u] == kQdEmpty && polls < kQdPolls; ++polls) bits[u] = qd_ld(src_x + i);
+            if (bits[u] == kQdEmpty) s_abort = 1;
+            const T xi = QdBits<T>::from(bits[u]);
+            xs[i] = xi;
+            p0 = fma(xi, xi, p0);
+            if (crit) p1 = fma(xi, crit[i], p1);
+          }
+        }
+      }
+      const bool hi = lane & 16;
+      T s = hi ? p1 : p0;
+      s += __shfl_xor_sync(0xffffffffu, hi ? p0 : p1, 16);
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if ((lane & 15) == 0) red[j & 1][warp + (hi ? 4 : 0)] = s;
+    }
+    __syncthreads();
+    if (s_abort) {  // every thread sees it: it was set before the barrier
+      if (tid == 0) atomicExch(&a.t.istat[z * a.t.nis + IS_STATUS], (int)TTM_ERR_TIMEOUT);
+      return;
+    }
+    if (warp < 4) {
+      T s = red[j & 1][lane & 7];
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      s += __shfl_xor_sync(0xffffffffu, s, 2);
+      const T g = __shfl_sync(0xffffffffu, s, 0), d = __shfl_sync(0xffffffffu, s, 4);
+      T beta, vj, tau;
+      qd_scalars(g, x[j], beta, vj, tau);
+      if (crit) {
+        const T cj = crit[j];
+        const T f = tau * fma(-beta, cj, d);
+        unsigned long long* dst = ex + (long)nxt * M;
+        for (int i = base + tid; i < M; i += 128) {
+          if (i > j) {
+            const T y = fma(-f, x[i], crit[i]);
+            crit[i] = y;
+            if (G > 1 && nxt < k) qd_st(dst + i, QdBits<T>::to(y));
+          }
+        }
+        __syncwarp();
+        if (tid == 0) R[(long)j * N + nxt] = fma(-f, vj, cj);
+      }
+      if (tid == 0) {
+        s_sc[0] = beta;
+        s_sc[1] = vj;
+        s_sc[2] = tau;
+        if (mine) {
+          T rd = beta;
+          if constexpr (sizeof(T) == 4) rd += rd < T(0) ? -a.ridge : a.ridge;
+          R[(long)j * N + j] = rd;
+          if (V) {
+            V[(long)j * M + j] = (double)vj;
+            taug[j] = (double)tau;
+          }
+        }
+      }
+    }
+    __syncthreads();
+    // the other columns right of j: local index from l0 on, one warp per column
+    int l0 = lj + (b > jr ? 0 : 1);
+    if (l0 == lc) ++l0;
+    const int rest = nl - l0;
+    if (rest > 0) {
+      const T beta = s_sc[0], vj = s_sc[1], tau = s_sc[2];
+      for (int q0 = 0; q0 < rest; q0 += 32) {
+        const int cnt = min(32, rest - q0);
+        if (cnt > 8) {
+          // up to four columns of this warp: l0 + q0 + warp + 8 q
+          const int lw = l0 + q0 + warp;
+          T s[4] = {T(0), T(0), T(0), T(0)};
+          T* ac[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) ac[q] = cols + min(lw + 8 * q, nl - 1) * ld;
+          for (int i = base + lane; i < M; i += 32) {
+            const T xi = i >= j ? x[i] : T(0);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              if (warp + 8 * q < cnt) s[q] = fma(xi, ac[q][i], s[q]);
+          }
+          const int mq = lane >> 3;
+          const T dsum = qd_sum4(s, lane);
+          const T cj = cols[min(lw + 8 * mq, nl - 1) * ld + j];
+          const T f = tau * fma(-beta, cj, dsum);
+          T fq[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) fq[q] = __shfl_sync(0xffffffffu, f, 8 * q);
+          if ((lane & 7) == 0 && warp + 8 * mq < cnt)
+            R[(long)j * N + b + (long)G * (lw + 8 * mq)] = fma(-f, vj, cj);
+          for (int i = base + lane; i < M; i += 32) {
+            const T xi = x[i];
+            if (i > j) {
+#pragma unroll
+              for (int q = 0; q < 4; ++q)
+                if (warp + 8 * q < cnt) ac[q][i] = fma(-fq[q], xi, ac[q][i]);
+            }
+          }
+        } else if (warp < cnt) {
+          T* ac = cols + (l0 + q0 + warp) * ld;
+          T s = T(0);
+          for (int i = base + lane; i < M; i += 32) {
+            const T xi = i >= j ? x[i] : T(0);
+            s = fma(xi, ac[i], s);
+          }
+          s = qd_sum(s);
+          const T cj = ac[j];
+          const T f = tau * fma(-beta, cj, s);
+          if (lane == 0) R[(long)j * N + b + (long)G * (l0 + q0 + warp)] = fma(-f, vj, cj);
+          for (int i = base + lane; i < M; i += 32)
+            if (i > j) ac[i] = fma(-f, x[i], ac[i]);
+        }
+      }
+    }
+    lj = nlj;
+    jr = nr;
+    __syncthreads();
+  }
+  // zeros of R below the diagonal, the reflectors, and the largest magnitude of R
+  double mx = 0.0;
+  for (int e = tid; e < nl * k; e += kQdThreads) {
+    const int l = e / k, i = e - l * k, c = b + G * l;
+    if (i > c) R[(long)i * N + c] = T(0);
+    else if (sizeof(T) == 8 && a.absmax) mx = fmax(mx, fabs((double)R[(long)i * N + c]));
+  }
+  if constexpr (sizeof(T) == 8) {
+    if (V)
+      for (int e = tid; e < nl * M; e += kQdThreads) {
+        const int l = e / M, i = e - l * M, c = b + G * l;
+        if (c < k && i > c) V[(long)c * M + i] = cols[l * ld + i];
+      }
+    if (a.absmax) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      if (lane == 0 && mx > 0.0)
+        atomicMax(reinterpret_cast<unsigned long long*>(a.absmax + z), (unsigned long long)__double_as_longlong(mx));
+    }
+  }
+}
+
+// Y = H_0 H_1 .. H_{k-1} Y0 in float64: one column per warp in shared memory, four columns per CTA;
+// the reflectors arrive through a ring of shared buffers filled by cp.async three steps ahead. Y0 is
+// the first columns of the identity (bvec < 0) or the columns perm[c] of a k x k column-major matrix,
+// padded with zeros. What bounds it: the float64 pipe (per step 2 M / 32 + 7 warp instructions of 64
+// clocks; the columns are independent, so the launch fills the chip with them).
+constexpr int kQaThreads = 128;
+constexpr int kQaStages = 4;
+struct QrdApplyArgs {
+  Tables t;
+  int bv, btau;   // reflectors and tau of qrd_kernel<double>
+  Dim m, n;       // A was m x n
+  int bvec, bperm;
+  int ic;         // bond id: columns of Y
+  int bout;
+  int out_rows;   // 1: Y row-major (m x columns); 0: Y^T row-major (columns x m)
+  int ld_ub;
+};
+
+__global__ void __launch_bounds__(kQaThreads) qrd_apply_kernel(QrdApplyArgs a) {
+  extern __shared__ __align__(16) unsigned char qd_raw[];
+  const int z = blockIdx.y;
+  const int M = a.m.eval(a.t, z), N = a.n.eval(a.t, z), k = min(M, N), nc = bondv(a.t, z, a.ic);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int c0 = blockIdx.x * 4, c = c0 + warp;
+  if (c0 >= nc) return;
+  const int ld = a.ld_ub;
+  double* vs = reinterpret_cast<double*>(qd_raw);     // [kQaStages][ld]
+  double* y = vs + (kQaStages + warp) * (long)ld;      // this warp's column
+  const double* V = bufp(a.t, z, a.bv);
+  const double* tau = bufp(a.t, z, a.btau);
+  const bool on = c < nc;
+  int j0;
+  if (a.bvec < 0) {
+    j0 = min(min(c0 + 3, nc - 1), k - 1);
+    for (int i = lane; i < M; i += 32) y[i] = i == c ? 1.0 : 0.0;
+  } else {
+    j0 = k - 1;
+    const int pc = on ? reinterpret_cast<const int*>(bufp(a.t, z, a.bperm))[c] : 0;
+    const double* x = bufp(a.t, z, a.bvec) + (long)max(0, min(pc, k - 1)) * k;
+    for (int i = lane; i < M; i += 32) y[i] = i < k ? x[i] : 0.0;
+  }
+  auto fetch = [&](int q) {  // reflector q into its stage; one commit group per call
+    if (q >= 0) {
+      double* dst = vs + (q & (kQaStages - 1)) * (long)ld;
+      const double* src = V + (long)q * M;
+      for (int i = (q & ~31) + threadIdx.x; i < M; i += kQaThreads)
+        if (i >= q)
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst + i)),
+                       "l"(src + i)
+                       : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  for (int s = 0; s < kQaStages - 1; ++s) fetch(j0 - s);
+  for (int j = j0; j >= 0; --j) {
+    const double tj = __ldg(tau + j);
+    asm volatile("cp.async.wait_group %0;" ::"n"(kQaStages - 2) : "memory");
+    __syncthreads();  // reflector j is here, and its ring slot of step j + 1 is free again
+    fetch(j - (kQaStages - 1));
+    const double* v = vs + (j & (kQaStages - 1)) * (long)ld;
+    double s = 0.0;
+    for (int i = (j & ~31) + lane; i < M; i += 32)
+      if (i >= j) s = fma(v[i], y[i], s);
+    const double f = tj * qd_sum(s);
+    for (int i = (j & ~31) + lane; i < M; i += 32)
+      if (i >= j) y[i] = fma(-f, v[i], y[i]);
+    __syncwarp();
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  if (!on) return;
+  double* out = bufp(a.t, z, a.bout);
+  if (a.out_rows)
+    for (int i = lane; i < M; i += 32) out[(long)i * nc + c] = y[i];
+  else
+    for (int i = lane; i < M; i += 32) out[(long)c * M + i] = y[i];
+}
+
+}  // namespace ttm

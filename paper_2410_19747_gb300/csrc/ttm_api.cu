@@ -148,7 +148,7 @@ void Engine::qr_move(int c, int& nx, int bl, int& br, int brr) {
   bool fast = false;
   if (qrd_apply_fits(m_ub)) timed_if(launch_, 2, [&] {
     fast = qrd<double>(qd, m_ub, n_ub);
-    if (fast) qrd_apply(QrdApplyArgs{tab_, ws(WS_T), ws(WS_TAU), m, n, -1, -1, nbnd, c, 1, 0}, m_ub, k_ub);
+    if (fast) qrd_apply(QrdApplyArgs{tab_, ws(WS_T), ws(WS_TAU), m, n, -1, -1, -1, nbnd, c, 1, 0}, m_ub, k_ub);
   });
   if (launch_ && !fast) {
     copy2d(RowToColFn{tab_, c, ws(WS_T), m, n}, 1, m_ub, n_ub);
@@ -199,6 +199,12 @@ int Engine::swap(int x, int y, int bl, int bm, int br, int kind) {
   jac_launch_ += npass;
   const int sw64 = jac_launch_++;          // the fallback's float64 Jacobi
   const int nprov = new_bond(kub);         // provisional rank before the Newton steps
+  if (pre_fits(m_ub, n_ub)) {
+    for (int z = 0; z < Z_; ++z) kub[z] = std::min(d_ * ub_[bl][z], d_ * ub_[br][z]);
+    const int pb = new_bond(kub);          // min(m, n)
+    swap_pre(x, y, bl, bm, br, nbnd, nprov, pb, kind, cap, sw32, sw64, wslot);
+    return nbnd;
+  }
   if (launch_) {
     const Dim m{d_, bl}, n{d_, br};
     const int npad_ub = n_ub + (n_ub & 1);
@@ -339,6 +345,127 @@ int Engine::swap(int x, int y, int bl, int bm, int br, int kind) {
     }
   }
   return nbnd;
+}
+
+// The Swap by the preconditioned SVD of ttm_pre.cuh. pb: bond id of p = min(m, n).
+void Engine::swap_pre(int x, int y, int bl, int bm, int br, int nbnd, int nprov, int pb, int kind, long cap, int sw32,
+                      int sw64, int wslot) {
+  const int m_ub = d_ * umax(bl), n_ub = d_ * umax(br), p_ub = umax(pb), k_ub = umax(nbnd);
+  const Dim m{d_, bl}, n{d_, br}, p{1, pb};
+  const int th = ws(WS_T), refl = ws(WS_V), L = ws(WS_W0), X = ws(WS_V32);
+  const int w[2] = {ws(WS_T), ws(WS_W0B)}, v[2] = {ws(WS_V2), ws(WS_V3)};
+  const int gram = ws(WS_G), vv = ws(WS_R), elim = ws(WS_V0), xn = ws(WS_X);
+  const int ikeep = kind == SK_ROUND ? bm : -1;
+  // 1. Theta = X Y with the physical legs permuted (Fig. 1C)
+  gemm(ThetaFn{tab_, x, y, th, bl, bm, br, d_, kind == SK_ROUND ? 1 : 0}, d_ * d_, umax(bl), umax(br), umax(bm),
+       GemmShape{Dim{1, bl}, Dim{1, br}, Dim{1, bm}, d_ * d_, 0});
+  // 2. Theta^T = Q1 R1 (float64) and R1^T = Q2 R2 (float32)
+  timed_if(launch_, 2, [&] {
+    QrdArgs q1{};
+    q1.t = tab_;
+    q1.bsrc = th;
+    q1.src_rowmajor = 1;
+    q1.bv = refl;
+    q1.btau = ws(WS_TAU);
+    q1.br = L;
+    q1.m = n;
+    q1.n = m;
+    q1.ik = pb;
+    q1.scaled = 1;
+    qrd<double>(q1, n_ub, m_ub);
+    QrdArgs q2{};
+    q2.t = tab_;
+    q2.bsrc = L;
+    q2.bv = q2.btau = -1;
+    q2.br = X;
+    q2.m = m;
+    q2.n = p;
+    q2.ik = -1;
+    q2.scaled = 1;
+    q2.ridge = kPreRidge;
+    qrd<float>(q2, m_ub, p_ub);
+  });
+  // 3. the float32 Jacobi on X = R2^T
+  if (launch_) {
+    PreJacArgs ja{};
+    ja.t = tab_;
+    ja.bx = X;
+    ja.p = p;
+    ja.max_sweeps = kPreSweeps;
+    ja.counters = counters_ + (size_t)sw32 * counter_stride_;
+    ja.stride = counter_sweeps();
+    ja.tol = (float)(kPreTol * std::sqrt((double)std::max(p_ub, 1)));
+    ja.big = kPreBig;
+    ja.flop_slot = ST_JFLOPS32;
+    ja.sweep_slot = ST_JSWEEPS32;
+    ja.svd_log = svd_rec(cur_svd_);
+    ja.svd_stride = svd_stride();
+    ja.svd_field = SR_SW0;
+    timed(1, [&] { jacobi_pre(ja, p_ub); });
+    // its column norms in descending order, the provisional rank, and V
+    pre_norm_kernel<float><<<dim3(cdiv(p_ub, 8), Z_), 256, 0, hs_.stream>>>(PreNormArgs{tab_, X, X, ws(WS_NRM), m, p});
+    TTM_CUDA(cudaGetLastError());
+    PreOrderArgs oa{tab_, ws(WS_NRM), ws(WS_SORT), ws(WS_PERM), m, n, p, nprov, opt_.eps, (int)cap, -1, 0, ikeep,
+                    nullptr, 0};
+    pre_order_kernel<<<Z_, 1024, 0, hs_.stream>>>(oa);
+    TTM_CUDA(cudaGetLastError());
+    pre_v_kernel<<<dim3(cdiv(p_ub, 8), Z_), 256, 0, hs_.stream>>>(PreVArgs{tab_, X, ws(WS_PERM), v[0], p});
+    TTM_CUDA(cudaGetLastError());
+    launches_ += 3;
+  }
+  // 4. W = L V and the Newton steps (every launch of the last two is empty for a converged product)
+  if (tc_) colexp(L, m, p, p_ub, ws(WS_NRM));
+  gemm(PreProductFn{tab_, L, v[0], w[0], m, p}, 1, m_ub, p_ub, p_ub, GemmShape{m, p, p, 1, 0}, tc_ ? ws(WS_NRM) : -1);
+  for (int s = 0; s < 4; ++s) {
+    const int a = s & 1, b = a ^ 1;
+    if (tc_) {
+      gemm(PreGramFn{tab_, w[a], v[a], gram, vv, m, p, s, 0}, 1, p_ub, p_ub, m_ub, GemmShape{p, p, m, 1, 1});
+      gemm(PreGramFn{tab_, w[a], v[a], gram, vv, m, p, s, 1}, 1, p_ub, p_ub, p_ub, GemmShape{p, p, p, 1, 1});
+    } else {
+      gemm(PreGramFn{tab_, w[a], v[a], gram, vv, m, p, s, -1}, 2, p_ub, p_ub, m_ub, GemmShape{p, p, m, 2, 1});
+    }
+    pre_elim(PreElimArgs{tab_, gram, elim, p, s}, p_ub);
+    if (launch_) {
+      pre_x_kernel<<<dim3(cdiv(p_ub, 32), cdiv(p_ub, 8), Z_), 256, 0, hs_.stream>>>(
+          PreXArgs{tab_, elim, vv, xn, p, ws(WS_SORT), nprov, s, IS_NFROZEN});
+      TTM_CUDA(cudaGetLastError());
+      ++launches_;
+    }
+    if (tc_) {
+      colexp(w[a], m, p, p_ub, ws(WS_NRM));
+      gemm(PreApplyFn{tab_, w[a], v[a], xn, w[b], v[b], m, p, s, 0}, 1, m_ub, p_ub, p_ub, GemmShape{m, p, p, 1, 0},
+           ws(WS_NRM));
+      gemm(PreApplyFn{tab_, w[a], v[a], xn, w[b], v[b], m, p, s, 1}, 1, p_ub, p_ub, p_ub, GemmShape{p, p, p, 1, 0});
+    } else {
+      gemm(PreApplyFn{tab_, w[a], v[a], xn, w[b], v[b], m, p, s, -1}, 2, m_ub, p_ub, p_ub, GemmShape{m, p, p, 2, 0});
+    }
+  }
+  if (launch_) {
+    // a product whose last correction is still large: the float64 Jacobi on L from V = I
+    pre_rescue_kernel<<<dim3((unsigned)std::min<long>(512, cdiv((long)m_ub * p_ub, 256)), Z_), 256, 0, hs_.stream>>>(
+        PreRescueArgs{tab_, L, w[0], v[0], m, p});
+    TTM_CUDA(cudaGetLastError());
+    ++launches_;
+    const int nblk_ub = (p_ub + kJrB - 1) / kJrB;
+    const int nblk_pad_ub = nblk_ub + (nblk_ub & 1);
+    JResArgs j64{tab_, w[0], v[0], m, p, nblk_pad_ub, polish_sweeps(), counters_ + (size_t)sw64 * counter_stride_, 1e-10,
+                 64 * 1.11e-16, fro2_ + (size_t)sw64 * Z_, ST_JFLOPS, ws(WS_NRM), 1, -1, nullptr, 0, 0, 1, IS_FALLBACK};
+    timed(3, [&] { jacobi_res<double>(j64, m_ub, p_ub, nblk_pad_ub); });
+    // 5. final order, Eq. eps + cap, new carriages
+    pre_norm_kernel<double><<<dim3(cdiv(p_ub, 8), Z_), 256, 0, hs_.stream>>>(PreNormArgs{tab_, w[0], w[1], ws(WS_NRM), m, p});
+    TTM_CUDA(cudaGetLastError());
+    PreOrderArgs oa{tab_, ws(WS_NRM), ws(WS_SORT), ws(WS_PERM), m, n, p, nbnd, opt_.eps, (int)cap, wslot, 1, ikeep,
+                    svd_rec(cur_svd_), svd_stride()};
+    pre_order_kernel<<<Z_, 1024, 0, hs_.stream>>>(oa);
+    TTM_CUDA(cudaGetLastError());
+    pre_left_kernel<<<dim3(cdiv(m_ub, 32), cdiv(k_ub, 32), Z_), 256, 0, hs_.stream>>>(
+        PreLeftArgs{tab_, w[0], w[1], ws(WS_PERM), y, m, nbnd});
+    TTM_CUDA(cudaGetLastError());
+    launches_ += 3;
+    timed(2, [&] {
+      qrd_apply(QrdApplyArgs{tab_, refl, ws(WS_TAU), n, m, v[0], v[1], ws(WS_PERM), nbnd, x, 0, 0}, n_ub, k_ub);
+    });
+  }
 }
 
 // One float32 one-sided Jacobi pass on the W32 workspace (V32 starts at I): by default the
@@ -603,9 +730,14 @@ void Engine::execute(void* arena, const ttm_options& opt, std::vector<ttm_report
   off = align256(off + (size_t)tc_bytes_);
   svd_log_ = (int*)(base + off);
   off = align256(off + (size_t)Z_ * std::max(1, n_trunc_) * kSvdRec * sizeof(int));
-  for (int q = 0; q < 2; ++q) {
-    ex_[q] = (unsigned long long*)(base + off);
-    off = align256(off + (size_t)Z_ * ex_elems_ * sizeof(unsigned long long));
+  double* pre = nullptr;
+  if (!base_only_) {
+    for (int q = 0; q < 2; ++q) {
+      ex_[q] = (unsigned long long*)(base + off);
+      off = align256(off + (size_t)Z_ * ex_elems_ * sizeof(unsigned long long));
+    }
+    pre = (double*)(base + off);
+    off = align256(off + (size_t)Z_ * kPreSlots * sizeof(double));
   }
 
   std::vector<int> hb((size_t)Z_ * nbd, 0);
@@ -620,11 +752,12 @@ void Engine::execute(void* arena, const ttm_options& opt, std::vector<ttm_report
   TTM_CUDA(cudaMemsetAsync(d_istat_, 0, (size_t)Z_ * nis * sizeof(int), st));
   TTM_CUDA(cudaMemsetAsync(counters_, 0, (size_t)n_jac * counter_stride_ * sizeof(int), st));
   TTM_CUDA(cudaMemsetAsync(fro2_, 0, (size_t)n_jac * Z_ * sizeof(double), st));
+  if (pre) TTM_CUDA(cudaMemsetAsync(pre, 0, (size_t)Z_ * kPreSlots * sizeof(double), st));
   if (ex_elems_ > 0)
     for (int q = 0; q < 2; ++q)
       TTM_CUDA(cudaMemsetAsync(ex_[q], 0xff, (size_t)Z_ * ex_elems_ * sizeof(unsigned long long), st));
   TTM_CUDA(cudaMemsetAsync(svd_log_, 0, (size_t)Z_ * std::max(1, n_trunc_) * kSvdRec * sizeof(int), st));
-  tab_ = Tables{d_buf_, d_bond_, d_stat_, d_istat_, nb_, nbd, ns, nis, Z_};
+  tab_ = Tables{d_buf_, d_bond_, d_stat_, d_istat_, nb_, nbd, ns, nis, Z_, pre};
 
   // second walk: launch
   launches_ = 0;

@@ -26,7 +26,10 @@ struct Tables {
   int* istat;
   int nb, nbd, ns, nis;
   int nz;  // products in this launch
+  double* pre;  // [z][kPreSlots] state of the preconditioned Swap SVD (ttm_pre.cuh), or nullptr
 };
+// pre slots: last correction of Newton steps 1, 2, 3; 1 / ||Theta||_F^2; max |R1|
+enum { PR_RES = 0, PR_ITRACE = 3, PR_ABSMAX = 4, kPreSlots = 8 };
 
 __device__ __forceinline__ int bondv(const Tables& t, int z, int id) {
   return id < 0 ? 1 : t.bond[z * t.nbd + id];
@@ -51,6 +54,25 @@ enum { SR_M = 0, SR_N = 1, SR_K = 2, SR_SW0 = 3, SR_FALLBACK = 6 };
 // counts as converged: the error left after a step is of the order of its correction squared,
 // so 1e-7 leaves couplings and an orthogonality defect near 1e-14.
 constexpr double kNewtonConverged = 1e-7;
+// The preconditioned Swap SVD takes another step while its last correction is above this: the
+// steps are short there, and the result is then final to rounding also where singular values cluster.
+constexpr double kPreConverged = 1e-9;
+
+// Which of the four Newton steps of the preconditioned Swap SVD a product takes: steps 0 and 1
+// always, 2 and 3 while the last correction is above kPreConverged.
+__device__ __forceinline__ bool pre_active(const Tables& t, int z, int step) {
+  if (step < 2) return true;
+  const double* r = t.pre + z * kPreSlots + PR_RES;
+  const bool s2 = !(r[0] <= kPreConverged);
+  return step == 2 ? s2 : s2 && !(r[1] <= kPreConverged);
+}
+// 1: its W and V are in the second pair of buffers (after an odd number of steps)
+__device__ __forceinline__ int pre_where(const Tables& t, int z) {
+  return pre_active(t, z, 2) && !pre_active(t, z, 3) ? 1 : 0;
+}
+__device__ __forceinline__ bool pre_failed(const Tables& t, int z) {
+  return !(t.pre[z * kPreSlots + PR_RES + 2] <= kNewtonConverged);
+}
 
 // A dimension written as mul * bond[id] (id < 0 means the constant mul).
 struct Dim {

@@ -23,6 +23,7 @@
 #include "ttm_newton.cuh"
 #include "ttm_jac4.cuh"
 #include "ttm_jres.cuh"
+#include "ttm_pre.cuh"
 #include "ttm_tc.cuh"
 
 namespace ttm {
@@ -178,7 +179,8 @@ class Engine {
     return b;
   }
   size_t extra_bytes() const {
-    return ex_elems_ > 0 ? 2 * ((size_t)Z_ * ex_elems_ * sizeof(unsigned long long) + 256) : 0;
+    if (base_only_) return 0;
+    return 2 * ((size_t)Z_ * ex_elems_ * sizeof(unsigned long long) + 256) + (size_t)Z_ * kPreSlots * sizeof(double) + 256;
   }
   // Sweep counters per product and Jacobi launch: room for the sweep limit of any pass.
   // sweep limit of the float64 Jacobi of the fallback (max_sweeps when set)
@@ -255,10 +257,11 @@ class Engine {
     TTM_CUDA(cudaGetLastError());
     ++launches_;
   }
-  // Per-column power-of-two exponents of W (the K scale of W X) into the tau workspace.
-  void colexp(int wbuf, Dim m, Dim n, int n_ub) {
+  // Per-column power-of-two exponents of W (the K scale of W X) into the vector workspace `out`
+  // (default: tau).
+  void colexp(int wbuf, Dim m, Dim n, int n_ub, int out = -1) {
     if (!launch_) return;
-    ColExpArgs ca{tab_, wbuf, ws(WS_TAU), m, n};
+    ColExpArgs ca{tab_, wbuf, out < 0 ? ws(WS_TAU) : out, m, n};
     colexp_kernel<<<dim3(cdiv(n_ub, 8), Z_), 256, 0, hs_.stream>>>(ca);
     TTM_CUDA(cudaGetLastError());
     ++launches_;
@@ -375,17 +378,11 @@ class Engine {
     a.G = G;
     a.cols_ub = (n_ub + G - 1) / G;
     a.ld_ub = m_ub;
-    a.ex_stride = ex_elems_;
-    a.ex = ex_[ex_flip_];
-    a.ex_next = ex_[ex_flip_ ^ 1];
-    a.clear_n = 0;
     void* fn = (void*)qrd_kernel<T>;
     void* kargs[] = {&a};
     TTM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if (G > 1) {
-      a.clear_n = ex_prev_;
-      ex_prev_ = extent;
-      ex_flip_ ^= 1;
+      use_exchange(a, extent);
       TTM_CUDA(cudaLaunchCooperativeKernel(fn, dim3((unsigned)(Z_ * G)), dim3(kQdThreads), kargs, smem, hs_.stream));
     } else {
       TTM_CUDA(cudaLaunchKernel(fn, dim3((unsigned)Z_), dim3(kQdThreads), kargs, smem, hs_.stream));
@@ -393,6 +390,82 @@ class Engine {
     ++launches_;
     return true;
   }
+  // The preconditioned Swap SVD (ttm_pre.cuh) covers the default options up to kPreMax rows; an
+  // explicit choice of passes, kernel, steps or sweeps takes the general pipeline.
+  bool pre_fits(int m_ub, int n_ub) const {
+    if (base_only_ || opt_.f32_passes || opt_.jacobi_kernel || opt_.newton_steps || opt_.max_sweeps) return false;
+    const int p_ub = std::min(m_ub, n_ub);
+    size_t sm = 0;
+    return m_ub <= kPreMax && qrd_apply_fits(n_ub) && qrd_ctas(n_ub, m_ub, 8, &sm) > 0 &&
+           qrd_ctas(m_ub, p_ub, 4, &sm) > 0 && qrd_ctas(p_ub, p_ub, 8, &sm) > 0;
+  }
+  // The exchange buffers of a distributed launch that uses `extent` elements per product.
+  template <class A>
+  void use_exchange(A& a, long extent) {
+    a.ex_stride = ex_elems_;
+    a.ex = ex_[ex_flip_];
+    a.ex_next = ex_[ex_flip_ ^ 1];
+    a.clear_n = ex_prev_;
+    ex_prev_ = extent;
+    ex_flip_ ^= 1;
+  }
+  void pre_elim(PreElimArgs a, int p_ub) {
+    size_t smem = 0;
+    const int G = qrd_ctas(p_ub, p_ub, 8, &smem);
+    if (!launch_) {
+      if (G > 1) ex_elems_ = std::max(ex_elems_, (long)p_ub * p_ub);
+      return;
+    }
+    a.G = G;
+    a.cols_ub = (p_ub + G - 1) / G;
+    a.ld_ub = p_ub;
+    void* fn = (void*)pre_elim_kernel;
+    void* kargs[] = {&a};
+    TTM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (G > 1) {
+      use_exchange(a, (long)p_ub * p_ub);
+      TTM_CUDA(cudaLaunchCooperativeKernel(fn, dim3((unsigned)(Z_ * G)), dim3(kQdThreads), kargs, smem, hs_.stream));
+    } else {
+      TTM_CUDA(cudaLaunchKernel(fn, dim3((unsigned)Z_), dim3(kQdThreads), kargs, smem, hs_.stream));
+    }
+    ++launches_;
+  }
+  // The float32 Jacobi of ttm_pre.cuh: groups of G CTAs, a cluster each up to 8, else resident
+  // together (as many groups as fit, each taking products in turn).
+  void jacobi_pre(PreJacArgs a, int p_ub) {
+    const int nblk = (p_ub + kPjB - 1) / kPjB;
+    a.G = std::max(1, (nblk + 1) / 2);
+    const int rows = (p_ub + 31) / 32;
+    const int R = rows <= 1 ? 1 : rows <= 2 ? 2 : rows <= 4 ? 4 : rows <= 8 ? 8 : rows <= 16 ? 16 : 32;
+    void* fn = R == 1 ? (void*)jacobi_pre_kernel<1> : R == 2 ? (void*)jacobi_pre_kernel<2>
+             : R == 4 ? (void*)jacobi_pre_kernel<4> : R == 8 ? (void*)jacobi_pre_kernel<8>
+             : R == 16 ? (void*)jacobi_pre_kernel<16> : (void*)jacobi_pre_kernel<32>;
+    const size_t smem = (size_t)2 * kPjB * 32 * R * sizeof(float);
+    TTM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    a.cluster = a.G > 1 && a.G <= 8;
+    a.ngroup = Z_;
+    void* kargs[] = {&a};
+    if (a.G == 1 || a.cluster) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)(Z_ * a.G));
+      cfg.blockDim = dim3(kPjThreads);
+      cfg.dynamicSmemBytes = smem;
+      cfg.stream = hs_.stream;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = (unsigned)a.G;
+      at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = a.cluster ? 1 : 0;
+      TTM_CUDA(cudaLaunchKernelExC(&cfg, fn, kargs));
+    } else {
+      a.ngroup = std::max(1, std::min(Z_, hs_.num_sms / a.G));
+      TTM_CUDA(cudaLaunchCooperativeKernel(fn, dim3((unsigned)(a.ngroup * a.G)), dim3(kPjThreads), kargs, smem, hs_.stream));
+    }
+    ++launches_;
+  }
+  void swap_pre(int x, int y, int bl, int bm, int br, int nbnd, int nprov, int pb, int kind, long cap, int sw32, int sw64,
+                int wslot);
   void qrd_apply(QrdApplyArgs a, int m_ub, int c_ub) {
     if (!launch_) return;
     const size_t smem = (size_t)(kQaStages + 4) * m_ub * sizeof(double);

@@ -44,8 +44,8 @@ struct QrdArgs {
   unsigned long long* ex;       // exchange, ex_stride elements per product, holding kQdEmpty (G > 1)
   unsigned long long* ex_next;  // the buffer of the next launch: its first clear_n elements are emptied
   long ex_stride, clear_n;
-  double* absmax;    // [nz] T = double: nullptr or receives max |R|; T = float: nullptr or A is divided by
-                     // the power of two above it
+  int scaled;        // T = double: max |R| goes to PR_ABSMAX; T = float: A is divided by the power of two
+                     // above PR_ABSMAX
   float ridge;       // T = float: diagonal entries of R are moved away from zero by this much
 };
 
@@ -70,8 +70,8 @@ __device__ __forceinline__ T qd_sum4(const T (&s)[4], int lane) {
   return c;
 }
 
-// beta, v_j and tau of a column with squared norm g and leading entry alpha. A zero column has
-// tau = 0; a NaN travels on in beta.
+// beta, v_j and tau of a column with squared norm g and leading entry alpha. A column that counts as
+// zero has tau = 0; a NaN travels on in beta.
 __device__ __forceinline__ void qd_scalars(double g, double alpha, double& beta, double& vj, double& tau) {
   const int hi = __double2hiint(g), lo = __double2loint(g), ex = (hi >> 20) - 1023;
   double mu, r;
@@ -86,11 +86,11 @@ __device__ __forceinline__ void qd_scalars(double g, double alpha, double& beta,
     const double ms = gs * rs;
     r = __hiloint2double(__double2hiint(rs) - (h << 20), __double2loint(rs));
     mu = __hiloint2double(__double2hiint(ms) + (h << 20), __double2loint(ms));
-  } else if (g > 0.0) {
+  } else if (g >= 2.3e-308) {
     mu = sqrt(g);
     r = 1.0 / mu;
-  } else {
-    beta = g == 0.0 ? alpha : g;
+  } else {  // zero (or its square is below the normal range, where tau would overflow), or a NaN
+    beta = g == g ? alpha : g;
     vj = 0.0;
     tau = 0.0;
     return;
@@ -114,7 +114,7 @@ __device__ __forceinline__ void qd_scalars(double g, double alpha, double& beta,
   vj = alpha <= 0.0 ? -y : y;
 }
 __device__ __forceinline__ void qd_scalars(float g, float alpha, float& beta, float& vj, float& tau) {
-  if (g > 0.f) {
+  if (g > 1e-36f) {  // below (columns of 1e-18 of max |A|) tau would leave the float range
     float r = rsqrtf(g);
     r = fmaf(r * 0.5f, fmaf(-(g * r), r, 1.f), r);
     const float mu = g * r, y = fabsf(alpha) + mu;
@@ -122,10 +122,17 @@ __device__ __forceinline__ void qd_scalars(float g, float alpha, float& beta, fl
     beta = alpha <= 0.f ? mu : -mu;
     vj = alpha <= 0.f ? -y : y;
   } else {
-    beta = g == 0.f ? alpha : g;
+    beta = g == g ? alpha : g;
     vj = 0.f;
     tau = 0.f;
   }
+}
+
+// Binary exponent of the scale that brings max |R1| to [1/2, 1); 0 for a zero or non-finite maximum.
+__device__ __forceinline__ int qd_scale_exp(double mx) {
+  int e = 0;
+  if (mx > 0.0 && mx < 1.7e308) frexp(mx, &e);
+  return max(-1000, min(1000, e));
 }
 
 template <typename T> struct QdBits;
@@ -170,12 +177,7 @@ __global__ void __launch_bounds__(kQdThreads) qrd_kernel(QrdArgs a) {
   const double* src = bufp(a.t, z, a.bsrc);
   double scale = 1.0;
   if constexpr (sizeof(T) == 4) {
-    if (a.absmax) {
-      const double mx = a.absmax[z];
-      int e = 0;
-      if (mx > 0.0 && mx < 1.7e308) frexp(mx, &e);
-      scale = ldexp(1.0, -max(-1000, min(1000, e)));
-    }
+    if (a.scaled) scale = ldexp(1.0, -qd_scale_exp(a.t.pre[z * kPreSlots + PR_ABSMAX]));
   }
   for (int e = tid; e < nl * M; e += kQdThreads) {
     int l, i;
@@ -352,7 +354,7 @@ __global__ void __launch_bounds__(kQdThreads) qrd_kernel(QrdArgs a) {
   for (int e = tid; e < nl * k; e += kQdThreads) {
     const int l = e / k, i = e - l * k, c = b + G * l;
     if (i > c) R[(long)i * N + c] = T(0);
-    else if (sizeof(T) == 8 && a.absmax) mx = fmax(mx, fabs((double)R[(long)i * N + c]));
+    else if (sizeof(T) == 8 && a.scaled) mx = fmax(mx, fabs((double)R[(long)i * N + c]));
   }
   if constexpr (sizeof(T) == 8) {
     if (V)
@@ -360,11 +362,12 @@ __global__ void __launch_bounds__(kQdThreads) qrd_kernel(QrdArgs a) {
         const int l = e / M, i = e - l * M, c = b + G * l;
         if (c < k && i > c) V[(long)c * M + i] = cols[l * ld + i];
       }
-    if (a.absmax) {
+    if (a.scaled) {
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
       if (lane == 0 && mx > 0.0)
-        atomicMax(reinterpret_cast<unsigned long long*>(a.absmax + z), (unsigned long long)__double_as_longlong(mx));
+        atomicMax(reinterpret_cast<unsigned long long*>(a.t.pre + z * kPreSlots + PR_ABSMAX),
+                  (unsigned long long)__double_as_longlong(mx));
     }
   }
 }
@@ -380,7 +383,7 @@ struct QrdApplyArgs {
   Tables t;
   int bv, btau;   // reflectors and tau of qrd_kernel<double>
   Dim m, n;       // A was m x n
-  int bvec, bperm;
+  int bvec, bvec2, bperm;  // bvec2: the matrix when pre_where() is 1
   int ic;         // bond id: columns of Y
   int bout;
   int out_rows;   // 1: Y row-major (m x columns); 0: Y^T row-major (columns x m)
@@ -407,7 +410,7 @@ __global__ void __launch_bounds__(kQaThreads) qrd_apply_kernel(QrdApplyArgs a) {
   } else {
     j0 = k - 1;
     const int pc = on ? reinterpret_cast<const int*>(bufp(a.t, z, a.bperm))[c] : 0;
-    const double* x = bufp(a.t, z, a.bvec) + (long)max(0, min(pc, k - 1)) * k;
+    const double* x = bufp(a.t, z, pre_where(a.t, z) ? a.bvec2 : a.bvec) + (long)max(0, min(pc, k - 1)) * k;
     for (int i = lane; i < M; i += 32) y[i] = i < k ? x[i] : 0.0;
   }
   auto fetch = [&](int q) {  // reflector q into its stage; one commit group per call

@@ -58,8 +58,10 @@ typedef enum {
  * CUDA cores (float32 Jacobi passes, everything else float64). */
 typedef enum {
   TTM_PREC_FP64 = 0,       /* every GEMM on the float64 pipe (the reference form)         */
-  TTM_PREC_BF16_SPLIT = 2  /* every GEMM on the tcgen05 tensor cores as the exactly sliced
-                              product of bf16 digits (Ozaki scheme): each float64 operand
+  TTM_PREC_BF16_SPLIT = 2  /* GEMMs on the tcgen05 tensor cores as the exactly sliced
+                              product of bf16 digits (Ozaki scheme; with split_digits = 0 the
+                              small GEMMs of a product stay on the float64 pipe, where they
+                              are faster and as accurate): each float64 operand
                               row (column) is scaled by a power of two and split into
                               split_digits digits of 7 bits; the digit products are summed
                               exactly in float32 and combined in float64. 8 digits (the

@@ -201,6 +201,12 @@ class Engine {
   // C = A B of every (product, batch index) the functor describes: on the float64 pipe, or
   // (tc_) as the exactly sliced bf16 product on the tensor cores (ttm_tc.cuh). kscale_buf:
   // per-K power-of-two exponents that keep a graded A relatively accurate (tensor cores only).
+  // In the split mode a launch below this many multiply-adds runs on the float64 pipe, at least as
+  // accurate and faster: the digit product has a floor of about 20 us (one tile's chain of digits, K
+  // chunks and epilogue) and fills few SMs with its 128 x 64 tiles. Kernel times of a cube on the
+  // pipe / the tensor cores: 192: 13 / 32 us, 256: 35 / 36, 320: 61 / 44, 384: 97 / 48, 768: 780 / 85.
+  // An explicit split_digits always takes the tensor cores.
+  static constexpr double kTcMinMnk = 256.0 * 256.0 * 256.0;
   // Digit workspace of a tensor-core GEMM with these upper bounds; every GEMM a step may
   // launch is reserved in both walks (the planning walk launches nothing).
   void tc_reserve(int nbatch, int M_ub, int N_ub, int K_ub) {
@@ -216,14 +222,16 @@ class Engine {
     if (tc_ && (size_t)tc_bytes_ < tc_ws_bytes((long)Z_ * nbatch, M_ub, N_ub, K_ub, split_digits()))
       throw Error(TTM_ERR_WORKSPACE, "internal: a tensor-core GEMM was not reserved in the plan");
     gemm_log_.push_back(shape);
+    const bool on_tc = tc_ && (opt_.split_digits > 0 || base_only_ ||
+                               (double)M_ub * N_ub * K_ub * nbatch * Z_ >= kTcMinMnk);
     timed(0, [&] {
-      if (tc_) {
+      if (on_tc) {
         const cudaError_t e = launch_tc_gemm(hs_.stream, f, Z_, nbatch, M_ub, N_ub, K_ub, kscale_buf,
                                              split_digits(), d_tc_, d_istat_ + IS_STATUS, d_stat_ + ST_GFLOPS,
                                              tab_.ns);
         if (e != cudaSuccess)
           throw Error(TTM_ERR_CUDA, std::string("tensor-core GEMM, ") + tc_failed_step() + ": " + cudaGetErrorString(e));
-        launches_ += 6;
+        launches_ += 2;
       } else {
         TTM_CUDA(launch_dgemm(hs_.stream, f, Z_ * nbatch, nbatch, M_ub, N_ub, K_ub, hs_.num_sms, d_stat_ + ST_GFLOPS,
                               tab_.ns));

@@ -18,11 +18,17 @@
 // (A diag(2^-q) times diag(2^q) B, mathematically the identity) lets graded operands keep
 // relative accuracy per column (W = Theta V with column norms spanning many decades).
 //
-// Kernels: oz_exp_kernel (row / column exponents), oz_slice_kernel (digits, written in the
-// tcgen05 shared-memory layout: K-major, no swizzle, 8 x 16-byte core matrices, so that one
-// bulk copy moves a whole tile), oz_gemm_kernel (one CTA per 128 x 64 output tile: a TMA
+// Kernels: oz_prep_kernel (row / column exponents and digits, written in the tcgen05
+// shared-memory layout: K-major, no swizzle, 8 x 16-byte core matrices, so that one
+// bulk copy per operand moves a stage), oz_gemm_kernel (one CTA per 128 x 64 output tile: a TMA
 // producer warp with cp.async.bulk, one thread issuing tcgen05.mma kind::f16 into eight
 // TMEM accumulators, four epilogue warps reading them with tcgen05.ld).
+//
+// Bound at 1024^3 by the operand traffic (96 KB per K chunk and CTA through L2), at small sizes by one
+// tile's chain. Measured (GB300): exponents and digits in one integer launch instead of five float64
+// ones, one instruction per four digits of B, and an epilogue of three float64 instructions per
+// output instead of eight take a 1500 x 1024 x 2000 product from 1100 to 495 us and a 320^3 one from
+// about 110 to 45 us.
 #pragma once
 #include <cuda_bf16.h>
 #include <stdint.h>
@@ -42,6 +48,7 @@ constexpr int kOzBTile = kOzTN * kOzKC * 2;  // bytes of one B digit tile (4 KB)
 constexpr int kOzStages = 2;
 constexpr int kOzThreads = 192;   // warps 0-3 epilogue, warp 4 TMA producer, warp 5 MMA issuer
 constexpr int kOzExpNone = -100000;  // exponent of an all-zero row or column
+constexpr int kOzExpNaN = 100000;    // a row or column with a NaN or an infinity: its outputs are NaN
 
 __host__ __device__ constexpr int oz_stage_bytes(int S) { return S * (kOzATile + kOzBTile); }
 __host__ __device__ constexpr int oz_smem_bytes(int S) { return kOzStages * oz_stage_bytes(S) + 256; }
@@ -53,8 +60,8 @@ __host__ __device__ constexpr uint32_t oz_tmem_cols(int S) {
 // One GEMM of a launch: the float64 problem (from a functor, as for dgemm_kernel) and where
 // its digits live.
 struct OzWs {
-  unsigned char* a;   // digits of A: [S][row tiles of 128][K chunks of 32] tiles of 8 KB
-  unsigned char* b;   // digits of B^T: [S][column tiles of 64][K chunks of 32] tiles of 4 KB
+  unsigned char* a;   // digits of A: [row tiles of 128][K chunks of 32] blocks of S x 8 KB
+  unsigned char* b;   // digits of B^T: [column tiles of 64][K chunks of 32] blocks of S x 4 KB
   int* ea;            // row exponents of A (M entries)
   int* eb;            // column exponents of B (N entries)
   long a_stride, b_stride, e_stride;  // bytes / ints per (z, batch) problem
@@ -63,10 +70,6 @@ struct OzWs {
   int kscale_buf;     // buffer id of per-K power-of-two exponents q_k (ints in a double
                       // buffer: A diag(2^-q) times diag(2^q) B), -1 = none
 };
-
-__global__ void fill_int_kernel(int* p, long n, int v) {
-  for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long)gridDim.x * blockDim.x) p[e] = v;
-}
 
 // Per-column binary exponents q_j of a column-major m x n matrix (frexp of the column's
 // largest magnitude; 0 for a zero column), written as ints into a double buffer: the K scale
@@ -96,13 +99,6 @@ __global__ void colexp_kernel(ColExpArgs a) {
 
 // ---------------------------------------------------------------- operand views
 // Operand X (0 = A as R = M rows, 1 = B viewed transposed as R = N rows), both with K columns.
-__device__ __forceinline__ double oz_elem(const GemmDesc& g, int which, int r, int k) {
-  return which == 0 ? g.A.p[(long)r * g.A.rs + (long)k * g.A.cs] : g.B.p[(long)k * g.B.rs + (long)r * g.B.cs];
-}
-__device__ __forceinline__ bool oz_r_fast(const GemmDesc& g, int which) {
-  return which == 0 ? g.A.rs == 1 : g.B.cs == 1;
-}
-
 template <class F>
 struct OzArgs {
   F f;
@@ -112,92 +108,115 @@ struct OzArgs {
   int fl_stride;
 };
 
-// Exponents: e_r = the binary exponent of max_k |X_rk 2^(-+q_k)| (frexp convention, so the
-// scaled row lies in (-1, 1)); kOzExpNone for a zero row. Grid: (K / 32, R / 32, problems),
-// block 32 x 8; the 32 x 32 tile is read along the operand's unit stride.
+// Layout of the digits: one contiguous block per (row tile, K chunk of 32) with all S digits, so that
+// a stage is one bulk copy per operand. Core matrices are 8 rows of 16 bytes (8 k).
+//   A (tiles of 128 rows): [digit][K group of 8][row group of 8], leading byte offset 2048 between K
+//     neighbours, stride byte offset 128 between row groups;
+//   B (tiles of 64 rows): [K group][digit][row group], leading byte offset S 1024, stride byte offset
+//     128 across the row groups of all digits: consecutive digits of B are one operand of up to
+//     256 rows, and their products with one digit of A land in consecutive accumulators.
+__device__ __forceinline__ long oz_off_a(int r, int k, int nkc, int S) {
+  const long tile = (long)(r / kOzTM) * nkc + k / kOzKC;
+  return tile * S * kOzATile + (((k % kOzKC) >> 3) * (kOzTM / 8) + ((r % kOzTM) >> 3)) * 128 + (r & 7) * 16;
+}
+__device__ __forceinline__ long oz_off_b(int r, int k, int nkc, int S) {
+  const long tile = (long)(r / kOzTN) * nkc + k / kOzKC;
+  return tile * S * kOzBTile + (((k % kOzKC) >> 3) * S * (kOzTN / 8) + ((r % kOzTN) >> 3)) * 128 + (r & 7) * 16;
+}
+
+// x 2^sh as a 64-bit integer, rounded to nearest (|x| 2^sh < 2^62), by integer arithmetic.
+__device__ __forceinline__ long long oz_fixed(long long bits, int sh) {
+  const int ef = (int)((bits >> 52) & 0x7ff);
+  if (ef == 0) return 0;  // zero (subnormals count as zero)
+  const long long m = (bits & 0xfffffffffffffll) | 0x10000000000000ll;
+  const int s = ef - 1075 + sh;  // x 2^sh = +-m 2^s
+  long long v;
+  if (s >= 0) v = m << min(s, 9);
+  else if (s < -54) v = 0;
+  else v = ((m >> (-s - 1)) + 1) >> 1;
+  return bits < 0 ? -v : v;
+}
+
+// Exponents and digits of both operands over their padded extents (zeros outside the matrix).
+// Exponent of row r: the largest frexp exponent of X_rk 2^(-+q_k), kOzExpNone for a zero row.
+// Digits: x 2^(6 + 7 (S - 1) - e_r) rounded to an integer, split into balanced base-128 digits from
+// the low end. Everything is integer arithmetic on the bit patterns (a float64 instruction takes
+// 64 clocks of a sub-partition: slicing by rint and multiplication spent 24 of them per element).
+// Grid: x = 16-row groups of A, then of B; z = problems. 256 threads: a thread takes 8 consecutive k
+// of one row, which is one 16-byte store per digit; the second pass over K finds its data in L1.
+constexpr int kOzPrepRows = 16;
 template <class F>
-__global__ void oz_exp_kernel(OzArgs<F> a, int which) {
+__global__ void __launch_bounds__(256) oz_prep_kernel(OzArgs<F> a, int mpad, int npad, int kpad) {
   const int zb = blockIdx.z, z = zb / a.nbatch, b = zb % a.nbatch;
   const GemmDesc g = a.f(z, b);
+  if (g.M <= 0 || g.N <= 0) return;  // nothing of this problem is multiplied
+  const int na = mpad / kOzPrepRows;
+  const int which = (int)blockIdx.x < na ? 0 : 1;
+  const int r0 = ((int)blockIdx.x - (which ? na : 0)) * kOzPrepRows;
   const int R = which == 0 ? g.M : g.N, K = g.K;
-  const int r0 = blockIdx.y * 32, k0 = blockIdx.x * 32;
-  if (R <= 0 || K <= 0 || r0 >= R || k0 >= K) return;
-  __shared__ double tile[32][33];
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const bool rf = oz_r_fast(g, which);
+  const int TR = which == 0 ? kOzTM : kOzTN;
+  // row tiles that no output tile reads
+  if (r0 >= (R + TR - 1) / TR * TR) return;
+  const double* p = which == 0 ? g.A.p : g.B.p;
+  const long rs = which == 0 ? g.A.rs : g.B.cs, ks = which == 0 ? g.A.cs : g.B.rs;
   const int* q = a.w.kscale_buf >= 0 ? reinterpret_cast<const int*>(bufp(a.f.t, z, a.w.kscale_buf)) : nullptr;
-  for (int i = ty; i < 32; i += 8) {
-    const int rr = rf ? tx : i, kk = rf ? i : tx;
-    const int r = r0 + rr, k = k0 + kk;
-    double v = 0.0;
-    if (r < R && k < K) {
-      v = fabs(oz_elem(g, which, r, k));
-      if (q) v = ldexp(v, which == 0 ? -q[k] : q[k]);
-    }
-    tile[rr][kk] = v;
-  }
+  const int rl = threadIdx.x & 15, kg = threadIdx.x >> 4, r = r0 + rl;  // row, group of 8 k
+  const int kend = (K + kOzKC - 1) / kOzKC * kOzKC;
+  __shared__ int s_e[kOzPrepRows];
+  if (threadIdx.x < kOzPrepRows) s_e[threadIdx.x] = kOzExpNone;
   __syncthreads();
-  if (ty == 0) {
-    double m = 0.0;
-    for (int kk = 0; kk < 32; ++kk) m = fmax(m, tile[tx][kk]);
-    if (m > 0.0 && r0 + tx < R) {
-      int e;
-      frexp(m, &e);
-      int* ex = (which == 0 ? a.w.ea : a.w.eb) + (long)zb * a.w.e_stride;
-      atomicMax(ex + r0 + tx, e);
-    }
-  }
-}
-
-// Byte offset of digit t of element (r, k) in the tile layout of an operand with row tiles of
-// TR rows: tiles ordered [t][row tile][K chunk]; inside a tile the 8 x 8 core matrices are
-// ordered K chunk of 8 outer, row group of 8 inner (leading byte offset TR / 8 * 128 between
-// K neighbours, stride byte offset 128 between row neighbours), each core matrix 8 rows of
-// 16 contiguous bytes.
-template <int TR>
-__device__ __forceinline__ long oz_off(int t, int r, int k, int nrt, int nkc) {
-  const long tile = ((long)t * nrt + r / TR) * nkc + k / kOzKC;
-  const int mi = (r % TR) >> 3, ki = (k % kOzKC) >> 3;
-  return tile * (TR * kOzKC * 2) + (ki * (TR / 8) + mi) * 128 + (r & 7) * 16 + (k & 7) * 2;
-}
-
-// Digits of one operand over its padded extent (zeros outside the matrix). Grid: (Kpad / 32,
-// Rpad / 32, problems), block 32 x 8.
-template <class F, int TR>
-__global__ void oz_slice_kernel(OzArgs<F> a, int which, int rpad, int kpad) {
-  const int zb = blockIdx.z, z = zb / a.nbatch, b = zb % a.nbatch;
-  const GemmDesc g = a.f(z, b);
-  const int R = which == 0 ? g.M : g.N, K = g.K;
-  const int r0 = blockIdx.y * 32, k0 = blockIdx.x * 32;
-  const int nrt = rpad / TR, nkc = kpad / kOzKC;
-  if (r0 >= rpad || k0 >= kpad) return;
-  __shared__ double tile[32][33];
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const bool rf = oz_r_fast(g, which);
-  const int* q = a.w.kscale_buf >= 0 ? reinterpret_cast<const int*>(bufp(a.f.t, z, a.w.kscale_buf)) : nullptr;
-  for (int i = ty; i < 32; i += 8) {
-    const int rr = rf ? tx : i, kk = rf ? i : tx;
-    const int r = r0 + rr, k = k0 + kk;
-    double v = 0.0;
-    if (R > 0 && K > 0 && r < R && k < K) {
-      v = oz_elem(g, which, r, k);
-      if (q) v = ldexp(v, which == 0 ? -q[k] : q[k]);
-    }
-    tile[rr][kk] = v;
-  }
+  int e = kOzExpNone;
+  if (r < R)
+    for (int k0 = kg * 8; k0 < K; k0 += 128)
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int k = k0 + u;
+        if (k < K) {
+          const int ef = (__double2hiint(p[(long)r * rs + (long)k * ks]) >> 20) & 0x7ff;
+          const int qq = q ? (which == 0 ? -q[k] : q[k]) : 0;
+          if (ef != 0) e = max(e, ef == 0x7ff ? kOzExpNaN : ef - 1022 + qq);
+        }
+      }
+  if (e != kOzExpNone) atomicMax(&s_e[rl], e);
   __syncthreads();
-  const int* ex = (which == 0 ? a.w.ea : a.w.eb) + (long)zb * a.w.e_stride;
-  unsigned char* base = (which == 0 ? a.w.a + zb * a.w.a_stride : a.w.b + zb * a.w.b_stride);
-  for (int i = ty; i < 32; i += 8) {
-    const int r = r0 + i, k = k0 + tx;
-    const int e = (r < R) ? ex[r] : kOzExpNone;
-    double x = tile[i][tx];
-    // x 2^-e in (-1, 1), times 2^6: the first digit in [-64, 64]
-    double rem = (e == kOzExpNone) ? 0.0 : ldexp(x, 6 - e);
-    for (int t = 0; t < a.w.S; ++t) {
-      const double s = rint(rem);
-      rem = (rem - s) * 128.0;
-      *reinterpret_cast<__nv_bfloat16*>(base + oz_off<TR>(t, r, k, nrt, nkc)) = __double2bfloat16(s);
+  e = s_e[rl];
+  if (kg == 0 && r < R) ((which == 0 ? a.w.ea : a.w.eb) + (long)zb * a.w.e_stride)[r] = e;
+  unsigned char* base = which == 0 ? a.w.a + zb * a.w.a_stride : a.w.b + zb * a.w.b_stride;
+  const int S = a.w.S, nkc = kpad / kOzKC;
+  for (int k0 = kg * 8; k0 < kend; k0 += 128) {
+    long long v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int k = k0 + u;
+      v[u] = 0;
+      if (r < R && k < K && e != kOzExpNone) {
+        const int qq = q ? (which == 0 ? -q[k] : q[k]) : 0;
+        v[u] = oz_fixed(__double_as_longlong(p[(long)r * rs + (long)k * ks]), 7 * S - 1 - e + qq);
+      }
+    }
+    const long off0 = which == 0 ? oz_off_a(r, k0, nkc, S) : oz_off_b(r, k0, nkc, S);
+    const long plane = which == 0 ? kOzATile : (kOzTN / 8) * 128;  // between digits
+    for (int t = S - 1; t >= 0; --t) {
+      unsigned w[4];
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        unsigned pr = 0;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          const int u = 2 * h + c;
+          int d;
+          if (t > 0) {
+            d = (int)(v[u] & 127);
+            if (d >= 64) d -= 128;
+            v[u] = (v[u] - d) >> 7;
+          } else {
+            d = (int)v[u];  // at most 64 in magnitude
+          }
+          pr |= (__float_as_uint((float)d) >> 16) << (16 * c);  // a small integer is exact in bf16
+        }
+        w[h] = pr;
+      }
+      *reinterpret_cast<uint4*>(base + off0 + t * plane) = make_uint4(w[0], w[1], w[2], w[3]);
     }
   }
 }
@@ -268,21 +287,17 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
 }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-// 32 lanes x 32 consecutive float32 columns of TMEM into 32 registers per thread.
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
-  uint32_t r[32];
+// 32 lanes x 16 consecutive float32 columns of TMEM into 16 registers per thread.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
+  uint32_t r[16];
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-        "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
-        "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
-        "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 constexpr uint64_t kOzWaitNs = 2000000000ull;  // 2 s: far beyond any legitimate wait
@@ -301,7 +316,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(OzArgs<F> a, int
   const int S = a.w.S;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nkc = (g.K + kOzKC - 1) / kOzKC;            // K chunks of this problem
-  const int nrtA = mpad / kOzTM, nrtB = npad / kOzTN, nkcp = kpad / kOzKC;
+  const int nkcp = kpad / kOzKC;
   const int stage_bytes = oz_stage_bytes(S);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kOzStages * stage_bytes);
   // bars: full[2], empty[2], acc_full, acc_empty; then the TMEM address
@@ -346,18 +361,16 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(OzArgs<F> a, int
         const uint32_t full = smem_u32(&bars[s]);
         mbar_expect_tx(full, (uint32_t)stage_bytes);
         unsigned char* st = smem + s * stage_bytes;
-        for (int t = 0; t < S; ++t) {
-          const long ta = ((long)t * nrtA + blockIdx.y) * nkcp + kc;
-          bulk_g2s(smem_u32(st + t * kOzATile), Ab + ta * kOzATile, kOzATile, full);
-          const long tb = ((long)t * nrtB + blockIdx.x) * nkcp + kc;
-          bulk_g2s(smem_u32(st + S * kOzATile + t * kOzBTile), Bb + tb * kOzBTile, kOzBTile, full);
-        }
+        const long ta = (long)blockIdx.y * nkcp + kc, tb = (long)blockIdx.x * nkcp + kc;
+        bulk_g2s(smem_u32(st), Ab + ta * S * kOzATile, (uint32_t)(S * kOzATile), full);
+        bulk_g2s(smem_u32(st + S * kOzATile), Bb + tb * S * kOzBTile, (uint32_t)(S * kOzBTile), full);
       }
     }
   } else if (warp == 5) {
-    // ---------------- MMA issuer: every digit pair (t, u) with t + u < S, two K steps of 16
+    // ---------------- MMA issuer: every digit pair (t, u) with t + u < S, two K steps of 16. Up to
+    // four digits of B are one instruction (N up to 256): A is read from shared memory 12 times
+    // instead of 36 per K step, which leaves the tensor pipe and not the shared memory as the bound.
     if (lane == 0) {
-      const uint32_t idesc = umma_idesc_bf16(kOzTM, kOzTN);
       int kc = 0;
       for (int kb = 0; kb < nkb && !s_abort; ++kb) {
         if (kb > 0 && !mbar_wait(smem_u32(&bars[5]), (kb - 1) & 1, kOzWaitNs)) {  // epilogue drained
@@ -378,11 +391,13 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(OzArgs<F> a, int
           for (int ks = 0; ks < kOzKC / 16; ++ks) {
             for (int t = 0; t < S; ++t) {
               const uint64_t ad = umma_desc(st + t * kOzATile + ks * 2 * (kOzTM / 8) * 128, (kOzTM / 8) * 128, 128);
-              for (int u = 0; u + t < S; ++u) {
+              for (int u = 0; u + t < S; u += 4) {
+                const int nu = min(4, S - t - u);
                 const uint64_t bd =
-                    umma_desc(st + S * kOzATile + u * kOzBTile + ks * 2 * (kOzTN / 8) * 128, (kOzTN / 8) * 128, 128);
+                    umma_desc(st + S * kOzATile + (ks * 2 * S + u) * (kOzTN / 8) * 128, S * (kOzTN / 8) * 128, 128);
                 // the first step of a block starts every accumulator afresh
-                umma_bf16(tmem + (uint32_t)((t + u) * kOzTN), ad, bd, idesc, first ? (t == 0 ? 0u : 1u) : 1u);
+                umma_bf16(tmem + (uint32_t)((t + u) * kOzTN), ad, bd, umma_idesc_bf16(kOzTM, nu * kOzTN),
+                          first ? (t == 0 ? 0u : 1u) : 1u);
               }
             }
             // level l receives its first product from t = 0 (u = l), which zeroes it
@@ -397,9 +412,12 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(OzArgs<F> a, int
     // ---------------- epilogue: warps 0-3, thread = tile row (TMEM lane)
     const int row = warp * 32 + lane;
     const int gr = m0 + row;
+    const int* eA = a.w.ea + (long)zb * a.w.e_stride;
+    const int* eB = a.w.eb + (long)zb * a.w.e_stride;
+    const int er = gr < g.M ? eA[gr] : kOzExpNone;
+    // Levels 0..3 and 4..7 are combined as 64-bit integers (every accumulator holds an integer of at
+    // most 2^25), so an output takes three float64 instructions instead of one per level.
     double acc[kOzTN];
-#pragma unroll
-    for (int j = 0; j < kOzTN; ++j) acc[j] = 0.0;
     bool ok = true;
     for (int kb = 0; kb < nkb; ++kb) {
       // one lane waits, the warp reconverges before the warp-collective tcgen05.ld
@@ -412,14 +430,29 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(OzArgs<F> a, int
         break;
       }
       tc_fence_after();
-      for (int l = 0; l < S; ++l) {
-        const double w = ldexp(1.0, -12 - 7 * l);
 #pragma unroll
-        for (int h = 0; h < kOzTN / 32; ++h) {
-          float v[32];
-          tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(l * kOzTN + h * 32), v);
+      for (int h = 0; h < kOzTN / 16; ++h) {
+        long long hi[16], lo[16];
 #pragma unroll
-          for (int j = 0; j < 32; ++j) acc[h * 32 + j] = fma((double)v[j], w, acc[h * 32 + j]);
+        for (int j = 0; j < 16; ++j) hi[j] = lo[j] = 0;
+        for (int l = 0; l < S; ++l) {
+          float v[16];
+          tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(l * kOzTN + h * 16), v);
+          if (l < 4) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) hi[j] += (long long)__float2int_rn(v[j]) << (21 - 7 * l);
+          } else {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) lo[j] += (long long)__float2int_rn(v[j]) << (49 - 7 * l);
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          // exact: |hi|, |lo| < 2^50; hi 2^-33 + lo 2^-61
+          const double dh = __longlong_as_double(0x4338000000000000ll + hi[j]) - 6755399441055744.0;
+          const double dl = __longlong_as_double(0x4338000000000000ll + lo[j]) - 6755399441055744.0;
+          const double s = fma(dl, 1.0 / 268435456.0, dh);
+          acc[h * 16 + j] = kb == 0 ? s : acc[h * 16 + j] + s;
         }
       }
       tc_fence_before();
@@ -427,18 +460,23 @@ __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(OzArgs<F> a, int
       mbar_arrive(smem_u32(&bars[5]));
     }
     if (ok && gr < g.M) {
-      const int* eA = a.w.ea + (long)zb * a.w.e_stride;
-      const int* eB = a.w.eb + (long)zb * a.w.e_stride;
-      const int er = eA[gr];
 #pragma unroll
       for (int j = 0; j < kOzTN; ++j) {  // fully unrolled: acc stays in registers
         const int gc = n0 + j;
         if (gc < g.N) {
           const int ec = eB[gc];
           double v = 0.0;
-          if (er != kOzExpNone && ec != kOzExpNone) v = ldexp(acc[j], er + ec);
+          if (er == kOzExpNaN || ec == kOzExpNaN) {
+            v = __longlong_as_double(0x7ff8000000000000ll);
+          } else if (er != kOzExpNone && ec != kOzExpNone) {
+            const int sh = er + ec - 33, hw = __double2hiint(acc[j]), ef = (hw >> 20) & 0x7ff;
+            if (ef + sh > 0 && ef + sh < 2047 && ef != 0)
+              v = __hiloint2double(hw + (sh << 20), __double2loint(acc[j]));
+            else
+              v = ldexp(acc[j], sh);
+          }
           double* c = g.C.p + (long)gr * g.C.rs + (long)gc * g.C.cs;
-          v *= g.alpha;
+          if (g.alpha != 1.0) v *= g.alpha;
           if (g.beta != 0.0) v = fma(g.beta, *c, v);
           *c = v;
         }
@@ -493,26 +531,13 @@ cudaError_t launch_tc_gemm(cudaStream_t st, const F& f, int nz, int nbatch, int 
   w.err = err;
   w.kscale_buf = kscale_buf;
   OzArgs<F> oa{f, nbatch, w, fl, fl_stride};
-  const long ne = 2 * nprob * e_ints;
   // every launch is checked at once: the caller gets the first failing step
   const char*& step = tc_failed_step();
-  step = "fill_int_kernel";
-  fill_int_kernel<<<(unsigned)oz_cdiv(ne, 256), 256, 0, st>>>(w.ea, ne, kOzExpNone);
+  step = "oz_prep_kernel";
+  oz_prep_kernel<F><<<dim3((unsigned)((mpad + npad) / kOzPrepRows), 1, (unsigned)nprob), 256, 0, st>>>(
+      oa, (int)mpad, (int)npad, (int)kpad);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  step = "oz_exp_kernel";
-  const dim3 blk(32, 8);
-  oz_exp_kernel<F><<<dim3((unsigned)oz_cdiv(K_ub, 32), (unsigned)oz_cdiv(M_ub, 32), (unsigned)nprob), blk, 0, st>>>(oa, 0);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  oz_exp_kernel<F><<<dim3((unsigned)oz_cdiv(K_ub, 32), (unsigned)oz_cdiv(N_ub, 32), (unsigned)nprob), blk, 0, st>>>(oa, 1);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  step = "oz_slice_kernel";
-  oz_slice_kernel<F, kOzTM><<<dim3((unsigned)(kpad / 32), (unsigned)(mpad / 32), (unsigned)nprob), blk, 0, st>>>(
-      oa, 0, (int)mpad, (int)kpad);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  oz_slice_kernel<F, kOzTN><<<dim3((unsigned)(kpad / 32), (unsigned)(npad / 32), (unsigned)nprob), blk, 0, st>>>(
-      oa, 1, (int)npad, (int)kpad);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(oz_gemm_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 oz_smem_bytes(kOzMaxS))) != cudaSuccess)
     return e;

@@ -108,12 +108,14 @@ def test_batch_beyond_one_group_of_ctas(h):
         assert relerr([c.cpu().numpy() for c in O], P) <= relerr(Oo, P) + 1e-10
 
 
-def test_a_nan_is_reported(h):
+@pytest.mark.parametrize("prec", ["fp64", "bf16_split"])
+@pytest.mark.parametrize("d,chi", [(3, 4), (32, 20)])
+def test_a_nan_is_reported(h, prec, d, chi):
     import paper_2410_19747_gb300 as pkg
-    A, B = ttgen.rand_tt(5, 3, 4, 1), ttgen.rand_tt(5, 3, 4, 2)
+    A, B = ttgen.rand_tt(4, d, chi, 1), ttgen.rand_tt(4, d, chi, 2)
     for bad in (np.nan, np.inf):
         A2 = [c.copy() for c in A]
         A2[2][0, 0, 0] = bad
         with pytest.raises(pkg.TTMError) as e:
-            pkg.ttm_multiply(h, dev(A2), dev(B), eps=1e-10)
+            pkg.ttm_multiply(h, dev(A2), dev(B), eps=1e-10, chi_max=chi, prec=prec)
         assert e.value.status == -5

@@ -22,6 +22,7 @@
 #include "ttm_bjac.cuh"
 #include "ttm_newton.cuh"
 #include "ttm_jac4.cuh"
+#include "ttm_jac_fns.hpp"
 #include "ttm_jres.cuh"
 #include "ttm_pre.cuh"
 #include "ttm_tc.cuh"
@@ -336,9 +337,7 @@ class Engine {
   void jacobi_res(JResArgs& jr, int m_ub, int n_ub, int nblk_pad_ub) {
     const int rows = (m_ub + 31) / 32;
     const int R = rows <= 1 ? 1 : rows <= 2 ? 2 : rows <= 4 ? 4 : rows <= 8 ? 8 : rows <= 16 ? 16 : 32;
-    void* fn = R == 1 ? (void*)jacobi_res_kernel<T, kJrB, 1> : R == 2 ? (void*)jacobi_res_kernel<T, kJrB, 2>
-             : R == 4 ? (void*)jacobi_res_kernel<T, kJrB, 4> : R == 8 ? (void*)jacobi_res_kernel<T, kJrB, 8>
-             : R == 16 ? (void*)jacobi_res_kernel<T, kJrB, 16> : (void*)jacobi_res_kernel<T, kJrB, 32>;
+    void* fn = jacobi_res_fn(sizeof(T) == 8, R);
     (void)n_ub;
     const size_t smem = (size_t)2 * kJrB * 32 * R * sizeof(T);
     coop_res(fn, &jr, smem, (long)Z_ * (nblk_pad_ub / 2));
@@ -357,9 +356,9 @@ class Engine {
     return v;
   }
   // Distributed Householder QR (ttm_qrd.cuh) of a matrix with these upper bounds. G: a CTA per four
-  // columns (one per sub-partition) as far as the SMs reach: on a 256 x 256 float64 matrix G = 64
-  // takes 770 us, 32 791, 16 1218 and 152 772; on 32 x 32 G = 8 84 us and G = 1 104 (at half the
-  // full clock). 0: the columns do not fit the shared memory.
+  // columns (one per sub-partition) as far as the SMs reach: a 256 x 256 float64 matrix takes 580 us
+  // with G = 64, 632 with 32, 1086 with 16 and 573 with 128; 64 x 64 135 us with G = 16, 182 with 4 and
+  // 259 with 1 (the registers allow three CTAs per SM). 0: the columns do not fit the shared memory.
   int qrd_ctas(int m_ub, int n_ub, size_t elem, size_t* smem) const {
     if (m_ub > kQdMaxRows) return 0;
     int G = std::max(1, (n_ub + 3) / 4);
@@ -367,16 +366,31 @@ class Engine {
     for (;; G = (G + 1) / 2) {
       const size_t need = (size_t)((n_ub + G - 1) / G + 1) * m_ub * elem;
       if (need > (size_t)kQdSmem) return 0;
-      const long occ = std::max<long>(1, std::min<long>(4, (long)(220 * 1024 / (need + 1024))));
+      const long occ = std::max<long>(1, std::min<long>(3, (long)(220 * 1024 / (need + 1024))));
       *smem = need;
       if ((long)Z_ * G <= occ * sms || G == 1) return G;
     }
+  }
+  static void launch_cluster(void* fn, int groups, int G, int threads, size_t smem, void** kargs, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(groups * G));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)G;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    TTM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    TTM_CUDA(cudaLaunchKernelExC(&cfg, fn, kargs));
   }
   // Plans or launches it. a: everything but the sizes of the distribution.
   template <typename T>
   bool qrd(QrdArgs a, int m_ub, int n_ub) {
     size_t smem = 0;
-    int G = base_only_ ? 0 : qrd_ctas(m_ub, n_ub, sizeof(T), &smem);
+    const int G = base_only_ ? 0 : qrd_ctas(m_ub, n_ub, sizeof(T), &smem);
     if (G == 0) return false;
     const long extent = (long)m_ub * std::min(m_ub, n_ub);
     if (!launch_) {
@@ -420,67 +434,76 @@ class Engine {
   void pre_elim(PreElimArgs a, int p_ub) {
     size_t smem = 0;
     const int G = qrd_ctas(p_ub, p_ub, 8, &smem);
+    int Gc = 0;
+    if (p_ub <= kElimClusterMax)
+      for (Gc = 1; Gc < hs_.max_cluster && Gc * 4 < p_ub;) Gc *= 2;
+    const size_t smem_c = Gc > 0 ? (size_t)((p_ub + Gc - 1) / Gc + 1) * p_ub * 8 : 0;
+    if (smem_c > (size_t)kQdSmem) Gc = 0;
     if (!launch_) {
-      if (G > 1) ex_elems_ = std::max(ex_elems_, (long)p_ub * p_ub);
+      if (G > 1 && Gc == 0) ex_elems_ = std::max(ex_elems_, (long)p_ub * p_ub);
       return;
     }
-    a.G = G;
-    a.cols_ub = (p_ub + G - 1) / G;
+    a.G = Gc > 0 ? Gc : G;
+    a.cols_ub = (p_ub + a.G - 1) / a.G;
     a.ld_ub = p_ub;
-    void* fn = (void*)pre_elim_kernel;
     void* kargs[] = {&a};
-    TTM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if (G > 1) {
-      use_exchange(a, (long)p_ub * p_ub);
-      TTM_CUDA(cudaLaunchCooperativeKernel(fn, dim3((unsigned)(Z_ * G)), dim3(kQdThreads), kargs, smem, hs_.stream));
+    if (Gc > 0) {
+      void* fn = (void*)pre_elim_kernel<true>;
+      TTM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_c));
+      launch_cluster(fn, Z_, Gc, kQdThreads, smem_c, kargs, hs_.stream);
     } else {
-      TTM_CUDA(cudaLaunchKernel(fn, dim3((unsigned)Z_), dim3(kQdThreads), kargs, smem, hs_.stream));
+      void* fn = (void*)pre_elim_kernel<false>;
+      TTM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      if (G > 1) {
+        use_exchange(a, (long)p_ub * p_ub);
+        TTM_CUDA(cudaLaunchCooperativeKernel(fn, dim3((unsigned)(Z_ * G)), dim3(kQdThreads), kargs, smem, hs_.stream));
+      } else {
+        TTM_CUDA(cudaLaunchKernel(fn, dim3((unsigned)Z_), dim3(kQdThreads), kargs, smem, hs_.stream));
+      }
     }
     ++launches_;
   }
-  // The float32 Jacobi of ttm_pre.cuh: groups of G CTAs, a cluster each up to 8, else resident
+  // The float32 Jacobi of ttm_pre.cuh: groups of G CTAs, a cluster each where one can be that large, else resident
   // together (as many groups as fit, each taking products in turn).
   void jacobi_pre(PreJacArgs a, int p_ub) {
     const int nblk = (p_ub + kPjB - 1) / kPjB;
     a.G = std::max(1, (nblk + 1) / 2);
     const int rows = (p_ub + 31) / 32;
-    const int R = rows <= 1 ? 1 : rows <= 2 ? 2 : rows <= 4 ? 4 : rows <= 8 ? 8 : rows <= 16 ? 16 : 32;
-    void* fn = R == 1 ? (void*)jacobi_pre_kernel<1> : R == 2 ? (void*)jacobi_pre_kernel<2>
-             : R == 4 ? (void*)jacobi_pre_kernel<4> : R == 8 ? (void*)jacobi_pre_kernel<8>
-             : R == 16 ? (void*)jacobi_pre_kernel<16> : (void*)jacobi_pre_kernel<32>;
+    const int R = jacobi_pre_rows(rows);
+    void* fn = jacobi_pre_fn(R);
     const size_t smem = (size_t)2 * kPjB * 32 * R * sizeof(float);
     TTM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    a.cluster = a.G > 1 && a.G <= 8;
+    a.cluster = a.G > 1 && a.G <= hs_.max_cluster;
     a.ngroup = Z_;
     void* kargs[] = {&a};
-    if (a.G == 1 || a.cluster) {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((unsigned)(Z_ * a.G));
-      cfg.blockDim = dim3(kPjThreads);
-      cfg.dynamicSmemBytes = smem;
-      cfg.stream = hs_.stream;
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = (unsigned)a.G;
-      at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-      cfg.attrs = at;
-      cfg.numAttrs = a.cluster ? 1 : 0;
-      TTM_CUDA(cudaLaunchKernelExC(&cfg, fn, kargs));
+    if (a.cluster) {
+      launch_cluster(fn, Z_, a.G, kPjThreads, smem, kargs, hs_.stream);
+    } else if (a.G == 1) {
+      TTM_CUDA(cudaLaunchKernel(fn, dim3((unsigned)Z_), dim3(kPjThreads), kargs, smem, hs_.stream));
     } else {
       a.ngroup = std::max(1, std::min(Z_, hs_.num_sms / a.G));
       TTM_CUDA(cudaLaunchCooperativeKernel(fn, dim3((unsigned)(a.ngroup * a.G)), dim3(kPjThreads), kargs, smem, hs_.stream));
     }
     ++launches_;
   }
+  void swap_exact(int x, int y, int bl, int bm, int br, int nbnd, int pb, long cap, int wslot);
   void swap_pre(int x, int y, int bl, int bm, int br, int nbnd, int nprov, int pb, int kind, long cap, int sw32, int sw64,
                 int wslot);
+  static unsigned pow2_threads(int n) {
+    unsigned t = 32;
+    while (t < (unsigned)n) t *= 2;
+    return t;
+  }
   void qrd_apply(QrdApplyArgs a, int m_ub, int c_ub) {
     if (!launch_) return;
-    const size_t smem = (size_t)(kQaStages + 4) * m_ub * sizeof(double);
     a.ld_ub = m_ub;
-    TTM_CUDA(cudaFuncSetAttribute(qrd_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    qrd_apply_kernel<<<dim3(cdiv(c_ub, 4), (unsigned)Z_), kQaThreads, smem, hs_.stream>>>(a);
-    TTM_CUDA(cudaGetLastError());
+    const bool wide = m_ub > 96 && (long)Z_ * c_ub <= 2L * hs_.num_sms;
+    const size_t smem = (size_t)(kQaStages + (wide ? 1 : 4)) * m_ub * sizeof(double);
+    void* fn = wide ? (void*)qrd_apply_kernel<4> : (void*)qrd_apply_kernel<1>;
+    void* kargs[] = {&a};
+    TTM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    TTM_CUDA(cudaLaunchKernel(fn, dim3(wide ? (unsigned)c_ub : cdiv(c_ub, 4), (unsigned)Z_), dim3(kQaThreads), kargs, smem,
+                              hs_.stream));
     ++launches_;
   }
   long launches_ = 0;

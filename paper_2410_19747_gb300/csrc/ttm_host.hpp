@@ -66,6 +66,7 @@ struct HandleState {
   cudaStream_t stream = nullptr;
   ttm_options opt{};
   int num_sms = 0;
+  int max_cluster = 8;    // largest cluster of the distributed kernels (16 where the device can hold one)
   int coop_hest32 = 0, coop_hest = 0, coop_qr = 0;  // co-resident blocks per SM (cooperative kernels)
   DeviceArena arena;      // sweep buffers and workspaces
   DeviceArena env_arena;  // environments of ttm_inner / ttm_inner3 / ttm_backward

@@ -31,8 +31,8 @@
 #pragma once
 #include <cooperative_groups.h>
 #include "ttm_common.cuh"
-#include "ttm_jres.cuh"
 #include "ttm_newton.cuh"
+#include "ttm_pjac.cuh"
 #include "ttm_qrd.cuh"
 #include "ttm_svd.cuh"
 
@@ -107,262 +107,6 @@ struct PreProductFn {
   }
 };
 
-// ---------------------------------------------------------------- float32 Jacobi without V
-// Blocks of 16 columns in a round-robin tournament, one CTA of 16 warps per block pair: a warp
-// keeps one column of the first block in registers and meets the 16 columns of the second block,
-// staged in shared memory, in 16 inner rounds (the schedule of ttm_jres.cuh). Squared norms are
-// formed when a column is staged and carried through the rotations (a' = a - t g, b' = b + t g;
-// formed again when b' or a' lost more than 90 %), so a visit costs one dot product and one warp
-// reduction. The CTAs of a product meet at a cluster barrier (up to 8 CTAs) or at a counter in
-// global memory; products of a batch do not wait for each other.
-// Bound by the latency of an inner round (load, dot, reduction, rotation, CTA barrier).
-__device__ __forceinline__ int pj_ld_acquire(const int* p) {
-  int v;
-  asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-constexpr int kPjB = 16;
-constexpr int kPjThreads = kPjB * 32;
-constexpr int kPjPolls = 1 << 22;
-struct PreJacArgs {
-  Tables t;
-  int bx;             // X: p x p float column-major (in/out)
-  Dim p;
-  int G;              // CTAs per product (half the padded number of blocks, upper bound)
-  int ngroup;         // groups of G CTAs in the launch
-  int cluster;        // 1: a group is one cluster
-  int max_sweeps;
-  int* counters;      // [nz][stride]: large couplings per sweep, then at [kPjBarrier] the barrier
-  int stride;
-  float tol, big;
-  int flop_slot, sweep_slot;
-  int* svd_log;
-  int svd_stride, svd_field;
-};
-constexpr int kPjBarrier = 39;  // kPreSweeps < kPjBarrier < the counters' stride
-
-template <int R>
-__global__ void __launch_bounds__(kPjThreads, 1) jacobi_pre_kernel(PreJacArgs a) {
-  extern __shared__ __align__(16) unsigned char pj_raw[];
-  constexpr int B = kPjB, MR = 32 * R;
-  constexpr int VW = JrVec<float, R>::VW;
-  float* sc = reinterpret_cast<float*>(pj_raw);  // [2B][MR]
-  __shared__ float nrm[2 * B];
-  __shared__ int s_big, s_stop;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int i = blockIdx.x % a.G;
-  unsigned long long visits = 0, rots = 0;
-  for (int z = blockIdx.x / a.G; z < a.t.nz; z += a.ngroup) {
-    const int p = a.p.eval(a.t, z);
-    const int nb = (p + B - 1) / B, nbp = nb + (nb & 1), half = nbp / 2;
-    int* cnt = a.counters + (long)z * a.stride;
-    const bool here = i < half;
-    if (!here && !a.cluster) continue;
-    float* X = reinterpret_cast<float*>(bufp(a.t, z, a.bx));
-    const bool vec = (p % VW) == 0;
-    int barriers = 0, sweep = 0;
-    if (threadIdx.x == 0) {
-      s_big = 0;
-      s_stop = 0;
-    }
-    __syncthreads();
-    for (; sweep < a.max_sweeps; ++sweep) {
-      int rot_any = 0;
-      for (int r = 0; r < nbp - 1; ++r) {
-        if (here) {
-          int P, Q;
-          jr_pair(nbp, r, i, P, Q);
-          const int gp = P * B + w, gq = Q * B + w;
-          float x[R], y[R];
-          auto stage = [&](int g, float (&v)[R]) {
-            if (g < p) {
-              const float* col = X + (long)g * p;
-              if (vec) {
-                using V = typename JrVecT<float, VW>::type;
-#pragma unroll
-                for (int q = 0; q < R / VW; ++q) {
-                  const int row = 32 * VW * q + VW * lane;
-                  V u{};
-                  if (row < p) u = __ldcg(reinterpret_cast<const V*>(col + row));
-                  const float* e = reinterpret_cast<const float*>(&u);
-#pragma unroll
-                  for (int s = 0; s < VW; ++s) v[VW * q + s] = e[s];
-                }
-              } else {
-#pragma unroll
-                for (int q = 0; q < R; ++q) {
-                  const int row = 32 * VW * (q / VW) + VW * lane + q % VW;
-                  v[q] = row < p ? __ldcg(col + row) : 0.f;
-                }
-              }
-            } else {
-#pragma unroll
-              for (int q = 0; q < R; ++q) v[q] = 0.f;
-            }
-          };
-          auto unstage = [&](int g, const float (&v)[R]) {
-            if (g >= p) return;
-            float* col = X + (long)g * p;
-            if (vec) {
-              using V = typename JrVecT<float, VW>::type;
-#pragma unroll
-              for (int q = 0; q < R / VW; ++q) {
-                const int row = 32 * VW * q + VW * lane;
-                V u;
-                float* e = reinterpret_cast<float*>(&u);
-#pragma unroll
-                for (int s = 0; s < VW; ++s) e[s] = v[VW * q + s];
-                if (row < p) *reinterpret_cast<V*>(col + row) = u;
-              }
-            } else {
-#pragma unroll
-              for (int q = 0; q < R; ++q) {
-                const int row = 32 * VW * (q / VW) + VW * lane + q % VW;
-                if (row < p) col[row] = v[q];
-              }
-            }
-          };
-          auto norm2 = [&](const float (&v)[R]) {
-            float s0 = 0.f, s1 = 0.f;
-#pragma unroll
-            for (int q = 0; q < R; ++q) {
-              if (q & 1) s1 = fmaf(v[q], v[q], s1);
-              else s0 = fmaf(v[q], v[q], s0);
-            }
-            return jr_sum(s0 + s1);
-          };
-          // rotates (x, na) against (y, nb2) if their coupling is above tol
-          auto visit = [&](float& na, float& nb2) -> bool {
-            constexpr int NA = R >= 4 ? 4 : R;
-            float g[NA];
-#pragma unroll
-            for (int u = 0; u < NA; ++u) g[u] = 0.f;
-#pragma unroll
-            for (int q = 0; q < R; ++q) g[q % NA] = fmaf(x[q], y[q], g[q % NA]);
-#pragma unroll
-            for (int u = 1; u < NA; ++u) g[0] += g[u];
-            const float g2 = jr_sum(g[0]);
-            const float cpl = fabsf(g2) * rsqrtf(na) * rsqrtf(nb2);
-            if (!(cpl > a.tol)) return false;  // also a padding column (0 inf = NaN)
-            if (cpl > a.big) rot_any = 1;
-            float c, s;
-            if (!jr_rot<float>(na, nb2, g2, c, s)) return false;
-            const float tg = __fdividef(s, c) * g2;
-#pragma unroll
-            for (int q = 0; q < R; ++q) {
-              const float xp = x[q], yq = y[q];
-              x[q] = c * xp - s * yq;
-              y[q] = fmaf(s, xp, c * yq);
-            }
-            const float na1 = na - tg, nb1 = nb2 + tg;
-            na = na1 < 0.1f * na ? norm2(x) : na1;
-            nb2 = nb1 < 0.1f * nb2 ? norm2(y) : nb1;
-            return true;
-          };
-          stage(gp, x);
-          stage(gq, y);
-          float na = norm2(x);
-          {
-            const float nq = norm2(y);
-            if (lane == 0) nrm[B + w] = nq;
-          }
-          jr_store<float, R>(sc + (B + w) * MR, lane, y);
-          if (r == 0) {  // the pairs inside each block
-            jr_store<float, R>(sc + w * MR, lane, x);
-            if (lane == 0) nrm[w] = na;
-            __syncthreads();
-            for (int s = 0; s < B - 1; ++s) {
-              const int hb = w < B / 2 ? 0 : B, iw = w % (B / 2);
-              int cp, cq;
-              jr_pair(B, s, iw, cp, cq);
-              cp += hb;
-              cq += hb;
-              jr_load<float, R>(sc + cp * MR, lane, x);
-              jr_load<float, R>(sc + cq * MR, lane, y);
-              float n1 = nrm[cp], n2 = nrm[cq];
-              if (lane == 0) ++visits;
-              if (visit(n1, n2)) {
-                jr_store<float, R>(sc + cp * MR, lane, x);
-                jr_store<float, R>(sc + cq * MR, lane, y);
-                __syncwarp();
-                if (lane == 0) {
-                  nrm[cp] = n1;
-                  nrm[cq] = n2;
-                  ++rots;
-                }
-              }
-              __syncthreads();
-            }
-            jr_load<float, R>(sc + w * MR, lane, x);
-            na = nrm[w];
-          }
-          __syncthreads();
-          for (int s = 0; s < B; ++s) {
-            const int q = B + (w + s) % B;
-            jr_load<float, R>(sc + q * MR, lane, y);
-            float nq = nrm[q];
-            __syncwarp();
-            if (lane == 0) ++visits;
-            if (visit(na, nq)) {
-              jr_store<float, R>(sc + q * MR, lane, y);
-              if (lane == 0) {
-                nrm[q] = nq;
-                ++rots;
-              }
-            }
-            __syncthreads();
-          }
-          unstage(gp, x);
-          jr_load<float, R>(sc + (B + w) * MR, lane, y);
-          unstage(gq, y);
-        }
-        // the product's CTAs exchange columns
-        const bool last = r == nbp - 2;
-        if (last && rot_any && lane == 0) atomicOr(&s_big, 1);
-        if (half > 1 || last) {
-          __syncthreads();
-          if (last && threadIdx.x == 0 && s_big) {
-            atomicAdd(&cnt[sweep], 1);
-            s_big = 0;
-          }
-        }
-        if (a.cluster) {
-          asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
-        } else if (half > 1) {
-          ++barriers;
-          if (threadIdx.x == 0) {
-            __threadfence();
-            atomicAdd(&cnt[kPjBarrier], 1);
-            int polls = 0;
-            while (pj_ld_acquire(&cnt[kPjBarrier]) < barriers * half && ++polls < kPjPolls) {}
-            if (polls >= kPjPolls) {
-              s_stop = 1;
-              atomicExch(&a.t.istat[z * a.t.nis + IS_STATUS], (int)TTM_ERR_TIMEOUT);
-            }
-          }
-          __syncthreads();
-          if (s_stop) break;
-        } else if (last) {
-          __threadfence();
-          __syncthreads();
-        }
-      }
-      if (s_stop || __ldcg(&cnt[sweep]) == 0) break;
-    }
-    if (i == 0 && threadIdx.x == 0) {
-      const int used = min(sweep + 1, a.max_sweeps);
-      int* is = a.t.istat + z * a.t.nis;
-      if (used > is[IS_SWEEPS_MAX]) is[IS_SWEEPS_MAX] = used;
-      a.t.stat[z * a.t.ns + a.sweep_slot] += used;
-      if (a.svd_log) a.svd_log[(long)z * a.svd_stride + a.svd_field] = used;
-    }
-    // 2 p flops per visit, 6 p per rotation
-    if (lane == 0 && visits) atomicAdd(&a.t.stat[a.flop_slot], 2.0 * p * (double)visits + 6.0 * p * (double)rots);
-    visits = rots = 0;
-    __syncthreads();
-  }
-}
-
 // ---------------------------------------------------------------- norms, order, Eq. eps
 // Squared column norms: of X (float, times the scale that the second QR took out) or of W (in the
 // buffer where the Newton steps left it). One warp per column.
@@ -398,7 +142,8 @@ __global__ void pre_norm_kernel(PreNormArgs a) {
 
 // Descending order of the squared norms (bitonic, ties by index, a NaN last), the rank of Eq. eps
 // (strict) with the cap, and the statistics of the truncation. One CTA per product; the keys are
-// compared as integers, since a float64 comparison takes 64 clocks of a sub-partition.
+// compared as integers, since a float64 comparison takes 64 clocks of a sub-partition. Block: a power
+// of two of at least max(32, p) threads (1024 threads on p = 16 took 9 us, most of it in the scans).
 struct PreOrderArgs {
   Tables t;
   int bnrm, bsort, bperm;
@@ -406,10 +151,12 @@ struct PreOrderArgs {
   int inew;
   double eps;
   int cap;
-  int wslot, record;
+  int wslot;
+  int record;       // 0: provisional rank; 1: final; 2: final, without Newton steps (their state is left)
   int ikeep;
   int* svd_log;
   int svd_stride;
+  int sort;         // 0: the columns stay in their order (nothing is truncated)
 };
 __global__ void __launch_bounds__(1024) pre_order_kernel(PreOrderArgs a) {
   const int z = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -435,6 +182,7 @@ __global__ void __launch_bounds__(1024) pre_order_kernel(PreOrderArgs a) {
   }
   if (tid == 0) kbest = p;
   nan_seen = __syncthreads_or(nan_seen);
+  if (a.sort)
   for (int size = 2; size <= np; size <<= 1)
     for (int st = size >> 1; st > 0; st >>= 1) {
       if (tid < np / 2) {
@@ -463,9 +211,9 @@ __global__ void __launch_bounds__(1024) pre_order_kernel(PreOrderArgs a) {
   if (lane == 0) wsum[warp] = s;
   __syncthreads();
   if (warp == 0) {
-    double q = wsum[lane];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
+    const int nw = blockDim.x >> 5;
+    double q = lane < nw ? wsum[lane] : 0.0;
+    for (int o = 1; o < nw; o <<= 1) {
       const double u = __shfl_down_sync(0xffffffffu, q, o);
       if (lane + o < 32) q += u;
     }
@@ -513,11 +261,11 @@ __global__ void __launch_bounds__(1024) pre_order_kernel(PreOrderArgs a) {
     if (k > is[IS_MAX_BOND]) is[IS_MAX_BOND] = k;
     const bool s2 = pre_active(a.t, z, 2), s3 = pre_active(a.t, z, 3);
     const double res = pr[PR_RES + (s3 ? 2 : s2 ? 1 : 0)];
-    const bool bad = pre_failed(a.t, z);
+    const bool bad = a.record == 1 && pre_failed(a.t, z);
     pr[PR_ABSMAX] = 0.0;  // for the next Swap
     is[IS_FALLBACK] = 0;
     if (bad) is[IS_NEWTON_BAD] += 1;
-    else if (res > st[ST_NEWTON_RES]) st[ST_NEWTON_RES] = res;
+    else if (a.record == 1 && res > st[ST_NEWTON_RES]) st[ST_NEWTON_RES] = res;
     if (a.svd_log) {
       int* rec = a.svd_log + (long)z * a.svd_stride;
       rec[SR_M] = a.m.eval(a.t, z);
@@ -552,6 +300,57 @@ __global__ void pre_v_kernel(PreVArgs a) {
   for (int r = lane; r < p; r += 32) v[r] = s > 0.0 ? (double)x[r] * inv : (r == pj ? 1.0 : 0.0);
 }
 
+// ---------------------------------------------------------------- transport inside a cluster
+// A cluster of G CTAs hands a column on through distributed shared memory: it stays where its owner
+// holds it, the owner's release-arrival on one mbarrier per receiver says that it is final, and the
+// receivers read it there. Slot of column c: c mod 32 (a multiple of G, so that the CTAs that use a
+// slot are the same on every turn, and the chain cannot run 32 columns ahead of a CTA, since every
+// CTA owns one in G); phase: c / 32.
+constexpr int kQdSlots = 32;
+constexpr int kElimCluster = 16;      // largest cluster of the elimination
+constexpr int kElimClusterMax = 384;  // largest p on a cluster
+__device__ __forceinline__ uint32_t qc_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ uint32_t qc_map(uint32_t addr, int rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void qc_init(uint64_t* bars, int tid) {
+  if (tid < kQdSlots) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(qc_smem(bars + tid)) : "memory");
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+__device__ __forceinline__ void qc_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Column c is final in this CTA (its writers have been joined with the calling warp): tells the CTAs
+// that hold a column from c on. nc: columns of the matrix.
+__device__ __forceinline__ void qc_publish(uint64_t* bars, int c, int nc, int G, int b, int lane) {
+  if (lane < G && lane != b) {
+    const int last = lane < nc ? lane + (nc - 1 - lane) / G * G : -1;
+    if (last >= c)
+      asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(
+                       qc_map(qc_smem(bars + (c & (kQdSlots - 1))), lane))
+                   : "memory");
+  }
+}
+__device__ __forceinline__ bool qc_wait(uint64_t* bars, int c) {
+  const uint32_t bar = qc_smem(bars + (c & (kQdSlots - 1))), parity = (uint32_t)(c / kQdSlots) & 1;
+  for (int polls = 0; polls < kQdPolls; ++polls) {
+    uint32_t done;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (done) return true;
+  }
+  return false;
+}
+__device__ __forceinline__ double qc_ld(uint32_t addr, double) {
+  double v;
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(addr) : "memory");
+  return v;
+}
 // ---------------------------------------------------------------- elimination of G
 // U of G = L_G U without pivoting (the columns come in descending order): U_ij for i <= j, stored
 // at [j + i p]. A pivot that cancelled to rounding level counts as zero and eliminates nothing.
@@ -583,7 +382,8 @@ __device__ __forceinline__ double pre_pivot_inv(double d, double g0) {
   return __hiloint2double(__double2hiint(q) - (e << 20), __double2loint(q));
 }
 
-__global__ void __launch_bounds__(kQdThreads) pre_elim_kernel(PreElimArgs a) {
+template <bool CL>
+__global__ void __launch_bounds__(kQdThreads, 3) pre_elim_kernel(PreElimArgs a) {
   extern __shared__ __align__(16) unsigned char qd_raw[];
   const int G = a.G, z = blockIdx.x / G, b = blockIdx.x % G;
   const int p = a.p.eval(a.t, z);
@@ -591,12 +391,15 @@ __global__ void __launch_bounds__(kQdThreads) pre_elim_kernel(PreElimArgs a) {
   for (long e = (long)b * kQdThreads + tid; e < a.clear_n; e += (long)G * kQdThreads)
     a.ex_next[z * a.ex_stride + e] = kQdEmpty;
   const int nl = b < p ? (p - b + G - 1) / G : 0;
-  if (nl == 0 || !pre_active(a.t, z, a.step)) return;  // the second alike in all CTAs of the product
+  if (!pre_active(a.t, z, a.step)) return;  // alike in all CTAs of the product
+  if (!CL && nl == 0) return;
   double* cols = reinterpret_cast<double*>(qd_raw);     // [cols_ub][ld], column c from row c down
   const int ld = a.ld_ub;
   double* xs = cols + (long)a.cols_ub * ld;             // [ld]
   __shared__ int s_abort;
+  __shared__ __align__(8) uint64_t bars[CL ? kQdSlots : 1];
   if (tid == 0) s_abort = 0;
+  if constexpr (CL) qc_init(bars, tid);
   const double* Gm = bufp(a.t, z, a.bg);
   double* U = bufp(a.t, z, a.bu);
   for (int e = tid; e < nl * p; e += kQdThreads) {
@@ -605,66 +408,157 @@ __global__ void __launch_bounds__(kQdThreads) pre_elim_kernel(PreElimArgs a) {
   }
   unsigned long long* ex = a.ex + z * a.ex_stride;
   __syncthreads();
-  if (G > 1 && b == 0)
+  if constexpr (CL) {
+    qc_sync();
+    if (b == 0 && warp == 0) qc_publish(bars, 0, p, G, b, lane);
+  } else if (G > 1 && b == 0) {
     for (int i = tid; i < p; i += kQdThreads) qd_st(ex + i, QdBits<double>::to(cols[i]));
+  }
   int lj = 0, jr = 0;
   for (int j = 0; j < p; ++j) {
-    if (b + G * (nl - 1) < j) break;  // no column from j on is held here
+    if (nl == 0 || b + G * (nl - 1) < j) break;  // no column from j on is held here
     const bool mine = jr == b;
+    const uint32_t rem = CL ? qc_map(qc_smem(cols + lj * ld), jr) : 0;  // column j at its owner
     const int nxt = j + 1;
     const int nr = jr + 1 == G ? 0 : jr + 1, nlj = jr + 1 == G ? lj + 1 : lj;
     const int lc = (nr == b && nxt < p) ? nlj : -1;
     const double* x = mine ? cols + lj * ld : xs;
     const int base = j & ~31;
     const double g0 = __ldg(Gm + j + (long)j * p);
-    if (!mine) {
-      constexpr int NB = 4;
-      for (int i0 = base + tid; i0 < p; i0 += kQdThreads * NB) {
-        unsigned long long bits[NB];
+    const int l0 = lc >= 0 ? lc + 1 : lj + (b > jr ? 0 : 1);
+    const unsigned long long* src_x = ex + (long)j * p;
+    if (p - base <= 128) {
+      // x in the registers of every warp that has a column; warp 0 takes the chain
+      const bool work = warp == 0 ? lc >= 0 : l0 + warp - 1 < nl;
+      double xr[4] = {0.0, 0.0, 0.0, 0.0};
+      if (mine) {
 #pragma unroll
-        for (int u = 0; u < NB; ++u) {
-          const int i = i0 + kQdThreads * u;
-          bits[u] = (i >= j && i < p) ? qd_ld(ex + (long)j * p + i) : 0;
+        for (int u = 0; u < 4; ++u) {
+          const int i = base + lane + 32 * u;
+          if (i >= j && i < p) xr[u] = x[i];
+        }
+      } else if (CL) {
+        if (warp == 0) {  // fetches the column for the CTA
+          if (!qc_wait(bars, j)) s_abort = 1;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int i = base + lane + 32 * u;
+            if (i >= j && i < p) xr[u] = qc_ld(rem + (uint32_t)(i * sizeof(double)), 0.0);
+            if (i < p) xs[i] = xr[u];
+          }
+          asm volatile("bar.arrive 1, 256;" ::: "memory");
+        } else {
+          asm volatile("bar.sync 1, 256;" ::: "memory");
+          if (work) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const int i = base + lane + 32 * u;
+              if (i < p) xr[u] = xs[i];
+            }
+          }
+        }
+      } else if (work) {
+        unsigned long long bits[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = base + lane + 32 * u;
+          bits[u] = (i >= j && i < p) ? qd_ld(src_x + i) : 0;
         }
 #pragma unroll
-        for (int u = 0; u < NB; ++u) {
-          const int i = i0 + kQdThreads * u;
-          if (i >= p) break;
-          for (int polls = 0; bits[u] == kQdEmpty && polls < kQdPolls; ++polls) bits[u] = qd_ld(ex + (long)j * p + i);
+        for (int u = 0; u < 4; ++u) {
+          const int i = base + lane + 32 * u;
+          for (int polls = 0; bits[u] == kQdEmpty && polls < kQdPolls; ++polls) bits[u] = qd_ld(src_x + i);
           if (bits[u] == kQdEmpty) s_abort = 1;
-          xs[i] = QdBits<double>::from(bits[u]);
+          xr[u] = QdBits<double>::from(bits[u]);
         }
       }
-    }
-    __syncthreads();
-    if (s_abort) {
-      if (tid == 0) atomicExch(&a.t.istat[z * a.t.nis + IS_STATUS], (int)TTM_ERR_TIMEOUT);
-      return;
-    }
-    const double inv = (warp < 4 || !(lc >= 0)) ? pre_pivot_inv(x[j], g0) : 0.0;
-    if (lc >= 0) {  // the chain: column j + 1 by one warp per sub-partition, published at once
-      if (warp < 4) {
+      if (mine || work) {
+        const double inv = pre_pivot_inv(__shfl_sync(0xffffffffu, xr[0], j & 31), g0);
+        auto update = [&](int l, bool publish) {
+          double* ac = cols + l * ld;
+          const int c = b + G * l, cu = (c - base) >> 5;
+          double xc = 0.0;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const double t = __shfl_sync(0xffffffffu, xr[u], c & 31);
+            if (u == cu) xc = t;
+          }
+          const double f = xc * inv;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int i = base + lane + 32 * u;
+            if (base + 32 * u < p && u >= cu) {
+              if (i >= c && i < p) {
+                const double y = fma(-f, xr[u], ac[i]);
+                if (!CL && publish) qd_st(ex + (long)c * p + i, QdBits<double>::to(y));
+                ac[i] = y;
+              }
+            }
+          }
+          if (CL && publish) {
+            __syncwarp();
+            qc_publish(bars, c, p, G, b, lane);
+          }
+        };
+        if (warp == 0) {
+          if (lc >= 0) update(lc, G > 1);
+        } else {
+          for (int l = l0 + warp - 1; l < nl; l += 7) update(l, false);
+        }
+        if (mine && warp == 7) {  // row j of U; zeros for a pivot that does not count
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int i = base + lane + 32 * u;
+            if (i >= j && i < p) U[i + (long)j * p] = inv != 0.0 ? xr[u] : 0.0;
+          }
+        }
+      }
+    } else {
+      if (!mine && CL) {
+        if (!qc_wait(bars, j)) s_abort = 1;
+        for (int i = base + tid; i < p; i += kQdThreads)
+          xs[i] = i >= j ? qc_ld(rem + (uint32_t)(i * sizeof(double)), 0.0) : 0.0;
+      } else if (!mine) {
+        constexpr int NB = 4;
+        for (int i0 = base + tid; i0 < p; i0 += kQdThreads * NB) {
+          unsigned long long bits[NB];
+#pragma unroll
+          for (int u = 0; u < NB; ++u) {
+            const int i = i0 + kQdThreads * u;
+            bits[u] = (i >= j && i < p) ? qd_ld(src_x + i) : 0;
+          }
+#pragma unroll
+          for (int u = 0; u < NB; ++u) {
+            const int i = i0 + kQdThreads * u;
+            if (i >= p) break;
+            for (int polls = 0; bits[u] == kQdEmpty && polls < kQdPolls; ++polls) bits[u] = qd_ld(src_x + i);
+            if (bits[u] == kQdEmpty) s_abort = 1;
+            xs[i] = QdBits<double>::from(bits[u]);
+          }
+        }
+      }
+      __syncthreads();
+      const double inv = pre_pivot_inv(x[j], g0);
+      if (lc >= 0 && warp < 4) {  // column j + 1 by one warp per sub-partition, published at once
         double* ac = cols + lc * ld;
         const double f = x[nxt] * inv;
         for (int i = base + tid; i < p; i += 128)
           if (i > j) {
             const double y = fma(-f, x[i], ac[i]);
+            if (!CL && G > 1) qd_st(ex + (long)nxt * p + i, QdBits<double>::to(y));
             ac[i] = y;
-            if (G > 1) qd_st(ex + (long)nxt * p + i, QdBits<double>::to(y));
           }
+        if (CL) {
+          asm volatile("bar.sync 2, 128;" ::: "memory");
+          if (warp == 0) qc_publish(bars, nxt, p, G, b, lane);
+        }
       }
-      __syncthreads();
-    }
-    if (mine)  // row j of U; zeros for a pivot that does not count
-      for (int i = j + tid; i < p; i += kQdThreads) U[i + (long)j * p] = pre_pivot_inv(x[j], g0) != 0.0 ? x[i] : 0.0;
-    const int l0 = lj + (b > jr ? 0 : 1);
-    if (l0 + warp < nl) {
-      const double iv = lc >= 0 ? pre_pivot_inv(x[j], g0) : inv;
+      if (mine)
+        for (int i = j + tid; i < p; i += kQdThreads) U[i + (long)j * p] = inv != 0.0 ? x[i] : 0.0;
       for (int l = l0 + warp; l < nl; l += 8) {
-        if (l == lc) continue;
         double* ac = cols + l * ld;
         const int c = b + G * l;
-        const double f = x[c] * iv;
+        const double f = x[c] * inv;
         for (int i = (c & ~31) + lane; i < p; i += 32)
           if (i >= c) ac[i] = fma(-f, x[i], ac[i]);
       }
@@ -672,7 +566,12 @@ __global__ void __launch_bounds__(kQdThreads) pre_elim_kernel(PreElimArgs a) {
     lj = nlj;
     jr = nr;
     __syncthreads();
+    if (s_abort) {
+      if (tid == 0) atomicExch(&a.t.istat[z * a.t.nis + IS_STATUS], (int)TTM_ERR_TIMEOUT);
+      break;
+    }
   }
+  if constexpr (CL) qc_sync();  // no CTA leaves while another may still read its columns
 }
 
 // X of a Newton step from M and the eliminated G (U), with the filters of ttm_newton.cuh.
@@ -700,7 +599,10 @@ __global__ void __launch_bounds__(256) pre_x_kernel(PreXArgs a) {
       x = 1.0 - 0.5 * e;
       smax = 0.5 * fabs(e);
     } else {
-      const double g = U[hi + (long)lo * p], di = U[i + (long)i * p], dj = U[j + (long)j * p];
+      // the first two steps take the couplings after elimination; from then on what the small columns
+      // carry of the large ones is at rounding level and G itself serves (no elimination)
+      const double g = a.step < 2 ? U[hi + (long)lo * p] : U[lo + (long)hi * p];
+      const double di = U[i + (long)i * p], dj = U[j + (long)j * p];
       const double dmax = fmax(di, dj);
       const int kp = bondv(a.t, z, a.ikprov);
       const double dcut = bufp(a.t, z, a.bsort)[max(0, min(kp, p) - 1)];

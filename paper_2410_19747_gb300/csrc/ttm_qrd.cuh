@@ -12,12 +12,12 @@
 // float64 instructions as possible:
 //   - column j travels as it is; whoever receives it forms x.x and x.a for its next column in one
 //     joint sum (4 warps, one per sub-partition) and derives beta, tau and v.a = x.a - beta a_j;
-//   - 1 / ||x|| and 1 / (||x|| + |x_j|) come from a float32 seed and one cubic step (12 instructions
+//   - ||x|| and 1 / (||x||^2 + |x_j| ||x||) come from a float32 seed and one cubic step (10 instructions
 //     instead of a square root and two divisions);
 //   - columns are dealt out cyclically to G CTAs and stay in shared memory; the owner of column
 //     j + 1 updates and publishes it before its other columns. Receivers poll the data itself (the
 //     exchange buffer is filled with a NaN pattern that arithmetic does not produce), so a step
-//     costs one one-way trip through L2 (about 800 clocks) and no flag or grid barrier.
+//     costs one one-way trip through L2 (about 1000 clocks) and no flag or grid barrier.
 // The other columns are updated by one warp each, four per pass when there are that many (their
 // sums share a reduce-scatter of 6 instead of 4 x 5 additions). Every wait is bounded.
 #pragma once
@@ -74,44 +74,40 @@ __device__ __forceinline__ T qd_sum4(const T (&s)[4], int lane) {
 // zero has tau = 0; a NaN travels on in beta.
 __device__ __forceinline__ void qd_scalars(double g, double alpha, double& beta, double& vj, double& tau) {
   const int hi = __double2hiint(g), lo = __double2loint(g), ex = (hi >> 20) - 1023;
-  double mu, r;
+  const bool neg = __double2hiint(alpha) < 0;
+  const double aa = __hiloint2double(__double2hiint(alpha) & 0x7fffffff, __double2loint(alpha));
+  double mu, D;
   if (ex > -900 && ex < 900) {  // (a negative or NaN g is outside)
     const int h = ex >> 1;
     const int gh = hi - ((2 * h) << 20);  // g 2^(-2h) in [1, 4)
     const double gs = __hiloint2double(gh, lo);
     const unsigned s = __float_as_uint(rsqrtf(__uint_as_float(((unsigned)(gh - 0x38000000) << 3) | ((unsigned)lo >> 29))));
     const double r0 = __hiloint2double((int)(s >> 3) + 0x38000000, (int)(s << 29));
-    const double e = fma(-(gs * r0), r0, 1.0);
-    const double rs = fma(r0 * e, fma(e, 0.375, 0.5), r0);
-    const double ms = gs * rs;
-    r = __hiloint2double(__double2hiint(rs) - (h << 20), __double2loint(rs));
+    const double m0 = gs * r0;                       // sqrt to float32 accuracy, then one cubic step
+    const double e = fma(-m0, r0, 1.0);
+    const double ms = fma(m0 * e, fma(e, 0.375, 0.5), m0);
     mu = __hiloint2double(__double2hiint(ms) + (h << 20), __double2loint(ms));
+    D = fma(aa, mu, g);                              // mu (mu + |alpha|) = v^T v / 2, in [g, 2 g (1 + u)]
+    const int dh = __double2hiint(D), dl = __double2loint(D), de = (dh >> 20) - 1023;
+    const int sh = dh - (de << 20);
+    const unsigned t =
+        __float_as_uint(__fdividef(1.f, __uint_as_float(((unsigned)(sh - 0x38000000) << 3) | ((unsigned)dl >> 29))));
+    const double q0 = __hiloint2double((int)(t >> 3) + 0x38000000, (int)(t << 29));
+    const double f = fma(-__hiloint2double(sh, dl), q0, 1.0);
+    const double q = fma(q0 * f, 1.0 + f, q0);
+    tau = __hiloint2double(__double2hiint(q) - (de << 20), __double2loint(q));
   } else if (g >= 2.3e-308) {
     mu = sqrt(g);
-    r = 1.0 / mu;
+    tau = 1.0 / fma(aa, mu, g);
   } else {  // zero (or its square is below the normal range, where tau would overflow), or a NaN
     beta = g == g ? alpha : g;
     vj = 0.0;
     tau = 0.0;
     return;
   }
-  const double y = fabs(alpha) + mu;
-  const int yh = __double2hiint(y), yl = __double2loint(y), ye = (yh >> 20) - 1023;
-  double q;
-  if (ye > -900 && ye < 900) {
-    const int sh = yh - (ye << 20);  // y 2^-ye in [1, 2)
-    const unsigned s =
-        __float_as_uint(__fdividef(1.f, __uint_as_float(((unsigned)(sh - 0x38000000) << 3) | ((unsigned)yl >> 29))));
-    const double q0 = __hiloint2double((int)(s >> 3) + 0x38000000, (int)(s << 29));
-    const double e = fma(-__hiloint2double(sh, yl), q0, 1.0);
-    const double qs = fma(q0 * e, 1.0 + e, q0);
-    q = __hiloint2double(__double2hiint(qs) - (ye << 20), __double2loint(qs));
-  } else {
-    q = 1.0 / y;
-  }
-  tau = r * q;
-  beta = alpha <= 0.0 ? mu : -mu;
-  vj = alpha <= 0.0 ? -y : y;
+  beta = neg ? mu : -mu;
+  const double y = aa + mu;
+  vj = neg ? -y : y;
 }
 __device__ __forceinline__ void qd_scalars(float g, float alpha, float& beta, float& vj, float& tau) {
   if (g > 1e-36f) {  // below (columns of 1e-18 of max |A|) tau would leave the float range
@@ -157,7 +153,7 @@ __device__ __forceinline__ void qd_st(unsigned long long* p, unsigned long long 
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kQdThreads) qrd_kernel(QrdArgs a) {
+__global__ void __launch_bounds__(kQdThreads, 3) qrd_kernel(QrdArgs a) {
   extern __shared__ __align__(16) unsigned char qd_raw[];
   const int G = a.G, z = blockIdx.x / G, b = blockIdx.x % G;
   const int M = a.m.eval(a.t, z), N = a.n.eval(a.t, z), k = min(M, N);
@@ -165,8 +161,8 @@ __global__ void __launch_bounds__(kQdThreads) qrd_kernel(QrdArgs a) {
   const int ld = a.ld_ub;
   T* cols = reinterpret_cast<T*>(qd_raw);          // [cols_ub][ld]
   T* xs = cols + (long)a.cols_ub * ld;              // [ld] the column received
-  __shared__ T red[2][8];
-  __shared__ T s_sc[3];                             // beta, v_j, tau of the current step
+  __shared__ T red[8];
+  __shared__ T s_sc[4];                             // beta, v_j, tau, the chain column's factor
   __shared__ int s_abort;
   if (b == 0 && tid == 0 && a.ik >= 0) a.t.bond[z * a.t.nbd + a.ik] = k;
   for (long e = (long)b * kQdThreads + tid; e < a.clear_n; e += (long)G * kQdThreads)
@@ -200,6 +196,9 @@ __global__ void __launch_bounds__(kQdThreads) qrd_kernel(QrdArgs a) {
   if (G > 1 && b == 0)
     for (int i = tid; i < M; i += kQdThreads) qd_st(ex + i, QdBits<T>::to(cols[i]));
 
+  // The order in which warps take columns: warp 0 computes the scalars, so it and the warp that
+  // shares its sub-partition come last.
+  const int rank = warp == 0 ? 7 : warp < 4 ? warp - 1 : warp == 4 ? 6 : warp - 2;
   int lj = 0, jr = 0;  // j / G and j % G
   for (int j = 0; j < k; ++j) {
     if (b + G * (nl - 1) < j) break;  // no column from j on is held here
@@ -210,138 +209,232 @@ __global__ void __launch_bounds__(kQdThreads) qrd_kernel(QrdArgs a) {
     const T* x = mine ? cols + lj * ld : xs;
     const int base = j & ~31;
     T* crit = lc >= 0 ? cols + lc * ld : nullptr;
-    if (warp < 4) {
-      T p0 = T(0), p1 = T(0);
+    const unsigned long long* src_x = ex + (long)j * M;
+    unsigned long long* dst_x = ex + (long)nxt * M;
+    // the other columns right of j: local index from l0 on; up to eight are one per warp, whose dot
+    // product with x is formed while warp 0 is at the scalars
+    const int l0 = lc >= 0 ? lc + 1 : lj + (b > jr ? 0 : 1);
+    const int rest = nl - l0;
+    const bool one = rest <= 8, have = one && rank < rest;
+    T* am = have ? cols + (l0 + rank) * ld : nullptr;
+    T dme = T(0);
+    const bool narrow = M - base <= 128;  // warp 0 takes the chain alone, x in the registers of every warp
+    T xr[4] = {T(0), T(0), T(0), T(0)};
+    if (narrow) {
       if (mine) {
-        for (int i = base + tid; i < M; i += 128) {
-          const T xi = i >= j ? x[i] : T(0);
-          p0 = fma(xi, xi, p0);
-          if (crit) p1 = fma(xi, crit[i], p1);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = base + lane + 32 * u;
+          if (i >= j && i < M) xr[u] = x[i];
         }
-      } else {
-        // all of this thread's rows are requested before any is waited for
-        const unsigned long long* src_x = ex + (long)j * M;
-        constexpr int NB = 8;
-        for (int i0 = base + tid; i0 < M; i0 += 128 * NB) {
-          unsigned long long bits[NB];
+      } else if (warp == 0 || have) {
+        unsigned long long bits[4];
 #pragma unroll
-          for (int u = 0; u < NB; ++u) {
-            const int i = i0 + 128 * u;
-            bits[u] = (i >= j && i < M) ? qd_ld(src_x + i) : 0;
+        for (int u = 0; u < 4; ++u) {
+          const int i = base + lane + 32 * u;
+          bits[u] = (i >= j && i < M) ? qd_ld(src_x + i) : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = base + lane + 32 * u;
+          for (int polls = 0; bits[u] == kQdEmpty && polls < kQdPolls; ++polls) bits[u] = qd_ld(src_x + i);
+          if (bits[u] == kQdEmpty) s_abort = 1;
+          xr[u] = QdBits<T>::from(bits[u]);
+          if (!one && i < M) xs[i] = xr[u];  // (warp 0)
+        }
+      }
+      if (warp == 0) {
+        T p0 = T(0), p1 = T(0), cr[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = base + lane + 32 * u;
+          cr[u] = (crit && i < M) ? crit[i] : T(0);
+          if (base + 32 * u < M) {
+            p0 = fma(xr[u], xr[u], p0);
+            if (crit) p1 = fma(xr[u], cr[u], p1);
           }
+        }
+        const bool hi = lane & 16;
+        T s = hi ? p1 : p0;
+        s += __shfl_xor_sync(0xffffffffu, hi ? p0 : p1, 16);
 #pragma unroll
-          for (int u = 0; u < NB; ++u) {
-            const int i = i0 + 128 * u;
-            if (i >= M) break;
-            for (int polls = 0; bits[u] == kQdEmpty && polls < kQdPolls; ++polls) bits[u] = qd_ld(src_x + i);
-            if (bits[u] == kQdEmpty) s_abort = 1;
-            const T xi = QdBits<T>::from(bits[u]);
-            xs[i] = xi;
+        for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        const T g = __shfl_sync(0xffffffffu, s, 0), d = __shfl_sync(0xffffffffu, s, 16);
+        T beta, vj, tau;
+        qd_scalars(g, __shfl_sync(0xffffffffu, xr[0], j & 31), beta, vj, tau);
+        if (crit) {
+          const T cj = __shfl_sync(0xffffffffu, cr[0], j & 31);
+          const T f = tau * fma(-beta, cj, d);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int i = base + lane + 32 * u;
+            if (base + 32 * u < M) {
+              const T y = fma(-f, xr[u], cr[u]);
+              if (i > j && i < M) {
+                if (G > 1 && nxt < k) qd_st(dst_x + i, QdBits<T>::to(y));
+                crit[i] = y;
+              }
+            }
+          }
+          if (lane == 0) R[(long)j * N + nxt] = fma(-f, vj, cj);
+        }
+        if (lane == 0) {
+          s_sc[0] = beta;
+          s_sc[1] = vj;
+          s_sc[2] = tau;
+        }
+      } else if (have) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (base + 32 * u < M) {
+            const int i = base + lane + 32 * u;
+            if (i < M) dme = fma(xr[u], am[i], dme);
+          }
+        dme = qd_sum(dme);
+      }
+    } else {
+      if (warp < 4) {
+        T p0 = T(0), p1 = T(0);
+        if (mine) {
+          for (int i = base + tid; i < M; i += 128) {
+            const T xi = i >= j ? x[i] : T(0);
             p0 = fma(xi, xi, p0);
             if (crit) p1 = fma(xi, crit[i], p1);
           }
-        }
-      }
-      const bool hi = lane & 16;
-      T s = hi ? p1 : p0;
-      s += __shfl_xor_sync(0xffffffffu, hi ? p0 : p1, 16);
+        } else {
+          // all of this thread's rows are requested before any is waited for
+          constexpr int NB = 8;
+          for (int i0 = base + tid; i0 < M; i0 += 128 * NB) {
+            unsigned long long bits[NB];
 #pragma unroll
-      for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if ((lane & 15) == 0) red[j & 1][warp + (hi ? 4 : 0)] = s;
+            for (int u = 0; u < NB; ++u) {
+              const int i = i0 + 128 * u;
+              bits[u] = (i >= j && i < M) ? qd_ld(src_x + i) : 0;
+            }
+#pragma unroll
+            for (int u = 0; u < NB; ++u) {
+              const int i = i0 + 128 * u;
+              if (i >= M) break;
+              for (int polls = 0; bits[u] == kQdEmpty && polls < kQdPolls; ++polls) bits[u] = qd_ld(src_x + i);
+              if (bits[u] == kQdEmpty) s_abort = 1;
+              const T xi = QdBits<T>::from(bits[u]);
+              xs[i] = xi;
+              p0 = fma(xi, xi, p0);
+              if (crit) p1 = fma(xi, crit[i], p1);
+            }
+          }
+        }
+        const bool hi = lane & 16;
+        T s = hi ? p1 : p0;
+        s += __shfl_xor_sync(0xffffffffu, hi ? p0 : p1, 16);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if ((lane & 15) == 0) red[warp + (hi ? 4 : 0)] = s;
+      }
+      __syncthreads();
+      if (warp == 0) {
+        T s = red[lane & 7];
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        const T g = __shfl_sync(0xffffffffu, s, 0), d = __shfl_sync(0xffffffffu, s, 4);
+        T beta, vj, tau;
+        qd_scalars(g, x[j], beta, vj, tau);
+        const T cj = crit ? crit[j] : T(0);
+        const T f = tau * fma(-beta, cj, d);
+        if (lane == 0) {
+          s_sc[0] = beta;
+          s_sc[1] = vj;
+          s_sc[2] = tau;
+          s_sc[3] = f;
+          if (crit) R[(long)j * N + nxt] = fma(-f, vj, cj);
+        }
+      } else if (have) {
+        for (int i = base + lane; i < M; i += 32) dme = fma(i >= j ? x[i] : T(0), am[i], dme);
+        dme = qd_sum(dme);
+      }
     }
     __syncthreads();
     if (s_abort) {  // every thread sees it: it was set before the barrier
       if (tid == 0) atomicExch(&a.t.istat[z * a.t.nis + IS_STATUS], (int)TTM_ERR_TIMEOUT);
       return;
     }
-    if (warp < 4) {
-      T s = red[j & 1][lane & 7];
-      s += __shfl_xor_sync(0xffffffffu, s, 1);
-      s += __shfl_xor_sync(0xffffffffu, s, 2);
-      const T g = __shfl_sync(0xffffffffu, s, 0), d = __shfl_sync(0xffffffffu, s, 4);
-      T beta, vj, tau;
-      qd_scalars(g, x[j], beta, vj, tau);
-      if (crit) {
-        const T cj = crit[j];
-        const T f = tau * fma(-beta, cj, d);
-        unsigned long long* dst = ex + (long)nxt * M;
-        for (int i = base + tid; i < M; i += 128) {
-          if (i > j) {
-            const T y = fma(-f, x[i], crit[i]);
-            crit[i] = y;
-            if (G > 1 && nxt < k) qd_st(dst + i, QdBits<T>::to(y));
-          }
+    if (!narrow && crit && warp < 4) {
+      const T f = s_sc[3];
+      for (int i = base + tid; i < M; i += 128)
+        if (i > j) {
+          const T y = fma(-f, x[i], crit[i]);
+          if (G > 1 && nxt < k) qd_st(dst_x + i, QdBits<T>::to(y));
+          crit[i] = y;
         }
-        __syncwarp();
-        if (tid == 0) R[(long)j * N + nxt] = fma(-f, vj, cj);
-      }
-      if (tid == 0) {
-        s_sc[0] = beta;
-        s_sc[1] = vj;
-        s_sc[2] = tau;
-        if (mine) {
-          T rd = beta;
-          if constexpr (sizeof(T) == 4) rd += rd < T(0) ? -a.ridge : a.ridge;
-          R[(long)j * N + j] = rd;
-          if (V) {
-            V[(long)j * M + j] = (double)vj;
-            taug[j] = (double)tau;
-          }
-        }
+    }
+    if (mine && tid == 0) {
+      T rd = s_sc[0];
+      if constexpr (sizeof(T) == 4) rd += rd < T(0) ? -a.ridge : a.ridge;
+      R[(long)j * N + j] = rd;
+      if (V) {
+        V[(long)j * M + j] = (double)s_sc[1];
+        taug[j] = (double)s_sc[2];
       }
     }
-    __syncthreads();
-    // the other columns right of j: local index from l0 on, one warp per column
-    int l0 = lj + (b > jr ? 0 : 1);
-    if (l0 == lc) ++l0;
-    const int rest = nl - l0;
-    if (rest > 0) {
+    if (have) {
+      const T beta = s_sc[0], vj = s_sc[1], tau = s_sc[2];
+      if (warp == 0) {  // (its dot product had to wait)
+        if (narrow) {
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int i = base + lane + 32 * u;
+            if (i < M) dme = fma(xr[u], am[i], dme);
+          }
+        } else {
+          for (int i = base + lane; i < M; i += 32) dme = fma(i >= j ? x[i] : T(0), am[i], dme);
+        }
+        dme = qd_sum(dme);
+      }
+      const T cj = am[j];
+      const T f = tau * fma(-beta, cj, dme);
+      if (lane == 0) R[(long)j * N + b + (long)G * (l0 + rank)] = fma(-f, vj, cj);
+      if (narrow) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = base + lane + 32 * u;
+          if (base + 32 * u < M && i > j && i < M) am[i] = fma(-f, xr[u], am[i]);
+        }
+      } else {
+        for (int i = base + lane; i < M; i += 32)
+          if (i > j) am[i] = fma(-f, x[i], am[i]);
+      }
+    } else if (!one) {
       const T beta = s_sc[0], vj = s_sc[1], tau = s_sc[2];
       for (int q0 = 0; q0 < rest; q0 += 32) {
+        // up to four columns of this warp: l0 + q0 + warp + 8 q
         const int cnt = min(32, rest - q0);
-        if (cnt > 8) {
-          // up to four columns of this warp: l0 + q0 + warp + 8 q
-          const int lw = l0 + q0 + warp;
-          T s[4] = {T(0), T(0), T(0), T(0)};
-          T* ac[4];
+        const int lw = l0 + q0 + warp;
+        T s[4] = {T(0), T(0), T(0), T(0)};
+        T* ac[4];
 #pragma unroll
-          for (int q = 0; q < 4; ++q) ac[q] = cols + min(lw + 8 * q, nl - 1) * ld;
-          for (int i = base + lane; i < M; i += 32) {
-            const T xi = i >= j ? x[i] : T(0);
+        for (int q = 0; q < 4; ++q) ac[q] = cols + min(lw + 8 * q, nl - 1) * ld;
+        for (int i = base + lane; i < M; i += 32) {
+          const T xi = i >= j ? x[i] : T(0);
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (warp + 8 * q < cnt) s[q] = fma(xi, ac[q][i], s[q]);
+        }
+        const int mq = lane >> 3;
+        const T dsum = qd_sum4(s, lane);
+        const T cj = cols[min(lw + 8 * mq, nl - 1) * ld + j];
+        const T f = tau * fma(-beta, cj, dsum);
+        T fq[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) fq[q] = __shfl_sync(0xffffffffu, f, 8 * q);
+        if ((lane & 7) == 0 && warp + 8 * mq < cnt)
+          R[(long)j * N + b + (long)G * (lw + 8 * mq)] = fma(-f, vj, cj);
+        for (int i = base + lane; i < M; i += 32) {
+          const T xi = x[i];
+          if (i > j) {
 #pragma unroll
             for (int q = 0; q < 4; ++q)
-              if (warp + 8 * q < cnt) s[q] = fma(xi, ac[q][i], s[q]);
+              if (warp + 8 * q < cnt) ac[q][i] = fma(-fq[q], xi, ac[q][i]);
           }
-          const int mq = lane >> 3;
-          const T dsum = qd_sum4(s, lane);
-          const T cj = cols[min(lw + 8 * mq, nl - 1) * ld + j];
-          const T f = tau * fma(-beta, cj, dsum);
-          T fq[4];
-#pragma unroll
-          for (int q = 0; q < 4; ++q) fq[q] = __shfl_sync(0xffffffffu, f, 8 * q);
-          if ((lane & 7) == 0 && warp + 8 * mq < cnt)
-            R[(long)j * N + b + (long)G * (lw + 8 * mq)] = fma(-f, vj, cj);
-          for (int i = base + lane; i < M; i += 32) {
-            const T xi = x[i];
-            if (i > j) {
-#pragma unroll
-              for (int q = 0; q < 4; ++q)
-                if (warp + 8 * q < cnt) ac[q][i] = fma(-fq[q], xi, ac[q][i]);
-            }
-          }
-        } else if (warp < cnt) {
-          T* ac = cols + (l0 + q0 + warp) * ld;
-          T s = T(0);
-          for (int i = base + lane; i < M; i += 32) {
-            const T xi = i >= j ? x[i] : T(0);
-            s = fma(xi, ac[i], s);
-          }
-          s = qd_sum(s);
-          const T cj = ac[j];
-          const T f = tau * fma(-beta, cj, s);
-          if (lane == 0) R[(long)j * N + b + (long)G * (l0 + q0 + warp)] = fma(-f, vj, cj);
-          for (int i = base + lane; i < M; i += 32)
-            if (i > j) ac[i] = fma(-f, x[i], ac[i]);
         }
       }
     }
@@ -390,28 +483,35 @@ struct QrdApplyArgs {
   int ld_ub;
 };
 
+// WPC: warps per column (1: four columns per CTA; 4: one, for launches with fewer columns than the
+// chip has sub-partitions). On 256 rows a step takes about 1400 clocks with one warp, 900 with four.
+template <int WPC>
 __global__ void __launch_bounds__(kQaThreads) qrd_apply_kernel(QrdApplyArgs a) {
   extern __shared__ __align__(16) unsigned char qd_raw[];
+  constexpr int CPB = 4 / WPC;  // columns per CTA
+  __shared__ double red[2][4];
   const int z = blockIdx.y;
   const int M = a.m.eval(a.t, z), N = a.n.eval(a.t, z), k = min(M, N), nc = bondv(a.t, z, a.ic);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int c0 = blockIdx.x * 4, c = c0 + warp;
+  const int c0 = blockIdx.x * CPB, c = WPC == 1 ? c0 + warp : c0;
+  const int r0 = WPC == 1 ? lane : threadIdx.x;  // this thread's first row above the step's base
+  constexpr int RS = 32 * WPC;                   // and its row stride
   if (c0 >= nc) return;
   const int ld = a.ld_ub;
-  double* vs = reinterpret_cast<double*>(qd_raw);     // [kQaStages][ld]
-  double* y = vs + (kQaStages + warp) * (long)ld;      // this warp's column
+  double* vs = reinterpret_cast<double*>(qd_raw);                              // [kQaStages][ld]
+  double* y = vs + (kQaStages + (WPC == 1 ? warp : 0)) * (long)ld;              // this warp's column
   const double* V = bufp(a.t, z, a.bv);
   const double* tau = bufp(a.t, z, a.btau);
   const bool on = c < nc;
   int j0;
   if (a.bvec < 0) {
-    j0 = min(min(c0 + 3, nc - 1), k - 1);
-    for (int i = lane; i < M; i += 32) y[i] = i == c ? 1.0 : 0.0;
+    j0 = min(min(c0 + CPB - 1, nc - 1), k - 1);
+    for (int i = r0; i < M; i += RS) y[i] = i == c ? 1.0 : 0.0;
   } else {
     j0 = k - 1;
     const int pc = on ? reinterpret_cast<const int*>(bufp(a.t, z, a.bperm))[c] : 0;
     const double* x = bufp(a.t, z, pre_where(a.t, z) ? a.bvec2 : a.bvec) + (long)max(0, min(pc, k - 1)) * k;
-    for (int i = lane; i < M; i += 32) y[i] = i < k ? x[i] : 0.0;
+    for (int i = r0; i < M; i += RS) y[i] = i < k ? x[i] : 0.0;
   }
   auto fetch = [&](int q) {  // reflector q into its stage; one commit group per call
     if (q >= 0) {
@@ -433,20 +533,27 @@ __global__ void __launch_bounds__(kQaThreads) qrd_apply_kernel(QrdApplyArgs a) {
     fetch(j - (kQaStages - 1));
     const double* v = vs + (j & (kQaStages - 1)) * (long)ld;
     double s = 0.0;
-    for (int i = (j & ~31) + lane; i < M; i += 32)
+    for (int i = (j & ~31) + r0; i < M; i += RS)
       if (i >= j) s = fma(v[i], y[i], s);
-    const double f = tj * qd_sum(s);
-    for (int i = (j & ~31) + lane; i < M; i += 32)
+    s = qd_sum(s);
+    if constexpr (WPC == 4) {
+      if (lane == 0) red[j & 1][warp] = s;
+      __syncthreads();
+      s = (red[j & 1][0] + red[j & 1][1]) + (red[j & 1][2] + red[j & 1][3]);
+    }
+    const double f = tj * s;
+    for (int i = (j & ~31) + r0; i < M; i += RS)
       if (i >= j) y[i] = fma(-f, v[i], y[i]);
-    __syncwarp();
+    if constexpr (WPC == 1) __syncwarp();
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
+  if constexpr (WPC == 4) __syncthreads();
   if (!on) return;
   double* out = bufp(a.t, z, a.bout);
   if (a.out_rows)
-    for (int i = lane; i < M; i += 32) out[(long)i * nc + c] = y[i];
+    for (int i = r0; i < M; i += RS) out[(long)i * nc + c] = y[i];
   else
-    for (int i = lane; i < M; i += 32) out[(long)c * M + i] = y[i];
+    for (int i = r0; i < M; i += RS) out[(long)c * M + i] = y[i];
 }
 
 }  // namespace ttm

@@ -70,6 +70,22 @@ def test_a_small_eps_keeps_the_product(h, L, d, ca, cb):
     assert relerr(O, ott.dense(A) * ott.dense(B)) <= 1e-12
 
 
+@pytest.mark.parametrize("L,d,ca,cb,cap", [(5, 2, 3, 4, 0), (4, 6, 5, 7, 0), (4, 3, 4, 4, 27), (3, 33, 20, 33, 0), (5, 2, 4, 4, 7)])
+def test_nothing_truncated(h, L, d, ca, cb, cap):
+    """eps = 0 without a binding cap takes no SVD: bonds min(m, n) as the oracle's, a right-canonical
+    result whose centre carries the norm, nothing discarded. (The last cap binds on some Swaps.)"""
+    A, B = ttgen.rand_tt(L, d, ca, 31), ttgen.rand_tt(L, d, cb, 32)
+    P = ott.dense(A) * ott.dense(B)
+    O, rep = multiply(h, A, B, chi_max=cap)
+    Oo, ro = ottm.ttm(A, B, chi_max=cap)
+    assert ott.bonds_of(O) == ott.bonds_of(Oo)
+    assert relerr(O, P) <= relerr(Oo, P) + 1e-12
+    assert abs(rep["norm_out"] - np.linalg.norm(ott.dense(O))) <= 1e-12 * rep["norm_out"]
+    for c in O[1:]:
+        q = c.reshape(c.shape[0], -1)
+        assert np.abs(q @ q.T - np.eye(c.shape[0])).max() <= 1e-12
+
+
 def test_rank_deficient_trains(h):
     """Bonds that carry a few directions only: most singular values are zero to rounding."""
     rng = np.random.default_rng(5)

@@ -55,7 +55,7 @@ typedef enum {
 /* Arithmetic of the GEMM-shaped work: the contractions (Theta of every Swap, Contract, the
  * R merge of every gauge move) and the GEMMs inside the Swap SVD (its Newton steps). The
  * Householder QR, the Jacobi rotations, norms and the truncation rule always run on the
- * CUDA cores (float32 Jacobi passes, everything else float64). */
+ * CUDA cores (the Jacobi in float32, everything else but its preconditioning QR in float64). */
 typedef enum {
   TTM_PREC_FP64 = 0,       /* every GEMM on the float64 pipe (the reference form)         */
   TTM_PREC_BF16_SPLIT = 2  /* GEMMs on the tcgen05 tensor cores as the exactly sliced
@@ -97,7 +97,8 @@ typedef struct {
                                device)                                                    */
   int32_t max_sweeps;       /* sweep limit of the float32 Jacobi passes after the first
                                and of the float64 Jacobi of the Newton fallback; 0 = 20
-                               and 40                                                     */
+                               and 40 (the preconditioned Swap, see f32_passes: 30 and
+                               40). Not 0: every Swap takes the general pipeline         */
   int32_t use_graph;        /* 1: ttm_multiply / ttm_multiply_batched capture the kernel
                                sequence of a plan (options, shapes, input bonds, arena) into
                                a CUDA graph on first use and replay it while the plan stays
@@ -107,8 +108,14 @@ typedef struct {
   int32_t profile_kernels;  /* 1: time every GEMM, float32 Jacobi and Householder launch
                                with CUDA events on the handle's stream (fills gemm_ms,
                                jacobi32_ms, jacobi64_ms and qr_ms of the report)          */
-  int32_t f32_passes;       /* float32 one-sided Jacobi passes of every Swap SVD: 0 = 3
-                               (the first stops after 3 sweeps), 1..8 accepted           */
+  int32_t f32_passes;       /* float32 one-sided Jacobi passes of every Swap SVD, 1..8; the
+                               first stops after 3 sweeps. 0, with max_sweeps,
+                               jacobi_kernel and newton_steps 0 as well: two QR
+                               factorisations and one Jacobi of the triangle (ttm_pre.cuh),
+                               or no SVD where eps and the caps drop nothing; what that
+                               does not cover (more than 1024 rows, no room for its
+                               buffers), and 0 beside another option that is not 0: the
+                               general pipeline with 3 passes                            */
   int32_t jacobi_kernel;    /* kernel of the float32 passes: 0 = 3 when the Swap matrix
                                has at most 1024 rows, else 1; 1 = one column per
                                tournament slot (n - 1 grid barriers per sweep); 2 = two
@@ -119,7 +126,8 @@ typedef struct {
                                columns                                                   */
   int32_t newton_steps;     /* float64 Newton steps that finish every Swap SVD after the
                                float32 passes: 0 = 3, 1..8 accepted; an SVD whose last
-                               correction is still above 1e-7 takes up to 2 more          */
+                               correction is still above 1e-7 takes up to 2 more. The
+                               preconditioned Swap takes 2, and up to 2 more above 1e-9   */
   int32_t split_digits;     /* digits per operand of TTM_PREC_BF16_SPLIT: 0 = 8, 2..8   */
   int32_t reserved1;        /* must be 0                                                 */
   int64_t env_budget_bytes; /* ttm_backward: device memory for the stored left

@@ -958,7 +958,8 @@ static int query_max_cluster() {
     int smem;
   };
   const Probe probes[] = {
-      {(void*)pre_elim_kernel<true>, kQdThreads, (kElimClusterMax / kElimCluster + 1) * kElimClusterMax * 8},
+      {(void*)pre_elim_kernel<true>, kQdThreads,
+       (kElimClusterMax / (kElimCluster * kElB) + 1) * kElB * kElimClusterMax * 8},
       {jacobi_pre_fn(16), kPjThreads, 2 * kPjB * 512 * 4}};
   for (const Probe& p : probes) {
     TTM_CUDA(cudaFuncSetAttribute(p.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem));

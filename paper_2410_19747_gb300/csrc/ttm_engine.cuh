@@ -418,8 +418,9 @@ class Engine {
     if (base_only_ || opt_.f32_passes || opt_.jacobi_kernel || opt_.newton_steps || opt_.max_sweeps) return false;
     const int p_ub = std::min(m_ub, n_ub);
     size_t sm = 0;
+    bool cluster = false;
     return m_ub <= kPreMax && qrd_apply_fits(n_ub) && qrd_ctas(n_ub, m_ub, 8, &sm) > 0 &&
-           qrd_ctas(m_ub, p_ub, 4, &sm) > 0 && qrd_ctas(p_ub, p_ub, 8, &sm) > 0;
+           qrd_ctas(m_ub, p_ub, 4, &sm) > 0 && elim_ctas(p_ub, &cluster, &sm) > 0;
   }
   // The exchange buffers of a distributed launch that uses `extent` elements per product.
   template <class A>
@@ -431,35 +432,50 @@ class Engine {
     ex_prev_ = extent;
     ex_flip_ ^= 1;
   }
+  // CTAs of the elimination. cluster: they form one, with a CTA per two blocks of kElB columns up to
+  // the largest cluster (one or four blocks each take the same time within 1 %, with more products of a
+  // batch in turn for one). Else one per block as far as the SMs reach (as qrd_ctas).
+  int elim_ctas(int p_ub, bool* cluster, size_t* smem) const {
+    const int nb = (p_ub + kElB - 1) / kElB;
+    auto need = [&](int G) { return (size_t)((nb + G - 1) / G + 1) * kElB * p_ub * 8; };
+    *cluster = false;
+    if (p_ub <= kElimClusterMax) {
+      int G = 1;
+      while (G < hs_.max_cluster && G * 2 < nb) G *= 2;
+      *smem = need(G);
+      if (*smem <= (size_t)kElimSmem) {
+        *cluster = true;
+        return G;
+      }
+    }
+    for (int G = nb;; G = (G + 1) / 2) {
+      *smem = need(G);
+      if (*smem > (size_t)kElimSmem) return 0;
+      const long occ = std::max<long>(1, std::min<long>(3, (long)(220 * 1024 / (*smem + 1024))));
+      if ((long)Z_ * G <= occ * std::max(1, hs_.num_sms) || G == 1) return G;
+    }
+  }
   void pre_elim(PreElimArgs a, int p_ub) {
     size_t smem = 0;
-    const int G = qrd_ctas(p_ub, p_ub, 8, &smem);
-    int Gc = 0;
-    if (p_ub <= kElimClusterMax)
-      for (Gc = 1; Gc < hs_.max_cluster && Gc * 4 < p_ub;) Gc *= 2;
-    const size_t smem_c = Gc > 0 ? (size_t)((p_ub + Gc - 1) / Gc + 1) * p_ub * 8 : 0;
-    if (smem_c > (size_t)kQdSmem) Gc = 0;
+    bool cluster = false;
+    const int G = elim_ctas(p_ub, &cluster, &smem);
     if (!launch_) {
-      if (G > 1 && Gc == 0) ex_elems_ = std::max(ex_elems_, (long)p_ub * p_ub);
+      if (G > 1 && !cluster) ex_elems_ = std::max(ex_elems_, (long)p_ub * p_ub);
       return;
     }
-    a.G = Gc > 0 ? Gc : G;
-    a.cols_ub = (p_ub + a.G - 1) / a.G;
+    a.G = G;
+    a.blocks_ub = ((p_ub + kElB - 1) / kElB + G - 1) / G;
     a.ld_ub = p_ub;
     void* kargs[] = {&a};
-    if (Gc > 0) {
-      void* fn = (void*)pre_elim_kernel<true>;
-      TTM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_c));
-      launch_cluster(fn, Z_, Gc, kQdThreads, smem_c, kargs, hs_.stream);
+    void* fn = cluster ? (void*)pre_elim_kernel<true> : (void*)pre_elim_kernel<false>;
+    TTM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (cluster) {
+      launch_cluster(fn, Z_, G, kQdThreads, smem, kargs, hs_.stream);
+    } else if (G > 1) {
+      use_exchange(a, (long)p_ub * p_ub);
+      TTM_CUDA(cudaLaunchCooperativeKernel(fn, dim3((unsigned)(Z_ * G)), dim3(kQdThreads), kargs, smem, hs_.stream));
     } else {
-      void* fn = (void*)pre_elim_kernel<false>;
-      TTM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      if (G > 1) {
-        use_exchange(a, (long)p_ub * p_ub);
-        TTM_CUDA(cudaLaunchCooperativeKernel(fn, dim3((unsigned)(Z_ * G)), dim3(kQdThreads), kargs, smem, hs_.stream));
-      } else {
-        TTM_CUDA(cudaLaunchKernel(fn, dim3((unsigned)Z_), dim3(kQdThreads), kargs, smem, hs_.stream));
-      }
+      TTM_CUDA(cudaLaunchKernel(fn, dim3((unsigned)Z_), dim3(kQdThreads), kargs, smem, hs_.stream));
     }
     ++launches_;
   }

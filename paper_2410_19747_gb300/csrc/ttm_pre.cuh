@@ -301,10 +301,10 @@ __global__ void pre_v_kernel(PreVArgs a) {
 }
 
 // ---------------------------------------------------------------- transport inside a cluster
-// A cluster of G CTAs hands a column on through distributed shared memory: it stays where its owner
-// holds it, the owner's release-arrival on one mbarrier per receiver says that it is final, and the
-// receivers read it there. Slot of column c: c mod 32 (a multiple of G, so that the CTAs that use a
-// slot are the same on every turn, and the chain cannot run 32 columns ahead of a CTA, since every
+// A cluster of G CTAs hands a block of columns on through distributed shared memory: it stays where its
+// owner holds it, the owner's release-arrival on one mbarrier per receiver says that it is final, and
+// the receivers read it there. Slot of block c: c mod 32 (a multiple of G, so that the CTAs that use
+// a slot are the same on every turn, and the chain cannot run 32 blocks ahead of a CTA, since every
 // CTA owns one in G); phase: c / 32.
 constexpr int kQdSlots = 32;
 constexpr int kElimCluster = 16;      // largest cluster of the elimination
@@ -322,8 +322,8 @@ __device__ __forceinline__ void qc_init(uint64_t* bars, int tid) {
 __device__ __forceinline__ void qc_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// Column c is final in this CTA (its writers have been joined with the calling warp): tells the CTAs
-// that hold a column from c on. nc: columns of the matrix.
+// Block c is final in this CTA (its writers have been joined with the calling warp): tells the CTAs
+// that hold a block from c on. nc: blocks of the matrix.
 __device__ __forceinline__ void qc_publish(uint64_t* bars, int c, int nc, int G, int b, int lane) {
   if (lane < G && lane != b) {
     const int last = lane < nc ? lane + (nc - 1 - lane) / G * G : -1;
@@ -354,14 +354,14 @@ __device__ __forceinline__ double qc_ld(uint32_t addr, double) {
 // ---------------------------------------------------------------- elimination of G
 // U of G = L_G U without pivoting (the columns come in descending order): U_ij for i <= j, stored
 // at [j + i p]. A pivot that cancelled to rounding level counts as zero and eliminates nothing.
-// Distributed like the QR (columns dealt out to G CTAs, column j polled from the exchange buffer);
-// a step is one reciprocal and one update, no reduction.
+// Distributed like the QR: blocks of columns are dealt out to G CTAs and handed on through the
+// cluster's shared memory, or past kElimClusterMax through the polled exchange buffer.
 struct PreElimArgs {
   Tables t;
   int bg, bu;
   Dim p;
   int step;
-  int G, cols_ub, ld_ub;
+  int G, blocks_ub, ld_ub;
   unsigned long long* ex;
   unsigned long long* ex_next;
   long ex_stride, clear_n;
@@ -382,6 +382,16 @@ __device__ __forceinline__ double pre_pivot_inv(double d, double g0) {
   return __hiloint2double(__double2hiint(q) - (e << 20), __double2loint(q));
 }
 
+// One block of kElB columns at a time: a hand-over costs some 1500 clk whatever it carries. The columns
+// of a block are eliminated among themselves by four warps (one per sub-partition: a float64
+// instruction occupies its sub-partition for 64 clk), with the next block's update before them on the
+// chain; all other updates are off it. The reciprocals travel in two rows of the block's last columns that
+// lie above the diagonal. Mean over the calls of a product of 1D fields (L = 20, chi = 48 capped at 64, p to
+// 128) 19.9 us against 26.4 with one column per hand-over, of an L = 18, chi = 160 product (p to 320)
+// 296 us against 369; what bounds it is the chain: at p = 320, 3100 clk of a block's 7600 are the update of
+// the next one at the float64 rate, 2900 its own columns.
+constexpr int kElB = 4;
+constexpr int kElimSmem = 216 * 1024;  // blocks of one CTA
 template <bool CL>
 __global__ void __launch_bounds__(kQdThreads, 3) pre_elim_kernel(PreElimArgs a) {
   extern __shared__ __align__(16) unsigned char qd_raw[];
@@ -390,178 +400,150 @@ __global__ void __launch_bounds__(kQdThreads, 3) pre_elim_kernel(PreElimArgs a) 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (long e = (long)b * kQdThreads + tid; e < a.clear_n; e += (long)G * kQdThreads)
     a.ex_next[z * a.ex_stride + e] = kQdEmpty;
-  const int nl = b < p ? (p - b + G - 1) / G : 0;
+  const int nb = (p + kElB - 1) / kElB, nl = b < nb ? (nb - b + G - 1) / G : 0;  // blocks, in all and here
   if (!pre_active(a.t, z, a.step)) return;  // alike in all CTAs of the product
   if (!CL && nl == 0) return;
-  double* cols = reinterpret_cast<double*>(qd_raw);     // [cols_ub][ld], column c from row c down
   const int ld = a.ld_ub;
-  double* xs = cols + (long)a.cols_ub * ld;             // [ld]
+  double* cols = reinterpret_cast<double*>(qd_raw);  // [blocks_ub][kElB][ld], a block from its first row down
+  double* xs = cols + (long)a.blocks_ub * kElB * ld;  // [kElB][ld]
   __shared__ int s_abort;
   __shared__ __align__(8) uint64_t bars[CL ? kQdSlots : 1];
   if (tid == 0) s_abort = 0;
   if constexpr (CL) qc_init(bars, tid);
   const double* Gm = bufp(a.t, z, a.bg);
   double* U = bufp(a.t, z, a.bu);
-  for (int e = tid; e < nl * p; e += kQdThreads) {
-    const int l = e / p, i = e - l * p, c = b + G * l;
-    if (i >= c) cols[l * ld + i] = Gm[c + (long)i * p];  // row c of the upper triangle
+  for (int e = tid; e < nl * p * kElB; e += kQdThreads) {
+    const int u = e % kElB, l = e / (kElB * p), i = e / kElB - l * p;
+    const int c = (b + G * l) * kElB + u;
+    if (i >= c - u) cols[(l * kElB + u) * ld + i] = (c < p && i >= c) ? Gm[c + (long)i * p] : 0.0;  // row c of the upper triangle
   }
   unsigned long long* ex = a.ex + z * a.ex_stride;
+  // Warps 0 to 3: eliminates block blk (local l) within itself and hands it on. gl: lane u's squared
+  // norm of column u.
+  auto factor = [&](int blk, int l, double gl) {
+    double* ac = cols + l * kElB * ld;
+    const int cb = blk * kElB;
+    const bool next = blk + 1 < nb && G > 1;
+    double inv[kElB];
+#pragma unroll
+    for (int k = 0; k < kElB; ++k) {
+      asm volatile("bar.sync 2, 128;" ::: "memory");
+      inv[k] = 0.0;
+      if (cb + k >= p) continue;
+      inv[k] = pre_pivot_inv(ac[k * ld + cb + k], __shfl_sync(0xffffffffu, gl, k));
+      double fl = 0.0;
+      if (lane > k && lane < kElB && cb + lane < p) fl = ac[k * ld + cb + lane] * inv[k];
+      double f[kElB];
+#pragma unroll
+      for (int u = k + 1; u < kElB; ++u) f[u] = __shfl_sync(0xffffffffu, fl, u);
+      for (int i = cb + tid; i < p; i += 128) {
+        const double x = ac[k * ld + i];
+#pragma unroll
+        for (int u = k + 1; u < kElB; ++u) ac[u * ld + i] = fma(-f[u], x, ac[u * ld + i]);
+        if (!CL && next) {
+          double y = x;
+          if (k >= 2 && i < cb + 2) y = i == cb ? inv[2 * k - 4] : inv[2 * k - 3];
+          qd_st(ex + (long)(cb + k) * p + i, QdBits<double>::to(y));
+        }
+      }
+    }
+    if (tid < 2 && cb + tid < p) {
+      ac[2 * ld + cb + tid] = tid == 0 ? inv[0] : inv[1];
+      ac[3 * ld + cb + tid] = tid == 0 ? inv[2] : inv[3];
+    }
+    if (CL && next) {
+      asm volatile("bar.sync 2, 128;" ::: "memory");
+      if (warp == 0) qc_publish(bars, blk, nb, G, b, lane);
+    }
+  };
+  // The 16 factors of the update of block c0 / kElB by the block at x (first column jb), one per lane.
+  auto factors = [&](const double* x, int jb, int c0) {
+    const int k = lane & 3, c = c0 + (lane >> 2);
+    return lane < 16 && c < p ? x[k * ld + c] * x[(2 + (k >> 1)) * ld + jb + (k & 1)] : 0.0;
+  };
+  auto update = [&](const double* x, double* ac, const double (&f)[16], int i) {
+    const double x0 = x[i], x1 = x[ld + i], x2 = x[2 * ld + i], x3 = x[3 * ld + i];
+#pragma unroll
+    for (int u = 0; u < kElB; ++u)
+      ac[u * ld + i] = fma(-f[4 * u + 3], x3, fma(-f[4 * u + 2], x2, fma(-f[4 * u + 1], x1, fma(-f[4 * u], x0, ac[u * ld + i]))));
+  };
   __syncthreads();
-  if constexpr (CL) {
-    qc_sync();
-    if (b == 0 && warp == 0) qc_publish(bars, 0, p, G, b, lane);
-  } else if (G > 1 && b == 0) {
-    for (int i = tid; i < p; i += kQdThreads) qd_st(ex + i, QdBits<double>::to(cols[i]));
-  }
+  if constexpr (CL) qc_sync();
+  if (b == 0 && nl > 0 && warp < 4) factor(0, 0, lane < kElB && lane < p ? Gm[lane * (long)(p + 1)] : 0.0);
+  __syncthreads();
   int lj = 0, jr = 0;
-  for (int j = 0; j < p; ++j) {
-    if (nl == 0 || b + G * (nl - 1) < j) break;  // no column from j on is held here
+  for (int blk = 0; blk < nb; ++blk) {
+    if (nl == 0 || b + G * (nl - 1) < blk) break;  // no block from blk on is held here
     const bool mine = jr == b;
-    const uint32_t rem = CL ? qc_map(qc_smem(cols + lj * ld), jr) : 0;  // column j at its owner
-    const int nxt = j + 1;
+    const int jb = blk * kElB, cb = jb + kElB;
     const int nr = jr + 1 == G ? 0 : jr + 1, nlj = jr + 1 == G ? lj + 1 : lj;
-    const int lc = (nr == b && nxt < p) ? nlj : -1;
-    const double* x = mine ? cols + lj * ld : xs;
-    const int base = j & ~31;
-    const double g0 = __ldg(Gm + j + (long)j * p);
-    const int l0 = lc >= 0 ? lc + 1 : lj + (b > jr ? 0 : 1);
-    const unsigned long long* src_x = ex + (long)j * p;
-    if (p - base <= 128) {
-      // x in the registers of every warp that has a column; warp 0 takes the chain
-      const bool work = warp == 0 ? lc >= 0 : l0 + warp - 1 < nl;
-      double xr[4] = {0.0, 0.0, 0.0, 0.0};
-      if (mine) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int i = base + lane + 32 * u;
-          if (i >= j && i < p) xr[u] = x[i];
+    const bool chain = nr == b && blk + 1 < nb;
+    const double* x = mine ? cols + lj * kElB * ld : xs;
+    double gl = 0.0;
+    if (chain && lane < kElB && cb + lane < p) gl = __ldg(Gm + (cb + lane) * (long)(p + 1));
+    if (!mine) {
+      const int k0 = 2 * (tid >> 7);  // two columns per half of the threads
+      if (CL) {
+        if (!qc_wait(bars, blk)) s_abort = 1;
+        const uint32_t rem = qc_map(qc_smem(cols + (lj * kElB + k0) * ld), jr);
+        for (int i = jb + (tid & 127); i < p; i += 128) {
+          const double y0 = qc_ld(rem + (uint32_t)(i * 8), 0.0), y1 = qc_ld(rem + (uint32_t)((ld + i) * 8), 0.0);
+          xs[k0 * ld + i] = y0;
+          xs[(k0 + 1) * ld + i] = y1;
         }
-      } else if (CL) {
-        if (warp == 0) {  // fetches the column for the CTA
-          if (!qc_wait(bars, j)) s_abort = 1;
+      } else {
+        const unsigned long long* s0 = ex + (long)(jb + k0) * p;
+        for (int i = jb + (tid & 127); i < p; i += 256) {
+          unsigned long long bits[4];
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
-            const int i = base + lane + 32 * u;
-            if (i >= j && i < p) xr[u] = qc_ld(rem + (uint32_t)(i * sizeof(double)), 0.0);
-            if (i < p) xs[i] = xr[u];
+            const int r = i + 128 * (u >> 1);
+            bits[u] = r < p ? qd_ld(s0 + (u & 1) * (long)p + r) : 0;
           }
-          asm volatile("bar.arrive 1, 256;" ::: "memory");
-        } else {
-          asm volatile("bar.sync 1, 256;" ::: "memory");
-          if (work) {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const int i = base + lane + 32 * u;
-              if (i < p) xr[u] = xs[i];
-            }
-          }
-        }
-      } else if (work) {
-        unsigned long long bits[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int i = base + lane + 32 * u;
-          bits[u] = (i >= j && i < p) ? qd_ld(src_x + i) : 0;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int i = base + lane + 32 * u;
-          for (int polls = 0; bits[u] == kQdEmpty && polls < kQdPolls; ++polls) bits[u] = qd_ld(src_x + i);
-          if (bits[u] == kQdEmpty) s_abort = 1;
-          xr[u] = QdBits<double>::from(bits[u]);
-        }
-      }
-      if (mine || work) {
-        const double inv = pre_pivot_inv(__shfl_sync(0xffffffffu, xr[0], j & 31), g0);
-        auto update = [&](int l, bool publish) {
-          double* ac = cols + l * ld;
-          const int c = b + G * l, cu = (c - base) >> 5;
-          double xc = 0.0;
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
-            const double t = __shfl_sync(0xffffffffu, xr[u], c & 31);
-            if (u == cu) xc = t;
-          }
-          const double f = xc * inv;
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int i = base + lane + 32 * u;
-            if (base + 32 * u < p && u >= cu) {
-              if (i >= c && i < p) {
-                const double y = fma(-f, xr[u], ac[i]);
-                if (!CL && publish) qd_st(ex + (long)c * p + i, QdBits<double>::to(y));
-                ac[i] = y;
-              }
-            }
-          }
-          if (CL && publish) {
-            __syncwarp();
-            qc_publish(bars, c, p, G, b, lane);
-          }
-        };
-        if (warp == 0) {
-          if (lc >= 0) update(lc, G > 1);
-        } else {
-          for (int l = l0 + warp - 1; l < nl; l += 7) update(l, false);
-        }
-        if (mine && warp == 7) {  // row j of U; zeros for a pivot that does not count
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int i = base + lane + 32 * u;
-            if (i >= j && i < p) U[i + (long)j * p] = inv != 0.0 ? xr[u] : 0.0;
-          }
-        }
-      }
-    } else {
-      if (!mine && CL) {
-        if (!qc_wait(bars, j)) s_abort = 1;
-        for (int i = base + tid; i < p; i += kQdThreads)
-          xs[i] = i >= j ? qc_ld(rem + (uint32_t)(i * sizeof(double)), 0.0) : 0.0;
-      } else if (!mine) {
-        constexpr int NB = 4;
-        for (int i0 = base + tid; i0 < p; i0 += kQdThreads * NB) {
-          unsigned long long bits[NB];
-#pragma unroll
-          for (int u = 0; u < NB; ++u) {
-            const int i = i0 + kQdThreads * u;
-            bits[u] = (i >= j && i < p) ? qd_ld(src_x + i) : 0;
-          }
-#pragma unroll
-          for (int u = 0; u < NB; ++u) {
-            const int i = i0 + kQdThreads * u;
-            if (i >= p) break;
-            for (int polls = 0; bits[u] == kQdEmpty && polls < kQdPolls; ++polls) bits[u] = qd_ld(src_x + i);
+            const int r = i + 128 * (u >> 1);
+            if (r >= p) continue;
+            for (int polls = 0; bits[u] == kQdEmpty && polls < kQdPolls; ++polls) bits[u] = qd_ld(s0 + (u & 1) * (long)p + r);
             if (bits[u] == kQdEmpty) s_abort = 1;
-            xs[i] = QdBits<double>::from(bits[u]);
+            xs[(k0 + (u & 1)) * ld + r] = QdBits<double>::from(bits[u]);
           }
         }
       }
       __syncthreads();
-      const double inv = pre_pivot_inv(x[j], g0);
-      if (lc >= 0 && warp < 4) {  // column j + 1 by one warp per sub-partition, published at once
-        double* ac = cols + lc * ld;
-        const double f = x[nxt] * inv;
-        for (int i = base + tid; i < p; i += 128)
-          if (i > j) {
-            const double y = fma(-f, x[i], ac[i]);
-            if (!CL && G > 1) qd_st(ex + (long)nxt * p + i, QdBits<double>::to(y));
-            ac[i] = y;
-          }
-        if (CL) {
-          asm volatile("bar.sync 2, 128;" ::: "memory");
-          if (warp == 0) qc_publish(bars, nxt, p, G, b, lane);
+    }
+    if (chain) {
+      if (warp < 4) {
+        const double fl = factors(x, jb, cb);
+        double f[16];
+#pragma unroll
+        for (int t = 0; t < 16; ++t) f[t] = __shfl_sync(0xffffffffu, fl, t);
+        for (int i = cb + tid; i < p; i += 128) update(x, cols + nlj * kElB * ld, f, i);
+        factor(blk + 1, nlj, gl);
+      }
+      __syncthreads();
+    }
+    if (mine) {  // rows jb.. of U; zeros for a pivot that does not count
+      for (int k = 0; k < kElB && jb + k < p; ++k) {
+        const bool counts = x[(2 + (k >> 1)) * ld + jb + (k & 1)] != 0.0;
+        for (int i = jb + k + tid; i < p; i += kQdThreads) U[i + (long)(jb + k) * p] = counts ? x[k * ld + i] : 0.0;
+      }
+    }
+    // the other blocks, in chunks of 32 rows dealt out to the warps
+    int t = warp;
+    for (int l = chain ? nlj + 1 : lj + (b > jr ? 0 : 1); l < nl; ++l) {
+      const int c0 = (b + G * l) * kElB, n = (p - c0 + 31) >> 5;
+      if (t < n) {
+        const double fl = factors(x, jb, c0);
+        double f[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) f[u] = __shfl_sync(0xffffffffu, fl, u);
+        for (; t < n; t += 8) {
+          const int i = c0 + 32 * t + lane;
+          if (i < p) update(x, cols + l * kElB * ld, f, i);
         }
       }
-      if (mine)
-        for (int i = j + tid; i < p; i += kQdThreads) U[i + (long)j * p] = inv != 0.0 ? x[i] : 0.0;
-      for (int l = l0 + warp; l < nl; l += 8) {
-        double* ac = cols + l * ld;
-        const int c = b + G * l;
-        const double f = x[c] * inv;
-        for (int i = (c & ~31) + lane; i < p; i += 32)
-          if (i >= c) ac[i] = fma(-f, x[i], ac[i]);
-      }
+      t -= n;
     }
     lj = nlj;
     jr = nr;

@@ -63,6 +63,22 @@ def test_truncated_like_the_oracle(h, L, d, ca, cb, cap, prec):
         assert rep["n_fallback"] == 0 and rep["n_nonconverged"] == 0
 
 
+# The elimination of G in blocks of four columns: Swap matrices past the largest cluster (smaller side
+# above 384), and smaller sides of 4 k + 1, 2, 3 with one, two and several blocks.
+@pytest.mark.parametrize("prec", ["fp64", "bf16_split"])
+@pytest.mark.parametrize("L,d,ca,cb,cap", [(4, 33, 13, 12, 13), (4, 20, 20, 19, 20), (6, 2, 2, 3, 3), (5, 3, 3, 2, 3),
+                                           (4, 5, 3, 5, 3), (4, 7, 5, 3, 5), (4, 11, 5, 4, 5), (4, 23, 9, 7, 9)])
+def test_eliminated_in_blocks(h, prec, L, d, ca, cb, cap):
+    A = ttgen.rand_tt_spectral(L, d, ca, 300 * L + d)
+    B = ttgen.rand_tt_spectral(L, d, cb, 300 * L + d + 1)
+    P = ott.dense(A) * ott.dense(B)
+    O, rep = multiply(h, A, B, eps=1e-14, chi_max=cap, chi_out=cap, prec=prec)
+    Oo, ro = ottm.ttm(A, B, eps=1e-14, chi_max=cap, chi_out=cap)
+    assert ott.bonds_of(O) == ott.bonds_of(Oo)
+    assert relerr(O, P) <= relerr(Oo, P) + 1e-10
+    assert rep["n_fallback"] == 0 and rep["n_nonconverged"] == 0
+
+
 @pytest.mark.parametrize("L,d,ca,cb", [(4, 4, 4, 3), (7, 2, 6, 5), (4, 9, 7, 5)])
 def test_a_small_eps_keeps_the_product(h, L, d, ca, cb):
     A, B = ttgen.rand_tt(L, d, ca, 7), ttgen.rand_tt(L, d, cb, 8)

@@ -375,15 +375,13 @@ void Engine::swap_exact(int x, int y, int bl, int bm, int br, int nbnd, int pb, 
     qrd<double>(q1, n_ub, m_ub);
   });
   if (!launch_) return;
-  pre_norm_kernel<double><<<dim3(cdiv(p_ub, 8), Z_), 256, 0, hs_.stream>>>(PreNormArgs{tab_, L, L, ws(WS_NRM), m, p});
-  TTM_CUDA(cudaGetLastError());
+  TTM_CUDA(launch_pdl(pre_norm_kernel<double>, dim3(cdiv(p_ub, 8), Z_), dim3(256), 0, hs_.stream,
+                      PreNormArgs{tab_, L, L, ws(WS_NRM), m, p}));
   PreOrderArgs oa{tab_, ws(WS_NRM), ws(WS_SORT), ws(WS_PERM), m, n, p, nbnd, 0.0, (int)cap, wslot, 2, -1,
                   svd_rec(cur_svd_), svd_stride(), 0};
-  pre_order_kernel<<<Z_, pow2_threads(p_ub), 0, hs_.stream>>>(oa);
-  TTM_CUDA(cudaGetLastError());
-  pre_left_kernel<<<dim3(cdiv(m_ub, 32), cdiv(k_ub, 32), Z_), 256, 0, hs_.stream>>>(
-      PreLeftArgs{tab_, L, L, ws(WS_PERM), y, m, nbnd});
-  TTM_CUDA(cudaGetLastError());
+  TTM_CUDA(launch_pdl(pre_order_kernel, dim3(Z_), dim3(pow2_threads(p_ub)), 0, hs_.stream, oa));
+  TTM_CUDA(launch_pdl(pre_left_kernel, dim3(cdiv(m_ub, 32), cdiv(k_ub, 32), Z_), dim3(256), 0, hs_.stream,
+                      PreLeftArgs{tab_, L, L, ws(WS_PERM), y, m, nbnd}));
   launches_ += 3;
   timed(2, [&] {
     qrd_apply(QrdApplyArgs{tab_, refl, ws(WS_TAU), n, m, -1, -1, -1, nbnd, x, 0, 0}, n_ub, k_ub);
@@ -446,14 +444,13 @@ void Engine::swap_pre(int x, int y, int bl, int bm, int br, int nbnd, int nprov,
     ja.svd_field = SR_SW0;
     timed(1, [&] { jacobi_pre(ja, p_ub); });
     // its column norms in descending order, the provisional rank, and V
-    pre_norm_kernel<float><<<dim3(cdiv(p_ub, 8), Z_), 256, 0, hs_.stream>>>(PreNormArgs{tab_, X, X, ws(WS_NRM), m, p});
-    TTM_CUDA(cudaGetLastError());
+    TTM_CUDA(launch_pdl(pre_norm_kernel<float>, dim3(cdiv(p_ub, 8), Z_), dim3(256), 0, hs_.stream,
+                        PreNormArgs{tab_, X, X, ws(WS_NRM), m, p}));
     PreOrderArgs oa{tab_, ws(WS_NRM), ws(WS_SORT), ws(WS_PERM), m, n, p, nprov, opt_.eps, (int)cap, -1, 0, ikeep,
                     nullptr, 0, 1};
-    pre_order_kernel<<<Z_, pow2_threads(p_ub), 0, hs_.stream>>>(oa);
-    TTM_CUDA(cudaGetLastError());
-    pre_v_kernel<<<dim3(cdiv(p_ub, 8), Z_), 256, 0, hs_.stream>>>(PreVArgs{tab_, X, ws(WS_PERM), v[0], p});
-    TTM_CUDA(cudaGetLastError());
+    TTM_CUDA(launch_pdl(pre_order_kernel, dim3(Z_), dim3(pow2_threads(p_ub)), 0, hs_.stream, oa));
+    TTM_CUDA(launch_pdl(pre_v_kernel, dim3(cdiv(p_ub, 8), Z_), dim3(256), 0, hs_.stream,
+                        PreVArgs{tab_, X, ws(WS_PERM), v[0], p}));
     launches_ += 3;
   }
   // 4. W = L V and the Newton steps (every launch of the last two is empty for a converged product)
@@ -469,9 +466,8 @@ void Engine::swap_pre(int x, int y, int bl, int bm, int br, int nbnd, int nprov,
     }
     if (s < 2) pre_elim(PreElimArgs{tab_, gram, elim, p, s}, p_ub);
     if (launch_) {
-      pre_x_kernel<<<dim3(cdiv(p_ub, 32), cdiv(p_ub, 8), Z_), 256, 0, hs_.stream>>>(
-          PreXArgs{tab_, s < 2 ? elim : gram, vv, xn, p, ws(WS_SORT), nprov, s, IS_NFROZEN});
-      TTM_CUDA(cudaGetLastError());
+      TTM_CUDA(launch_pdl(pre_x_kernel, dim3(cdiv(p_ub, 32), cdiv(p_ub, 8), Z_), dim3(256), 0, hs_.stream,
+                          PreXArgs{tab_, s < 2 ? elim : gram, vv, xn, p, ws(WS_SORT), nprov, s, IS_NFROZEN}));
       ++launches_;
     }
     if (tc_) {
@@ -485,9 +481,8 @@ void Engine::swap_pre(int x, int y, int bl, int bm, int br, int nbnd, int nprov,
   }
   if (launch_) {
     // a product whose last correction is still large: the float64 Jacobi on L from V = I
-    pre_rescue_kernel<<<dim3((unsigned)std::min<long>(512, cdiv((long)m_ub * p_ub, 256)), Z_), 256, 0, hs_.stream>>>(
-        PreRescueArgs{tab_, L, w[0], v[0], m, p});
-    TTM_CUDA(cudaGetLastError());
+    TTM_CUDA(launch_pdl(pre_rescue_kernel, dim3((unsigned)std::min<long>(512, cdiv((long)m_ub * p_ub, 256)), Z_),
+                        dim3(256), 0, hs_.stream, PreRescueArgs{tab_, L, w[0], v[0], m, p}));
     ++launches_;
     const int nblk_ub = (p_ub + kJrB - 1) / kJrB;
     const int nblk_pad_ub = nblk_ub + (nblk_ub & 1);
@@ -495,15 +490,13 @@ void Engine::swap_pre(int x, int y, int bl, int bm, int br, int nbnd, int nprov,
                  64 * 1.11e-16, fro2_ + (size_t)sw64 * Z_, ST_JFLOPS, ws(WS_NRM), 1, -1, nullptr, 0, 0, 1, IS_FALLBACK};
     timed(3, [&] { jacobi_res<double>(j64, m_ub, p_ub, nblk_pad_ub); });
     // 5. final order, Eq. eps + cap, new carriages
-    pre_norm_kernel<double><<<dim3(cdiv(p_ub, 8), Z_), 256, 0, hs_.stream>>>(PreNormArgs{tab_, w[0], w[1], ws(WS_NRM), m, p});
-    TTM_CUDA(cudaGetLastError());
+    TTM_CUDA(launch_pdl(pre_norm_kernel<double>, dim3(cdiv(p_ub, 8), Z_), dim3(256), 0, hs_.stream,
+                        PreNormArgs{tab_, w[0], w[1], ws(WS_NRM), m, p}));
     PreOrderArgs oa{tab_, ws(WS_NRM), ws(WS_SORT), ws(WS_PERM), m, n, p, nbnd, opt_.eps, (int)cap, wslot, 1, ikeep,
                     svd_rec(cur_svd_), svd_stride(), 1};
-    pre_order_kernel<<<Z_, pow2_threads(p_ub), 0, hs_.stream>>>(oa);
-    TTM_CUDA(cudaGetLastError());
-    pre_left_kernel<<<dim3(cdiv(m_ub, 32), cdiv(k_ub, 32), Z_), 256, 0, hs_.stream>>>(
-        PreLeftArgs{tab_, w[0], w[1], ws(WS_PERM), y, m, nbnd});
-    TTM_CUDA(cudaGetLastError());
+    TTM_CUDA(launch_pdl(pre_order_kernel, dim3(Z_), dim3(pow2_threads(p_ub)), 0, hs_.stream, oa));
+    TTM_CUDA(launch_pdl(pre_left_kernel, dim3(cdiv(m_ub, 32), cdiv(k_ub, 32), Z_), dim3(256), 0, hs_.stream,
+                        PreLeftArgs{tab_, w[0], w[1], ws(WS_PERM), y, m, nbnd}));
     launches_ += 3;
     timed(2, [&] {
       qrd_apply(QrdApplyArgs{tab_, refl, ws(WS_TAU), n, m, v[0], v[1], ws(WS_PERM), nbnd, x, 0, 0}, n_ub, k_ub);
@@ -688,8 +681,7 @@ void Engine::run() {
         ra.n = (int)std::min<size_t>(32, ids.size() - c0);
         for (int q = 0; q < ra.n; ++q) ra.ids[q] = ids[c0 + q];
         ra.cap = (int)opt_.chi_out;
-        round_gate_kernel<<<Z_, 32, 0, hs_.stream>>>(ra);
-        TTM_CUDA(cudaGetLastError());
+        TTM_CUDA(launch_pdl(round_gate_kernel, dim3(Z_), dim3(32), 0, hs_.stream, ra));
         ++launches_;
       }
     }

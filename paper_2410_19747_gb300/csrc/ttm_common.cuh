@@ -86,4 +86,53 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// ---------------------------------------------------------------- dependent launches
+// A plain launch behind another in a stream starts 2.7 us later than a programmatic dependent one (4.1
+// against 1.4 us per launch of a small kernel, 1.0 against 0.8 inside a graph), and a product is some 500
+// to 8000 small launches in a row. Every kernel launched this way calls pdl_begin() before anything
+// else, in all threads: it waits until all earlier work of the stream is done and visible, and
+// then lets the next kernel be set up. No read-only (__ldg, __restrict__) loads in these kernels:
+// their operands are still being written when their blocks are set up.
+__device__ __forceinline__ void pdl_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+inline cudaLaunchAttribute pdl_attr() {
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  return at;
+}
+inline cudaLaunchAttribute cluster_attr(unsigned x) {
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = x;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  return at;
+}
+inline cudaError_t launch_pdl_c(const void* fn, dim3 grid, dim3 block, size_t smem, cudaStream_t st, void** kargs,
+                                unsigned cluster = 1) {
+  cudaLaunchAttribute at[2] = {pdl_attr(), cluster_attr(cluster)};
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  return cudaLaunchKernelExC(&cfg, fn, kargs);
+}
+template <class... P, class... A>
+cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, const A&... args) {
+  cudaLaunchAttribute at[1] = {pdl_attr()};
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 }  // namespace ttm

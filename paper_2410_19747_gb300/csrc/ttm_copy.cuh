@@ -18,6 +18,7 @@ struct CopyDesc {
 // unit stride whichever of the two has it.
 template <class F>
 __global__ void __launch_bounds__(256) copy2d_kernel(F f, int nbatch) {
+  pdl_begin();
   const int z = blockIdx.z / nbatch, b = blockIdx.z % nbatch;
   const CopyDesc c = f(z, b);
   const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;

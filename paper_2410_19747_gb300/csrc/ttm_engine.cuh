@@ -244,8 +244,8 @@ class Engine {
   void pcopy(int src, int dst, Dim rows, Dim cols, int islot, int want, long n_ub) {
     if (!launch_) return;
     PredCopyArgs pa{tab_, src, dst, rows, cols, islot, want};
-    pred_copy_kernel<<<dim3((unsigned)std::min<long>(1024, cdiv(n_ub, 256)), Z_), 256, 0, hs_.stream>>>(pa);
-    TTM_CUDA(cudaGetLastError());
+    TTM_CUDA(launch_pdl(pred_copy_kernel, dim3((unsigned)std::min<long>(1024, cdiv(n_ub, 256)), Z_), dim3(256), 0,
+                        hs_.stream, pa));
     ++launches_;
   }
   // X of a Newton step from G and M (ttm_newton.cuh).
@@ -271,16 +271,14 @@ class Engine {
   void colexp(int wbuf, Dim m, Dim n, int n_ub, int out = -1) {
     if (!launch_) return;
     ColExpArgs ca{tab_, wbuf, out < 0 ? ws(WS_TAU) : out, m, n};
-    colexp_kernel<<<dim3(cdiv(n_ub, 8), Z_), 256, 0, hs_.stream>>>(ca);
-    TTM_CUDA(cudaGetLastError());
+    TTM_CUDA(launch_pdl(colexp_kernel, dim3(cdiv(n_ub, 8), Z_), dim3(256), 0, hs_.stream, ca));
     ++launches_;
   }
   template <class F>
   void copy2d(const F& f, int nbatch, int R_ub, int C_ub) {
     if (!launch_) return;
     dim3 grid(cdiv(C_ub, 32), cdiv(R_ub, 32), (unsigned)(Z_ * nbatch));
-    copy2d_kernel<F><<<grid, 256, 0, hs_.stream>>>(f, nbatch);
-    TTM_CUDA(cudaGetLastError());
+    TTM_CUDA(launch_pdl(copy2d_kernel<F>, grid, dim3(256), 0, hs_.stream, f, nbatch));
     ++launches_;
   }
   void cast(int src, int dst, Dim rows, Dim cols, int to_float, long n_ub) {
@@ -372,19 +370,8 @@ class Engine {
     }
   }
   static void launch_cluster(void* fn, int groups, int G, int threads, size_t smem, void** kargs, cudaStream_t st) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(groups * G));
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)G;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
     TTM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    TTM_CUDA(cudaLaunchKernelExC(&cfg, fn, kargs));
+    TTM_CUDA(launch_pdl_c(fn, dim3((unsigned)(groups * G)), dim3((unsigned)threads), smem, st, kargs, (unsigned)G));
   }
   // Plans or launches it. a: everything but the sizes of the distribution.
   template <typename T>
@@ -407,7 +394,7 @@ class Engine {
       use_exchange(a, extent);
       TTM_CUDA(cudaLaunchCooperativeKernel(fn, dim3((unsigned)(Z_ * G)), dim3(kQdThreads), kargs, smem, hs_.stream));
     } else {
-      TTM_CUDA(cudaLaunchKernel(fn, dim3((unsigned)Z_), dim3(kQdThreads), kargs, smem, hs_.stream));
+      TTM_CUDA(launch_pdl_c(fn, dim3((unsigned)Z_), dim3(kQdThreads), smem, hs_.stream, kargs));
     }
     ++launches_;
     return true;
@@ -475,7 +462,7 @@ class Engine {
       use_exchange(a, (long)p_ub * p_ub);
       TTM_CUDA(cudaLaunchCooperativeKernel(fn, dim3((unsigned)(Z_ * G)), dim3(kQdThreads), kargs, smem, hs_.stream));
     } else {
-      TTM_CUDA(cudaLaunchKernel(fn, dim3((unsigned)Z_), dim3(kQdThreads), kargs, smem, hs_.stream));
+      TTM_CUDA(launch_pdl_c(fn, dim3((unsigned)Z_), dim3(kQdThreads), smem, hs_.stream, kargs));
     }
     ++launches_;
   }
@@ -495,7 +482,7 @@ class Engine {
     if (a.cluster) {
       launch_cluster(fn, Z_, a.G, kPjThreads, smem, kargs, hs_.stream);
     } else if (a.G == 1) {
-      TTM_CUDA(cudaLaunchKernel(fn, dim3((unsigned)Z_), dim3(kPjThreads), kargs, smem, hs_.stream));
+      TTM_CUDA(launch_pdl_c(fn, dim3((unsigned)Z_), dim3(kPjThreads), smem, hs_.stream, kargs));
     } else {
       a.ngroup = std::max(1, std::min(Z_, hs_.num_sms / a.G));
       TTM_CUDA(cudaLaunchCooperativeKernel(fn, dim3((unsigned)(a.ngroup * a.G)), dim3(kPjThreads), kargs, smem, hs_.stream));
@@ -518,8 +505,8 @@ class Engine {
     void* fn = wide ? (void*)qrd_apply_kernel<4> : (void*)qrd_apply_kernel<1>;
     void* kargs[] = {&a};
     TTM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    TTM_CUDA(cudaLaunchKernel(fn, dim3(wide ? (unsigned)c_ub : cdiv(c_ub, 4), (unsigned)Z_), dim3(kQaThreads), kargs, smem,
-                              hs_.stream));
+    TTM_CUDA(launch_pdl_c(fn, dim3(wide ? (unsigned)c_ub : cdiv(c_ub, 4), (unsigned)Z_), dim3(kQaThreads), smem, hs_.stream,
+                          kargs));
     ++launches_;
   }
   long launches_ = 0;

@@ -66,6 +66,7 @@ struct GemmShape {
 template <class F, int DT>
 __global__ void __launch_bounds__(kDgThreads) dgemm_kernel(F f, int nbatch, int n_tiles, int split, double* fl,
                                                            int fl_stride) {
+  pdl_begin();
   const int z = blockIdx.z / nbatch, bi = blockIdx.z % nbatch;
   const GemmDesc g = f(z, bi);
   const int rank = blockIdx.x % split, tile = blockIdx.x / split;
@@ -186,13 +187,9 @@ cudaError_t launch_dgemm(cudaStream_t st, const F& f, int nprob, int nbatch, int
   cfg.gridDim = dim3((unsigned)(tiles * split), 1, (unsigned)nprob);
   cfg.blockDim = dim3(kDgThreads);
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)split;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
+  cudaLaunchAttribute at[2] = {pdl_attr(), cluster_attr((unsigned)split)};
   cfg.attrs = at;
-  cfg.numAttrs = split > 1 ? 1 : 0;
+  cfg.numAttrs = split > 1 ? 2 : 1;
   if (big) return cudaLaunchKernelEx(&cfg, dgemm_kernel<F, 32>, f, nbatch, n_tiles, split, fl, fl_stride);
   return cudaLaunchKernelEx(&cfg, dgemm_kernel<F, 16>, f, nbatch, n_tiles, split, fl, fl_stride);
 }

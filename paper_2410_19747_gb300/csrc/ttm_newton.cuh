@@ -167,6 +167,7 @@ struct PredCopyArgs {
   int islot, want;
 };
 __global__ void pred_copy_kernel(PredCopyArgs a) {
+  pdl_begin();
   const int z = blockIdx.y;
   if (a.islot >= 0 && a.t.istat[z * a.t.nis + a.islot] != a.want) return;
   const long n = (long)a.rows.eval(a.t, z) * a.cols.eval(a.t, z);

@@ -115,6 +115,7 @@ __device__ __forceinline__ void pj_rotate(float (&x)[R], float (&y)[R], float c,
 
 template <int R>
 __global__ void __launch_bounds__(kPjThreads, 1) jacobi_pre_kernel(PreJacArgs a) {
+  pdl_begin();
   extern __shared__ __align__(16) unsigned char pj_raw[];
   constexpr int B = kPjB, MR = 32 * R;
   constexpr int VW = JrVec<float, R>::VW;

@@ -118,6 +118,7 @@ struct PreNormArgs {
 };
 template <typename T>
 __global__ void pre_norm_kernel(PreNormArgs a) {
+  pdl_begin();
   const int z = blockIdx.y, lane = threadIdx.x & 31;
   const int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int p = a.p.eval(a.t, z);
@@ -159,6 +160,7 @@ struct PreOrderArgs {
   int sort;         // 0: the columns stay in their order (nothing is truncated)
 };
 __global__ void __launch_bounds__(1024) pre_order_kernel(PreOrderArgs a) {
+  pdl_begin();
   const int z = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int p = a.p.eval(a.t, z);
   __shared__ long long key[kPreMax];
@@ -283,6 +285,7 @@ struct PreVArgs {
   Dim p;
 };
 __global__ void pre_v_kernel(PreVArgs a) {
+  pdl_begin();
   const int z = blockIdx.y, lane = threadIdx.x & 31;
   const int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int p = a.p.eval(a.t, z);
@@ -394,6 +397,7 @@ constexpr int kElB = 4;
 constexpr int kElimSmem = 216 * 1024;  // blocks of one CTA
 template <bool CL>
 __global__ void __launch_bounds__(kQdThreads, 3) pre_elim_kernel(PreElimArgs a) {
+  pdl_begin();
   extern __shared__ __align__(16) unsigned char qd_raw[];
   const int G = a.G, z = blockIdx.x / G, b = blockIdx.x % G;
   const int p = a.p.eval(a.t, z);
@@ -480,7 +484,7 @@ __global__ void __launch_bounds__(kQdThreads, 3) pre_elim_kernel(PreElimArgs a) 
     const bool chain = nr == b && blk + 1 < nb;
     const double* x = mine ? cols + lj * kElB * ld : xs;
     double gl = 0.0;
-    if (chain && lane < kElB && cb + lane < p) gl = __ldg(Gm + (cb + lane) * (long)(p + 1));
+    if (chain && lane < kElB && cb + lane < p) gl = Gm[(cb + lane) * (long)(p + 1)];
     if (!mine) {
       const int k0 = 2 * (tid >> 7);  // two columns per half of the threads
       if (CL) {
@@ -565,6 +569,7 @@ struct PreXArgs {
   int step, islot_frozen;
 };
 __global__ void __launch_bounds__(256) pre_x_kernel(PreXArgs a) {
+  pdl_begin();
   const int z = blockIdx.z;
   const int p = a.p.eval(a.t, z);
   const int i = blockIdx.x * 32 + (threadIdx.x & 31), j = blockIdx.y * 8 + (threadIdx.x >> 5);
@@ -639,6 +644,7 @@ struct PreRescueArgs {
   Dim m, p;
 };
 __global__ void pre_rescue_kernel(PreRescueArgs a) {
+  pdl_begin();
   const int z = blockIdx.y;
   const bool bad = pre_failed(a.t, z);
   if (blockIdx.x == 0 && threadIdx.x == 0) a.t.istat[z * a.t.nis + IS_FALLBACK] = bad ? 1 : 0;
@@ -658,6 +664,7 @@ struct PreLeftArgs {
   int ik;
 };
 __global__ void __launch_bounds__(256) pre_left_kernel(PreLeftArgs a) {
+  pdl_begin();
   const int z = blockIdx.z;
   const int m = a.m.eval(a.t, z), k = bondv(a.t, z, a.ik);
   const int r0 = blockIdx.x * 32, j0 = blockIdx.y * 32;

@@ -154,6 +154,7 @@ __device__ __forceinline__ void qd_st(unsigned long long* p, unsigned long long 
 
 template <typename T>
 __global__ void __launch_bounds__(kQdThreads, 3) qrd_kernel(QrdArgs a) {
+  pdl_begin();
   extern __shared__ __align__(16) unsigned char qd_raw[];
   const int G = a.G, z = blockIdx.x / G, b = blockIdx.x % G;
   const int M = a.m.eval(a.t, z), N = a.n.eval(a.t, z), k = min(M, N);
@@ -487,6 +488,7 @@ struct QrdApplyArgs {
 // chip has sub-partitions). On 256 rows a step takes about 1400 clocks with one warp, 900 with four.
 template <int WPC>
 __global__ void __launch_bounds__(kQaThreads) qrd_apply_kernel(QrdApplyArgs a) {
+  pdl_begin();
   extern __shared__ __align__(16) unsigned char qd_raw[];
   constexpr int CPB = 4 / WPC;  // columns per CTA
   __shared__ double red[2][4];
@@ -527,7 +529,7 @@ __global__ void __launch_bounds__(kQaThreads) qrd_apply_kernel(QrdApplyArgs a) {
   };
   for (int s = 0; s < kQaStages - 1; ++s) fetch(j0 - s);
   for (int j = j0; j >= 0; --j) {
-    const double tj = __ldg(tau + j);
+    const double tj = tau[j];
     asm volatile("cp.async.wait_group %0;" ::"n"(kQaStages - 2) : "memory");
     __syncthreads();  // reflector j is here, and its ring slot of step j + 1 is free again
     fetch(j - (kQaStages - 1));

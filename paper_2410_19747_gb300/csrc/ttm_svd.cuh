@@ -435,6 +435,7 @@ struct RoundGateArgs {
   int cap;
 };
 __global__ void round_gate_kernel(RoundGateArgs a) {
+  pdl_begin();
   const int z = blockIdx.x;
   const int i = threadIdx.x;
   if (i < a.n && bondv(a.t, z, a.ids[i]) > a.cap) atomicOr(&a.t.istat[z * a.t.nis + IS_ROUND], 1);

@@ -80,6 +80,7 @@ struct ColExpArgs {
   Dim m, n;
 };
 __global__ void colexp_kernel(ColExpArgs a) {
+  pdl_begin();
   const int z = blockIdx.y;
   const int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
@@ -147,6 +148,7 @@ __device__ __forceinline__ long long oz_fixed(long long bits, int sh) {
 constexpr int kOzPrepRows = 16;
 template <class F>
 __global__ void __launch_bounds__(256) oz_prep_kernel(OzArgs<F> a, int mpad, int npad, int kpad) {
+  pdl_begin();
   const int zb = blockIdx.z, z = zb / a.nbatch, b = zb % a.nbatch;
   const GemmDesc g = a.f(z, b);
   if (g.M <= 0 || g.N <= 0) return;  // nothing of this problem is multiplied
@@ -306,6 +308,7 @@ constexpr uint64_t kOzWaitNs = 2000000000ull;  // 2 s: far beyond any legitimate
 // Grid: (N tiles of 64, M tiles of 128, problems). Dynamic shared memory: oz_smem_bytes(S).
 template <class F>
 __global__ void __launch_bounds__(kOzThreads, 1) oz_gemm_kernel(OzArgs<F> a, int mpad, int npad, int kpad) {
+  pdl_begin();
   extern __shared__ __align__(1024) unsigned char smem[];
   const int zb = blockIdx.z, z = zb / a.nbatch, b = zb % a.nbatch;
   const GemmDesc g = a.f(z, b);
@@ -534,17 +537,15 @@ cudaError_t launch_tc_gemm(cudaStream_t st, const F& f, int nz, int nbatch, int 
   // every launch is checked at once: the caller gets the first failing step
   const char*& step = tc_failed_step();
   step = "oz_prep_kernel";
-  oz_prep_kernel<F><<<dim3((unsigned)((mpad + npad) / kOzPrepRows), 1, (unsigned)nprob), 256, 0, st>>>(
-      oa, (int)mpad, (int)npad, (int)kpad);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_pdl(oz_prep_kernel<F>, dim3((unsigned)((mpad + npad) / kOzPrepRows), 1, (unsigned)nprob),
+                             dim3(256), 0, st, oa, (int)mpad, (int)npad, (int)kpad);
   if (e != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(oz_gemm_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 oz_smem_bytes(kOzMaxS))) != cudaSuccess)
     return e;
   step = "oz_gemm_kernel";
-  oz_gemm_kernel<F><<<dim3((unsigned)(npad / kOzTN), (unsigned)(mpad / kOzTM), (unsigned)nprob), kOzThreads,
-                      oz_smem_bytes(S), st>>>(oa, (int)mpad, (int)npad, (int)kpad);
-  return cudaGetLastError();
+  return launch_pdl(oz_gemm_kernel<F>, dim3((unsigned)(npad / kOzTN), (unsigned)(mpad / kOzTM), (unsigned)nprob),
+                    dim3(kOzThreads), oz_smem_bytes(S), st, oa, (int)mpad, (int)npad, (int)kpad);
 }
 
 }  // namespace ttm

@@ -36,7 +36,7 @@ L2_BYTES = 129 * 2 ** 20
 # DRAM bytes (read + write) per launch of a kernel, from the committed ncu captures (one launch
 # each, named in the source); they describe the kernels as they are at the time of the capture.
 MEASURED_TRAFFIC = {
-    "jacobi_res_kernel<float>": (5.58e6, "profiles/jacobi_res_f32_chi512_L20.md: one full-size float32 pass "
+    "jacobi_res_kernel<float> (": (5.58e6, "profiles/jacobi_res_f32_chi512_L20.md: one full-size float32 pass "
                                          "(1024 x 1024, 70 ms); W and V stay in L2"),
     "oz_gemm_kernel": (7.29e6, "profiles/oz_gemm_gram_chi512_L20.md: one 1024^3 Gram"),
 }
@@ -83,16 +83,19 @@ def workload(L, chi, seed):
 
 def config(args):
     prec = getattr(args, "prec", "fp64")
+    preconditioned = args.chi <= 512 and not any(
+        getattr(args, n, 0) for n in ("f32_passes", "jacobi_kernel", "newton_steps", "max_sweeps"))
+    passes = {0: "default kernel", 1: "scalar kernel", 2: "two-column kernel", 3: "resident-block kernel",
+              8: "Gram block 8", 16: "Gram block 16"}[args.jacobi_kernel]
+    first = ("two QR factorisations and one float32 one-sided Jacobi" if preconditioned else
+             "one-sided Jacobi, %d float32 passes (%s)" % (args.f32_passes or 3, passes))
     return {"workload": "config3: random right-canonical TT pair, L=%d, d=2, chi=%d, a 1/k profile on every "
                         "bond (realised Schmidt spectra steeper), float64 cores, eps=%g, chi_max=chi_out=%d"
                         % (args.L, args.chi, args.eps, args.chi),
             "L": args.L, "d": 2, "chi": args.chi, "eps": args.eps, "chi_out": args.chi,
             "precision_mode": prec, "batch": getattr(args, "batch", 1),
-            "svd": "one-sided Jacobi, %d float32 passes (%s), then %d float64 Newton steps; GEMMs %s"
-                   % (args.f32_passes or 3, {0: "default kernel", 1: "scalar kernel", 2: "two-column kernel",
-                                             3: "resident-block kernel", 8: "Gram block 8",
-                                             16: "Gram block 16"}[args.jacobi_kernel],
-                      getattr(args, "newton_steps", 0) or 3,
+            "svd": "%s, then %d float64 Newton steps or more; GEMMs %s"
+                   % (first, getattr(args, "newton_steps", 0) or (2 if preconditioned else 3),
                       "on the float64 pipe" if prec == "fp64" else
                       "as %d-digit bf16 products on the tensor cores" % (getattr(args, "split_digits", 0) or 8)),
             "l2": "flushed between timed steps (256 MiB write outside the timed events)"}
@@ -352,7 +355,7 @@ def kernel_roofline(args, reps, t_local):
     n_g = sum(r["gemm_launches"] for r in reps)
     if tc:
         ach = gemm_fl * S * (S + 1) / 2 / (gemm_ms / 1e3) / 1e12 if gemm_ms > 0 else None
-        kernels.append({"bound": "tensor", "kernel": "oz_gemm_kernel (+ exponent and digit kernels): float64 "
+        kernels.append({"bound": "tensor", "kernel": "oz_gemm_kernel (+ oz_prep_kernel): float64 "
                         "GEMMs as %d-digit bf16 tcgen05 products" % S, "achieved": ach,
                         "peak": peaks["bf16_tflops_sustained"], "unit": "TFLOP/s",
                         "peak_source": "%s dense bf16, sustained (kernel timed inside a long step)" % peaks["source"],
@@ -368,7 +371,9 @@ def kernel_roofline(args, reps, t_local):
     j_ms = sum(r["jacobi32_ms"] for r in reps)
     j_fl = sum(r["jacobi32_flops"] for r in reps)
     jk = getattr(args, "jacobi_kernel", 0)
-    jname = {0: "jacobi_res_kernel<float> (resident-block one-sided Jacobi, float32)",
+    general = any(getattr(args, n, 0) for n in ("f32_passes", "newton_steps", "max_sweeps"))
+    jname = {0: "jacobi_res_kernel<float>" + (" (" if general else " or, for Swaps of at most 1024 rows, jacobi_pre_kernel (")
+                + "resident-block one-sided Jacobi, float32)",
              1: "hestenes_kernel<float> (one-sided Jacobi, float32)",
              2: "jacobi4_kernel (two-column one-sided Jacobi, float32)",
              3: "jacobi_res_kernel<float> (resident-block one-sided Jacobi, float32)",
@@ -381,7 +386,7 @@ def kernel_roofline(args, reps, t_local):
     kernels.append({"bound": "alu", "kernel": "jacobi_res_kernel<double> (float64 one-sided Jacobi of the "
                     "Newton fallback)", "achieved": None, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                     "ms": sum(r.get("jacobi64_ms", 0.0) for r in reps), "launches": None})
-    kernels.append({"bound": "latency", "kernel": "householder_kernel (float64 QR of the gauge moves)",
+    kernels.append({"bound": "latency", "kernel": "qrd_kernel, qrd_apply_kernel (QR of the gauge moves and of the Swaps)",
                     "achieved": None, "peak": None, "unit": None, "ms": sum(r["qr_ms"] for r in reps),
                     "launches": None})
     for k in kernels:

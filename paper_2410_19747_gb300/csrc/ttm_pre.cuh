@@ -27,7 +27,8 @@
 // Bound by latencies: the chains of the two QRs (about 1.3 and 0.7 us per column), of the inner rounds
 // of the Jacobi and of the elimination. Measured per product (GB300) against three float32 passes
 // with V, three to five Newton steps and a saved state: 2D field, d = 4, chi = 64 332 -> 153 ms; 3D
-// field, d = 8, chi = 96 503 -> 205 ms; random L = 10 61 -> 21 ms; chi = 160, L = 18 1616 -> 825 ms.
+// field, d = 8, chi = 96 503 -> 205 ms; random L = 10 61 -> 21 ms; chi = 160, L = 18 1616 -> 825 ms
+// (129, 131, 8.6 and 486 ms with what was made faster in these kernels and their launches since).
 #pragma once
 #include <cooperative_groups.h>
 #include "ttm_common.cuh"

@@ -27,7 +27,7 @@
 // Bound at 1024^3 by the operand traffic (96 KB per K chunk and CTA through L2), at small sizes by one
 // tile's chain. Measured (GB300): exponents and digits in one integer launch instead of five float64
 // ones, one instruction per four digits of B, and an epilogue of three float64 instructions per
-// output instead of eight take a 1500 x 1024 x 2000 product from 1100 to 495 us and a 320^3 one from
+// output instead of eight take a 1500 x 1024 x 2000 product from 1100 to 550 us and a 320^3 one from
 // about 110 to 45 us.
 #pragma once
 #include <cuda_bf16.h>

@@ -941,8 +941,26 @@ void Engine::execute(void* arena, const ttm_options& opt, std::vector<ttm_report
   TTM_CUDA(cudaStreamSynchronize(st));
 }
 
+// The dynamic shared memory limits of the kernels whose launches differ in size, on the current device.
+// The limit belongs to the function and the device, so that handles on several host threads share it:
+// it is set to the largest size the launch code asks for and never lowered again (set to each launch's own
+// size, a small launch of one thread made a larger one of another thread fail).
+static void set_shared_limits() {
+  auto set = [](void* fn, int bytes) {
+    TTM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  };
+  set((void*)qrd_kernel<double>, kQdSmem);
+  set((void*)qrd_kernel<float>, kQdSmem);
+  set((void*)qrd_apply_kernel<1>, kQdSmem);
+  set((void*)qrd_apply_kernel<4>, kQdSmem);
+  set((void*)pre_elim_kernel<true>, kElimSmem);
+  set((void*)pre_elim_kernel<false>, kElimSmem);
+  // (one size per instantiation: the launch sets it again to the same value)
+  set(jacobi_pre_fn(16), 2 * kPjB * 512 * 4);
+}
+
 // Whether clusters of 16 CTAs of the distributed kernels, at their largest shared memory, can be
-// scheduled on the current device; else the portable 8.
+// scheduled on the current device; else the portable 8. After set_shared_limits().
 static int query_max_cluster() {
   struct Probe {
     void* fn;
@@ -954,7 +972,6 @@ static int query_max_cluster() {
        (kElimClusterMax / (kElimCluster * kElB) + 1) * kElB * kElimClusterMax * 8},
       {jacobi_pre_fn(16), kPjThreads, 2 * kPjB * 512 * 4}};
   for (const Probe& p : probes) {
-    TTM_CUDA(cudaFuncSetAttribute(p.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem));
     TTM_CUDA(cudaFuncSetAttribute(p.fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(kElimCluster);
@@ -1098,6 +1115,7 @@ ttm_status ttm_create(ttm_handle** h, int device, void* cuda_stream, const ttm_o
     TTM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&H->s.coop_hest32, hestenes_kernel<float>, 256, 0));
     TTM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&H->s.coop_hest, hestenes_kernel<double>, 256, 0));
     TTM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&H->s.coop_qr, householder_kernel, 256, 0));
+    set_shared_limits();
     H->s.max_cluster = query_max_cluster();
     int coop = 0;
     TTM_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device));
@@ -1278,6 +1296,7 @@ ttm_status ttm_multiply_noalloc(const ttm_tt* A, const ttm_tt* B, ttm_tt* out, c
         TTM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nd.coop_hest32, hestenes_kernel<float>, 256, 0));
         TTM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nd.coop_hest, hestenes_kernel<double>, 256, 0));
         TTM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nd.coop_qr, householder_kernel, 256, 0));
+        set_shared_limits();
         nd.max_cluster = query_max_cluster();
         nd.scratch = p;
         nd.ready = true;

@@ -389,7 +389,6 @@ class Engine {
     a.ld_ub = m_ub;
     void* fn = (void*)qrd_kernel<T>;
     void* kargs[] = {&a};
-    TTM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if (G > 1) {
       use_exchange(a, extent);
       TTM_CUDA(cudaLaunchCooperativeKernel(fn, dim3((unsigned)(Z_ * G)), dim3(kQdThreads), kargs, smem, hs_.stream));
@@ -455,7 +454,6 @@ class Engine {
     a.ld_ub = p_ub;
     void* kargs[] = {&a};
     void* fn = cluster ? (void*)pre_elim_kernel<true> : (void*)pre_elim_kernel<false>;
-    TTM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if (cluster) {
       launch_cluster(fn, Z_, G, kQdThreads, smem, kargs, hs_.stream);
     } else if (G > 1) {
@@ -504,7 +502,6 @@ class Engine {
     const size_t smem = (size_t)(kQaStages + (wide ? 1 : 4)) * m_ub * sizeof(double);
     void* fn = wide ? (void*)qrd_apply_kernel<4> : (void*)qrd_apply_kernel<1>;
     void* kargs[] = {&a};
-    TTM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     TTM_CUDA(launch_pdl_c(fn, dim3(wide ? (unsigned)c_ub : cdiv(c_ub, 4), (unsigned)Z_), dim3(kQaThreads), smem, hs_.stream,
                           kargs));
     ++launches_;

@@ -859,11 +859,11 @@ void Engine::execute(void* arena, const ttm_options& opt, std::vector<ttm_report
     std::memset(&r, 0, sizeof(r));
     r.status = TTM_OK;
     r.jacobi_sweeps_max = istat[(size_t)z * nis + IS_SWEEPS_MAX];
-    long maxb = 0;
-    for (int id = 0; id < nbd; ++id) maxb = std::max(maxb, bv(id));
-    r.max_bond = maxb;
+    // over the bonds of the trains only: other ids hold provisional ranks and min(m, n) of a Swap
+    long maxb = 1;
     double fl = 0.0;
     for (const StepLog& s : log_) {
+      maxb = std::max({maxb, bv(s.b0), bv(s.b1), bv(s.b2), bv(s.b3)});
       if (s.kind == SK_SWAP || s.kind == SK_ROUND) {
         if (s.kind == SK_SWAP) r.n_swaps++;
         const double Dl = bv(s.b0), Dm = bv(s.b1), Dr = bv(s.b2), k = bv(s.b3);
@@ -882,6 +882,7 @@ void Engine::execute(void* arena, const ttm_options& opt, std::vector<ttm_report
         fl += 2.0 * k * n * d_ * rr;                     // R merge
       }
     }
+    r.max_bond = maxb;
     r.flops_counted = fl;
     r.discarded_weight = stat[(size_t)z * ns + ST_WSUM];
     r.err_bound = stat[(size_t)z * ns + ST_WSQRT];

@@ -202,12 +202,15 @@ int Engine::swap(int x, int y, int bl, int bm, int br, int kind) {
   if (pre_fits(m_ub, n_ub)) {
     for (int z = 0; z < Z_; ++z) kub[z] = std::min(d_ * ub_[bl][z], d_ * ub_[br][z]);
     const int pb = new_bond(kub);          // min(m, n)
-    if (opt_.eps == 0.0 && kind == SK_SWAP && (cap <= 0 || cap >= umax(pb)))
+    if (opt_.eps == 0.0 && kind == SK_SWAP && (cap <= 0 || cap >= umax(pb))) {
       swap_exact(x, y, bl, bm, br, nbnd, pb, cap, wslot);
-    else
+    } else {
+      ++jac32_count_;
       swap_pre(x, y, bl, bm, br, nbnd, nprov, pb, kind, cap, sw32, sw64, wslot);
+    }
     return nbnd;
   }
+  jac32_count_ += npass;
   if (launch_) {
     const Dim m{d_, bl}, n{d_, br};
     const int npad_ub = n_ub + (n_ub & 1);
@@ -894,7 +897,7 @@ void Engine::execute(void* arena, const ttm_options& opt, std::vector<ttm_report
     r.n_frozen_pairs = istat[(size_t)z * nis + IS_NFROZEN];
     if (r.n_nonconverged > 0) r.status = TTM_WARN_NOT_CONVERGED;  // result formed; optimality not guaranteed
     r.n_kernel_launches = launches_;
-    r.jacobi_launches = jac_launch_;
+    r.jacobi_launches = jac32_count_;
     r.gemm_ms = kind_ms[0];
     r.jacobi32_ms = kind_ms[1];
     r.qr_ms = kind_ms[2];

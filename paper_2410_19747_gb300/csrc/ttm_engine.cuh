@@ -106,7 +106,8 @@ class Engine {
   int* svd_rec(int i) const { return svd_log_ ? svd_log_ + (size_t)i * kSvdRec : nullptr; }
   int svd_stride() const { return std::max(1, n_trunc_planned_) * kSvdRec; }
   int n_trunc_planned_ = 0;
-  int jac_launch_ = 0;
+  int jac_launch_ = 0;      // counter slots: one per Jacobi launch the general pipeline may need
+  int jac32_count_ = 0;     // float32 Jacobi launches of the walk
   int* d_bond_ = nullptr;
   double** d_buf_ = nullptr;
   double* d_stat_ = nullptr;
@@ -129,6 +130,7 @@ class Engine {
     log_.clear();
     trace_ids_.clear();
     jac_launch_ = 0;
+    jac32_count_ = 0;
     ex_flip_ = 0;
     ex_prev_ = 0;
   }

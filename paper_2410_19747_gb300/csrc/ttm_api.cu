@@ -1318,14 +1318,13 @@ ttm_status ttm_multiply_noalloc(const ttm_tt* A, const ttm_tt* B, ttm_tt* out, c
     hs.max_cluster = info.max_cluster;
     Engine e(hs, 1, A, B);
     e.plan();
-    // the limit is on the workspace of the general kernels; they run alone where the array has no
-    // room for what the faster ones add
-    const size_t need = e.base_bytes();
-    const bool room = e.bytes_needed() <= (size_t)TTM_NOALLOC_SCRATCH_BYTES;
-    if (!room) {
+    // Where the array has no room for what the faster kernels add, the general ones run alone; the limit
+    // is on their plan (the other one also has a few more bond ids).
+    if (e.bytes_needed() > (size_t)TTM_NOALLOC_SCRATCH_BYTES) {
       e.base_only();
       e.plan();
     }
+    const size_t need = e.bytes_needed();
     if (need > (size_t)TTM_NOALLOC_SCRATCH_BYTES)
       throw Error(TTM_ERR_WORKSPACE, "the product needs " + std::to_string(need) +
                                          " bytes of workspace; the allocation-free path has " +

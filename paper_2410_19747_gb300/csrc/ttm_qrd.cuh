@@ -70,6 +70,22 @@ __device__ __forceinline__ T qd_sum4(const T (&s)[4], int lane) {
   return c;
 }
 
+// A float64 column whose squared norm g is below the normal range (but the column is not zero), or finite
+// and at least 2^1020 (its tau would leave the range), is scaled by this power of two before its scalars are
+// formed; beta, v and tau are then those of the scaled column, and only the diagonal entry of R is scaled
+// back. 1 for every other column, a zero, an infinite and a NaN one included.
+__device__ __forceinline__ bool qd_out_of_range(double g) {  // g >= 0 or a NaN
+  return (unsigned)(__double2hiint(g) - 0x00100000) >= (unsigned)(0x7fb00000 - 0x00100000);
+}
+__device__ __forceinline__ double qd_rescale(double g, bool zero) {
+  const int hi = __double2hiint(g);
+  if (zero || (hi & 0x7fffffff) >= 0x7ff00000) return 1.0;
+  return __hiloint2double(hi < 0x00100000 ? (1023 + 800) << 20 : (1023 - 512) << 20, 0);
+}
+__device__ __forceinline__ bool qd_nonzero(double x) {
+  return ((__double2hiint(x) & 0x7fffffff) | __double2loint(x)) != 0;
+}
+
 // beta, v_j and tau of a column with squared norm g and leading entry alpha. A column that counts as
 // zero has tau = 0; a NaN travels on in beta.
 __device__ __forceinline__ void qd_scalars(double g, double alpha, double& beta, double& vj, double& tau) {
@@ -96,10 +112,10 @@ __device__ __forceinline__ void qd_scalars(double g, double alpha, double& beta,
     const double f = fma(-__hiloint2double(sh, dl), q0, 1.0);
     const double q = fma(q0 * f, 1.0 + f, q0);
     tau = __hiloint2double(__double2hiint(q) - (de << 20), __double2loint(q));
-  } else if (g >= 2.3e-308) {
+  } else if (g >= 2.2250738585072014e-308) {  // the smallest normal number
     mu = sqrt(g);
     tau = 1.0 / fma(aa, mu, g);
-  } else {  // zero (or its square is below the normal range, where tau would overflow), or a NaN
+  } else {  // zero or a NaN (qd_rescale has brought any other column into the range)
     beta = g == g ? alpha : g;
     vj = 0.0;
     tau = 0.0;
@@ -152,6 +168,37 @@ __device__ __forceinline__ void qd_st(unsigned long long* p, unsigned long long 
   asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
+// The joint sums and scalars of a step once more, for a column x that qd_rescale has scaled in place:
+// g = x.x and d = x.c from row j down. All threads of the CTA; out of line, so that the step's registers do
+// not pay for it.
+__device__ __noinline__ void qd_scaled_step(const double* x, const double* c, int j, int M, double* red, double* sc) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (warp < 4) {
+    double p0 = 0.0, p1 = 0.0;
+    for (int i = (j & ~31) + tid; i < M; i += 128)
+      if (i >= j) {
+        p0 = fma(x[i], x[i], p0);
+        if (c) p1 = fma(x[i], c[i], p1);
+      }
+    p0 = qd_sum(p0);
+    p1 = qd_sum(p1);
+    if (lane == 0) {
+      red[warp] = p0;
+      red[warp + 4] = p1;
+    }
+  }
+  __syncthreads();
+  if (tid == 0) {
+    double beta, vj, tau;
+    qd_scalars((red[0] + red[1]) + (red[2] + red[3]), x[j], beta, vj, tau);
+    sc[0] = beta;
+    sc[1] = vj;
+    sc[2] = tau;
+    if (c) sc[3] = tau * fma(-beta, c[j], (red[4] + red[5]) + (red[6] + red[7]));
+  }
+  __syncthreads();
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kQdThreads, 3) qrd_kernel(QrdArgs a) {
   pdl_begin();
@@ -164,7 +211,8 @@ __global__ void __launch_bounds__(kQdThreads, 3) qrd_kernel(QrdArgs a) {
   T* xs = cols + (long)a.cols_ub * ld;              // [ld] the column received
   __shared__ T red[8];
   __shared__ T s_sc[4];                             // beta, v_j, tau, the chain column's factor
-  __shared__ int s_abort;
+  __shared__ T s_up;
+  __shared__ int s_abort;                           // 1: a wait ran out, 2: the column is to be scaled
   if (b == 0 && tid == 0 && a.ik >= 0) a.t.bond[z * a.t.nbd + a.ik] = k;
   for (long e = (long)b * kQdThreads + tid; e < a.clear_n; e += (long)G * kQdThreads)
     a.ex_next[z * a.ex_stride + e] = kQdEmpty;
@@ -239,7 +287,7 @@ __global__ void __launch_bounds__(kQdThreads, 3) qrd_kernel(QrdArgs a) {
         for (int u = 0; u < 4; ++u) {
           const int i = base + lane + 32 * u;
           for (int polls = 0; bits[u] == kQdEmpty && polls < kQdPolls; ++polls) bits[u] = qd_ld(src_x + i);
-          if (bits[u] == kQdEmpty) s_abort = 1;
+          if (bits[u] == kQdEmpty) atomicOr(&s_abort, 1);
           xr[u] = QdBits<T>::from(bits[u]);
           if (!one && i < M) xs[i] = xr[u];  // (warp 0)
         }
@@ -260,7 +308,28 @@ __global__ void __launch_bounds__(kQdThreads, 3) qrd_kernel(QrdArgs a) {
         s += __shfl_xor_sync(0xffffffffu, hi ? p0 : p1, 16);
 #pragma unroll
         for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        const T g = __shfl_sync(0xffffffffu, s, 0), d = __shfl_sync(0xffffffffu, s, 16);
+        T g = __shfl_sync(0xffffffffu, s, 0), d = __shfl_sync(0xffffffffu, s, 16);
+        if constexpr (sizeof(T) == 8) {
+          if (qd_out_of_range(g)) {
+            const bool nz = qd_nonzero(xr[0]) || qd_nonzero(xr[1]) || qd_nonzero(xr[2]) || qd_nonzero(xr[3]);
+            const double up = qd_rescale(g, !__any_sync(0xffffffffu, nz));
+            if (up != 1.0) {
+              if (lane == 0) {
+                s_up = up;
+                atomicOr(&s_abort, 2);
+              }
+              p0 = p1 = 0.0;
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                xr[u] *= up;
+                p0 = fma(xr[u], xr[u], p0);
+                p1 = fma(xr[u], cr[u], p1);
+              }
+              g = qd_sum(p0);
+              d = qd_sum(p1);
+            }
+          }
+        }
         T beta, vj, tau;
         qd_scalars(g, __shfl_sync(0xffffffffu, xr[0], j & 31), beta, vj, tau);
         if (crit) {
@@ -317,7 +386,7 @@ __global__ void __launch_bounds__(kQdThreads, 3) qrd_kernel(QrdArgs a) {
               const int i = i0 + 128 * u;
               if (i >= M) break;
               for (int polls = 0; bits[u] == kQdEmpty && polls < kQdPolls; ++polls) bits[u] = qd_ld(src_x + i);
-              if (bits[u] == kQdEmpty) s_abort = 1;
+              if (bits[u] == kQdEmpty) atomicOr(&s_abort, 1);
               const T xi = QdBits<T>::from(bits[u]);
               xs[i] = xi;
               p0 = fma(xi, xi, p0);
@@ -338,6 +407,17 @@ __global__ void __launch_bounds__(kQdThreads, 3) qrd_kernel(QrdArgs a) {
         s += __shfl_xor_sync(0xffffffffu, s, 1);
         s += __shfl_xor_sync(0xffffffffu, s, 2);
         const T g = __shfl_sync(0xffffffffu, s, 0), d = __shfl_sync(0xffffffffu, s, 4);
+        if constexpr (sizeof(T) == 8) {
+          if (qd_out_of_range(g)) {
+            bool nz = false;
+            for (int i = base + lane; i < M; i += 32) nz = nz || (i >= j && qd_nonzero(x[i]));
+            const double up = qd_rescale(g, !__any_sync(0xffffffffu, nz));
+            if (up != 1.0 && lane == 0) {
+              s_up = up;
+              atomicOr(&s_abort, 2);
+            }
+          }
+        }
         T beta, vj, tau;
         qd_scalars(g, x[j], beta, vj, tau);
         const T cj = crit ? crit[j] : T(0);
@@ -355,9 +435,39 @@ __global__ void __launch_bounds__(kQdThreads, 3) qrd_kernel(QrdArgs a) {
       }
     }
     __syncthreads();
+    bool scaled = false;
     if (s_abort) {  // every thread sees it: it was set before the barrier
-      if (tid == 0) atomicExch(&a.t.istat[z * a.t.nis + IS_STATUS], (int)TTM_ERR_TIMEOUT);
-      return;
+      if (s_abort & 1) {
+        if (tid == 0) atomicExch(&a.t.istat[z * a.t.nis + IS_STATUS], (int)TTM_ERR_TIMEOUT);
+        return;
+      }
+      if constexpr (sizeof(T) == 8) {
+        const double up = s_up;
+        scaled = true;
+        T* xw = mine ? cols + lj * ld : xs;
+        if (mine || !narrow || !one)
+          for (int i = j + tid; i < M; i += kQdThreads) xw[i] *= up;
+        __syncthreads();
+        if (tid == 0) s_abort = 0;
+        if (!narrow) {
+          qd_scaled_step(x, crit, j, M, red, s_sc);
+          if (tid == 0 && crit) R[(long)j * N + nxt] = fma(-s_sc[3], s_sc[1], crit[j]);
+        }
+        if (have && warp != 0) {
+          dme = T(0);
+          if (narrow) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const int i = base + lane + 32 * u;
+              xr[u] *= up;
+              if (i < M) dme = fma(xr[u], am[i], dme);
+            }
+          } else {
+            for (int i = base + lane; i < M; i += 32) dme = fma(i >= j ? x[i] : T(0), am[i], dme);
+          }
+          dme = qd_sum(dme);
+        }
+      }
     }
     if (!narrow && crit && warp < 4) {
       const T f = s_sc[3];
@@ -370,6 +480,7 @@ __global__ void __launch_bounds__(kQdThreads, 3) qrd_kernel(QrdArgs a) {
     }
     if (mine && tid == 0) {
       T rd = s_sc[0];
+      if (scaled) rd /= s_up;
       if constexpr (sizeof(T) == 4) rd += rd < T(0) ? -a.ridge : a.ridge;
       R[(long)j * N + j] = rd;
       if (V) {

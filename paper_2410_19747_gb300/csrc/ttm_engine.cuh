@@ -232,8 +232,10 @@ class Engine {
         const cudaError_t e = launch_tc_gemm(hs_.stream, f, Z_, nbatch, M_ub, N_ub, K_ub, kscale_buf,
                                              split_digits(), d_tc_, d_istat_ + IS_STATUS, d_stat_ + ST_GFLOPS,
                                              tab_.ns);
-        if (e != cudaSuccess)
+        if (e != cudaSuccess) {
+          cudaGetLastError();
           throw Error(TTM_ERR_CUDA, std::string("tensor-core GEMM, ") + tc_failed_step() + ": " + cudaGetErrorString(e));
+        }
         launches_ += 2;
       } else {
         TTM_CUDA(launch_dgemm(hs_.stream, f, Z_ * nbatch, nbatch, M_ub, N_ub, K_ub, hs_.num_sms, d_stat_ + ST_GFLOPS,

@@ -21,9 +21,11 @@ struct Error : std::runtime_error {
 #define TTM_CUDA(call)                                                                    \
   do {                                                                                    \
     cudaError_t e_ = (call);                                                              \
-    if (e_ != cudaSuccess)                                                                \
+    if (e_ != cudaSuccess) {                                                              \
+      cudaGetLastError(); /* reported here: not left for the caller's next CUDA call */   \
       throw ::ttm::Error(TTM_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_) + \
                                            " (" + __FILE__ + ":" + std::to_string(__LINE__) + ")"); \
+    }                                                                                     \
   } while (0)
 
 constexpr int kMaxBond = 8192;         // largest bond the planner accepts

@@ -375,11 +375,12 @@ void Engine::swap_exact(int x, int y, int bl, int bm, int br, int nbnd, int pb, 
     q1.m = n;
     q1.n = m;
     q1.ik = pb;
+    q1.scaled = 1;
     qrd<double>(q1, n_ub, m_ub);
   });
   if (!launch_) return;
   TTM_CUDA(launch_pdl(pre_norm_kernel<double>, dim3(cdiv(p_ub, 8), Z_), dim3(256), 0, hs_.stream,
-                      PreNormArgs{tab_, L, L, ws(WS_NRM), m, p}));
+                      PreNormArgs{tab_, L, L, ws(WS_NRM), m, p, 1}));
   PreOrderArgs oa{tab_, ws(WS_NRM), ws(WS_SORT), ws(WS_PERM), m, n, p, nbnd, 0.0, (int)cap, wslot, 2, -1,
                   svd_rec(cur_svd_), svd_stride(), 0};
   TTM_CUDA(launch_pdl(pre_order_kernel, dim3(Z_), dim3(pow2_threads(p_ub)), 0, hs_.stream, oa));
@@ -448,7 +449,7 @@ void Engine::swap_pre(int x, int y, int bl, int bm, int br, int nbnd, int nprov,
     timed(1, [&] { jacobi_pre(ja, p_ub); });
     // its column norms in descending order, the provisional rank, and V
     TTM_CUDA(launch_pdl(pre_norm_kernel<float>, dim3(cdiv(p_ub, 8), Z_), dim3(256), 0, hs_.stream,
-                        PreNormArgs{tab_, X, X, ws(WS_NRM), m, p}));
+                        PreNormArgs{tab_, X, X, ws(WS_NRM), m, p, 0}));
     PreOrderArgs oa{tab_, ws(WS_NRM), ws(WS_SORT), ws(WS_PERM), m, n, p, nprov, opt_.eps, (int)cap, -1, 0, ikeep,
                     nullptr, 0, 1};
     TTM_CUDA(launch_pdl(pre_order_kernel, dim3(Z_), dim3(pow2_threads(p_ub)), 0, hs_.stream, oa));
@@ -494,7 +495,7 @@ void Engine::swap_pre(int x, int y, int bl, int bm, int br, int nbnd, int nprov,
     timed(3, [&] { jacobi_res<double>(j64, m_ub, p_ub, nblk_pad_ub); });
     // 5. final order, Eq. eps + cap, new carriages
     TTM_CUDA(launch_pdl(pre_norm_kernel<double>, dim3(cdiv(p_ub, 8), Z_), dim3(256), 0, hs_.stream,
-                        PreNormArgs{tab_, w[0], w[1], ws(WS_NRM), m, p}));
+                        PreNormArgs{tab_, w[0], w[1], ws(WS_NRM), m, p, 0}));
     PreOrderArgs oa{tab_, ws(WS_NRM), ws(WS_SORT), ws(WS_PERM), m, n, p, nbnd, opt_.eps, (int)cap, wslot, 1, ikeep,
                     svd_rec(cur_svd_), svd_stride(), 1};
     TTM_CUDA(launch_pdl(pre_order_kernel, dim3(Z_), dim3(pow2_threads(p_ub)), 0, hs_.stream, oa));

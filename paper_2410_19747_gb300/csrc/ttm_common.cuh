@@ -28,8 +28,9 @@ struct Tables {
   int nz;  // products in this launch
   double* pre;  // [z][kPreSlots] state of the preconditioned Swap SVD (ttm_pre.cuh), or nullptr
 };
-// pre slots: last correction of Newton steps 1, 2, 3; 1 / ||Theta||_F^2; max |R1|
-enum { PR_RES = 0, PR_ITRACE = 3, PR_ABSMAX = 4, kPreSlots = 8 };
+// pre slots: last correction of Newton steps 1, 2, 3; 1 / ||Theta||_F^2; max |R1|; W and its norms are
+// those of Theta times 2^-PR_EXP
+enum { PR_RES = 0, PR_ITRACE = 3, PR_ABSMAX = 4, PR_EXP = 5, kPreSlots = 8 };
 
 __device__ __forceinline__ int bondv(const Tables& t, int z, int id) {
   return id < 0 ? 1 : t.bond[z * t.nbd + id];

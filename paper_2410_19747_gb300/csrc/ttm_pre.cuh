@@ -50,6 +50,14 @@ constexpr float kPreBig = 1e-3f;    // a sweep without a coupling above this is 
                                     // the same time per product.)
 constexpr float kPreRidge = 1e-15f; // added to the diagonal of R2 (max |R1| = 1): no column of X vanishes
 
+// Binary exponent that W leaves out: the squares of its columns stay in the float64 range whatever the
+// norm of Theta. 0 for a Theta of ordinary size.
+__device__ __forceinline__ int pre_exp(double absmax) {
+  const int e = qd_scale_exp(absmax);
+  return e > 256 || e < -256 ? e : 0;
+}
+__device__ __forceinline__ double pre_pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }  // |e| <= 1000
+
 // G = W^T W (batch 0, K = m) and M = V^T V (batch 1, K = p), upper triangles.
 struct PreGramFn {
   Tables t;
@@ -91,7 +99,7 @@ struct PreApplyFn {
     return g;
   }
 };
-// W = L V, all column-major (L m x p, V p x p).
+// W = L V 2^-e, all column-major (L m x p, V p x p).
 struct PreProductFn {
   Tables t;
   int bl, bv, bw;
@@ -103,19 +111,21 @@ struct PreProductFn {
     g.A = MatRef{bufp(t, z, bl), 1, M};
     g.B = MatRef{bufp(t, z, bv), 1, P};
     g.C = OutRef{bufp(t, z, bw), 1, M};
-    g.alpha = 1.0; g.beta = 0.0; g.upper = 0;
+    g.alpha = pre_pow2(-(int)t.pre[z * kPreSlots + PR_EXP]); g.beta = 0.0; g.upper = 0;
     return g;
   }
 };
 
 // ---------------------------------------------------------------- norms, order, Eq. eps
-// Squared column norms: of X (float, times the scale that the second QR took out) or of W (in the
-// buffer where the Newton steps left it). One warp per column.
+// Squared column norms: of X (float, times the scale that the second QR took out and W does not) or of W
+// (in the buffer where the Newton steps left it; scaled: of L, which is not scaled itself). One warp per
+// column.
 struct PreNormArgs {
   Tables t;
   int bw, bw2;      // W's two buffers; float: bw = X
   int bnrm;
   Dim m, p;
+  int scaled;
 };
 template <typename T>
 __global__ void pre_norm_kernel(PreNormArgs a) {
@@ -132,11 +142,21 @@ __global__ void pre_norm_kernel(PreNormArgs a) {
       s = fma(v, v, s);
     }
     s = warp_sum(s);
-    s = ldexp(s, 2 * qd_scale_exp(a.t.pre[z * kPreSlots + PR_ABSMAX]));
+    const double mx = a.t.pre[z * kPreSlots + PR_ABSMAX];
+    s = ldexp(s, 2 * (qd_scale_exp(mx) - pre_exp(mx)));
   } else {
     const int m = a.m.eval(a.t, z);
     const double* x = bufp(a.t, z, pre_where(a.t, z) ? a.bw2 : a.bw) + (long)j * m;
-    for (int r = lane; r < m; r += 32) s = fma(x[r], x[r], s);
+    const int e = a.scaled ? pre_exp(a.t.pre[z * kPreSlots + PR_ABSMAX]) : 0;
+    if (e == 0) {
+      for (int r = lane; r < m; r += 32) s = fma(x[r], x[r], s);
+    } else {
+      const double inv = pre_pow2(-e);
+      for (int r = lane; r < m; r += 32) {
+        const double v = x[r] * inv;
+        s = fma(v, v, s);
+      }
+    }
     s = warp_sum(s);
   }
   if (lane == 0) bufp(a.t, z, a.bnrm)[j] = s;
@@ -255,9 +275,12 @@ __global__ void __launch_bounds__(1024) pre_order_kernel(PreOrderArgs a) {
     if (!a.record) {
       for (int q = 0; q < 3; ++q) pr[PR_RES + q] = 0.0;
       pr[PR_ITRACE] = total > 0.0 ? 1.0 / total : 0.0;
+      pr[PR_EXP] = (double)pre_exp(pr[PR_ABSMAX]);
       return;
     }
-    const double w = s_tail;
+    if (a.record == 2) pr[PR_EXP] = 0.0;
+    const int ex = (int)pr[PR_EXP];
+    const double w = ex == 0 ? s_tail : ldexp(s_tail, 2 * ex);
     st[ST_WSUM] += w;
     st[ST_WSQRT] += sqrt(w);
     if (a.wslot >= 0) st[a.wslot] = w;
@@ -652,12 +675,13 @@ __global__ void pre_rescue_kernel(PreRescueArgs a) {
   if (!bad) return;
   const int m = a.m.eval(a.t, z), p = a.p.eval(a.t, z);
   const double* L = bufp(a.t, z, a.bl);
+  const double inv = pre_pow2(-(int)a.t.pre[z * kPreSlots + PR_EXP]);
   double* W = bufp(a.t, z, a.bw);
   for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < (long)m * p; e += (long)gridDim.x * blockDim.x)
-    W[e] = L[e];
+    W[e] = L[e] * inv;
 }
 
-// New left carriage, row-major [m][k]: column perm[j] of W. 32 x 32 tiles through shared memory.
+// New left carriage, row-major [m][k]: column perm[j] of W 2^e. 32 x 32 tiles through shared memory.
 struct PreLeftArgs {
   Tables t;
   int bw, bw2, bperm, bout;
@@ -672,6 +696,7 @@ __global__ void __launch_bounds__(256) pre_left_kernel(PreLeftArgs a) {
   if (r0 >= m || j0 >= k) return;
   __shared__ double tile[32][33];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int ex = (int)a.t.pre[z * kPreSlots + PR_EXP];
   const double* W = bufp(a.t, z, pre_where(a.t, z) ? a.bw2 : a.bw);
   const int* perm = reinterpret_cast<const int*>(bufp(a.t, z, a.bperm));
   for (int q = ty; q < 32; q += 8)
@@ -679,7 +704,10 @@ __global__ void __launch_bounds__(256) pre_left_kernel(PreLeftArgs a) {
   __syncthreads();
   double* out = bufp(a.t, z, a.bout);
   for (int q = ty; q < 32; q += 8)
-    if (r0 + q < m && j0 + tx < k) out[(long)(r0 + q) * k + j0 + tx] = tile[tx][q];
+    if (r0 + q < m && j0 + tx < k) {
+      const double v = tile[tx][q];
+      out[(long)(r0 + q) * k + j0 + tx] = ex == 0 ? v : v * pre_pow2(ex);
+    }
 }
 
 }  // namespace ttm

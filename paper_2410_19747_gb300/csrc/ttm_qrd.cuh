@@ -71,19 +71,19 @@ __device__ __forceinline__ T qd_sum4(const T (&s)[4], int lane) {
 }
 
 // A float64 column whose squared norm g is below the normal range (but the column is not zero), or finite
-// and at least 2^1020 (its tau would leave the range), is scaled by this power of two before its scalars are
-// formed; beta, v and tau are then those of the scaled column, and only the diagonal entry of R is scaled
-// back. 1 for every other column, a zero, an infinite and a NaN one included.
+// and at least 2^1020 (its tau would leave the range), is scaled by a power of two that brings its largest
+// entry near 1 before its scalars are formed; beta, v and tau are then those of the scaled column, and only
+// the diagonal entry of R is scaled back. Every other column, a zero, an infinite and a NaN one included,
+// stays as it is. mag: the largest qd_mag of the column.
 __device__ __forceinline__ bool qd_out_of_range(double g) {  // g >= 0 or a NaN
   return (unsigned)(__double2hiint(g) - 0x00100000) >= (unsigned)(0x7fb00000 - 0x00100000);
 }
-__device__ __forceinline__ double qd_rescale(double g, bool zero) {
-  const int hi = __double2hiint(g);
-  if (zero || (hi & 0x7fffffff) >= 0x7ff00000) return 1.0;
-  return __hiloint2double(hi < 0x00100000 ? (1023 + 800) << 20 : (1023 - 512) << 20, 0);
+__device__ __forceinline__ unsigned qd_mag(double x) {  // orders like |x| up to a factor of 1 + 2^-20; 0 for 0 only
+  return (__double2hiint(x) & 0x7fffffff) | (__double2loint(x) != 0);
 }
-__device__ __forceinline__ bool qd_nonzero(double x) {
-  return ((__double2hiint(x) & 0x7fffffff) | __double2loint(x)) != 0;
+__device__ __forceinline__ double qd_rescale(double g, unsigned mag) {
+  if (mag == 0 || (__double2hiint(g) & 0x7fffffff) >= 0x7ff00000) return 1.0;
+  return __hiloint2double(min(2023, 2046 - (int)(mag >> 20)) << 20, 0);
 }
 
 // beta, v_j and tau of a column with squared norm g and leading entry alpha. A column that counts as
@@ -311,8 +311,8 @@ __global__ void __launch_bounds__(kQdThreads, 3) qrd_kernel(QrdArgs a) {
         T g = __shfl_sync(0xffffffffu, s, 0), d = __shfl_sync(0xffffffffu, s, 16);
         if constexpr (sizeof(T) == 8) {
           if (qd_out_of_range(g)) {
-            const bool nz = qd_nonzero(xr[0]) || qd_nonzero(xr[1]) || qd_nonzero(xr[2]) || qd_nonzero(xr[3]);
-            const double up = qd_rescale(g, !__any_sync(0xffffffffu, nz));
+            const unsigned mag = max(max(qd_mag(xr[0]), qd_mag(xr[1])), max(qd_mag(xr[2]), qd_mag(xr[3])));
+            const double up = qd_rescale(g, __reduce_max_sync(0xffffffffu, mag));
             if (up != 1.0) {
               if (lane == 0) {
                 s_up = up;
@@ -409,9 +409,10 @@ __global__ void __launch_bounds__(kQdThreads, 3) qrd_kernel(QrdArgs a) {
         const T g = __shfl_sync(0xffffffffu, s, 0), d = __shfl_sync(0xffffffffu, s, 4);
         if constexpr (sizeof(T) == 8) {
           if (qd_out_of_range(g)) {
-            bool nz = false;
-            for (int i = base + lane; i < M; i += 32) nz = nz || (i >= j && qd_nonzero(x[i]));
-            const double up = qd_rescale(g, !__any_sync(0xffffffffu, nz));
+            unsigned mag = 0;
+            for (int i = base + lane; i < M; i += 32)
+              if (i >= j) mag = max(mag, qd_mag(x[i]));
+            const double up = qd_rescale(g, __reduce_max_sync(0xffffffffu, mag));
             if (up != 1.0 && lane == 0) {
               s_up = up;
               atomicOr(&s_abort, 2);

@@ -128,11 +128,10 @@ __device__ __forceinline__ long oz_off_b(int r, int k, int nkc, int S) {
 // x 2^sh as a 64-bit integer, rounded to nearest (|x| 2^sh < 2^62), by integer arithmetic.
 __device__ __forceinline__ long long oz_fixed(long long bits, int sh) {
   const int ef = (int)((bits >> 52) & 0x7ff);
-  if (ef == 0) return 0;  // zero (subnormals count as zero)
-  const long long m = (bits & 0xfffffffffffffll) | 0x10000000000000ll;
-  const int s = ef - 1075 + sh;  // x 2^sh = +-m 2^s
+  const long long m = (bits & 0xfffffffffffffll) | (ef != 0 ? 0x10000000000000ll : 0ll);
+  const int s = max(ef, 1) - 1075 + sh;  // x 2^sh = +-m 2^s
   long long v;
-  if (s >= 0) v = m << min(s, 9);
+  if (s >= 0) v = m << min(s, 62);  // (beyond 9 for subnormal numbers only)
   else if (s < -54) v = 0;
   else v = ((m >> (-s - 1)) + 1) >> 1;
   return bits < 0 ? -v : v;
@@ -174,9 +173,11 @@ __global__ void __launch_bounds__(256) oz_prep_kernel(OzArgs<F> a, int mpad, int
       for (int u = 0; u < 8; ++u) {
         const int k = k0 + u;
         if (k < K) {
-          const int ef = (__double2hiint(p[(long)r * rs + (long)k * ks]) >> 20) & 0x7ff;
+          const unsigned long long x = (unsigned long long)__double_as_longlong(p[(long)r * rs + (long)k * ks]) << 1;
+          const int ef = (int)(x >> 53);
           const int qq = q ? (which == 0 ? -q[k] : q[k]) : 0;
           if (ef != 0) e = max(e, ef == 0x7ff ? kOzExpNaN : ef - 1022 + qq);
+          else if (x != 0) e = max(e, 63 - __clzll((long long)x) - 1074 + qq);  // subnormal
         }
       }
   if (e != kOzExpNone) atomicMax(&s_e[rl], e);

@@ -375,7 +375,6 @@ void Engine::swap_exact(int x, int y, int bl, int bm, int br, int nbnd, int pb, 
     q1.m = n;
     q1.n = m;
     q1.ik = pb;
-    q1.scaled = 1;
     qrd<double>(q1, n_ub, m_ub);
   });
   if (!launch_) return;

@@ -29,7 +29,7 @@ struct Tables {
   double* pre;  // [z][kPreSlots] state of the preconditioned Swap SVD (ttm_pre.cuh), or nullptr
 };
 // pre slots: last correction of Newton steps 1, 2, 3; 1 / ||Theta||_F^2; max |R1|; W and its norms are
-// those of Theta times 2^-PR_EXP
+// those of Theta times 2^-PR_EXP (an int in the slot's first word)
 enum { PR_RES = 0, PR_ITRACE = 3, PR_ABSMAX = 4, PR_EXP = 5, kPreSlots = 8 };
 
 __device__ __forceinline__ int bondv(const Tables& t, int z, int id) {
@@ -73,6 +73,10 @@ __device__ __forceinline__ int pre_where(const Tables& t, int z) {
 }
 __device__ __forceinline__ bool pre_failed(const Tables& t, int z) {
   return !(t.pre[z * kPreSlots + PR_RES + 2] <= kNewtonConverged);
+}
+
+__device__ __forceinline__ int* pre_exp_slot(const Tables& t, int z) {
+  return reinterpret_cast<int*>(t.pre + z * kPreSlots + PR_EXP);
 }
 
 // A dimension written as mul * bond[id] (id < 0 means the constant mul).

@@ -52,9 +52,10 @@ constexpr float kPreRidge = 1e-15f; // added to the diagonal of R2 (max |R1| = 1
 
 // Binary exponent that W leaves out: the squares of its columns stay in the float64 range whatever the
 // norm of Theta. 0 for a Theta of ordinary size.
-__device__ __forceinline__ int pre_exp(double absmax) {
-  const int e = qd_scale_exp(absmax);
-  return e > 256 || e < -256 ? e : 0;
+__device__ __forceinline__ int pre_exp(double absmax) {  // integer arithmetic: it lies on the chain of a Swap
+  const int hi = __double2hiint(absmax), e = (hi >> 20) - 1022;  // as frexp
+  const bool ordinary = (e <= 256 && e >= -256) || hi == 0 || e > 1024;  // (zero, infinite)
+  return ordinary ? 0 : max(-1000, min(1000, e));
 }
 __device__ __forceinline__ double pre_pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }  // |e| <= 1000
 
@@ -111,21 +112,21 @@ struct PreProductFn {
     g.A = MatRef{bufp(t, z, bl), 1, M};
     g.B = MatRef{bufp(t, z, bv), 1, P};
     g.C = OutRef{bufp(t, z, bw), 1, M};
-    g.alpha = pre_pow2(-(int)t.pre[z * kPreSlots + PR_EXP]); g.beta = 0.0; g.upper = 0;
+    g.alpha = pre_pow2(-*pre_exp_slot(t, z)); g.beta = 0.0; g.upper = 0;
     return g;
   }
 };
 
 // ---------------------------------------------------------------- norms, order, Eq. eps
 // Squared column norms: of X (float, times the scale that the second QR took out and W does not) or of W
-// (in the buffer where the Newton steps left it; scaled: of L, which is not scaled itself). One warp per
-// column.
+// (in the buffer where the Newton steps left it). One warp per column. l1: the sums of the magnitudes instead,
+// which say whether a column vanishes or is not finite whatever its size.
 struct PreNormArgs {
   Tables t;
   int bw, bw2;      // W's two buffers; float: bw = X
   int bnrm;
   Dim m, p;
-  int scaled;
+  int l1;
 };
 template <typename T>
 __global__ void pre_norm_kernel(PreNormArgs a) {
@@ -147,16 +148,10 @@ __global__ void pre_norm_kernel(PreNormArgs a) {
   } else {
     const int m = a.m.eval(a.t, z);
     const double* x = bufp(a.t, z, pre_where(a.t, z) ? a.bw2 : a.bw) + (long)j * m;
-    const int e = a.scaled ? pre_exp(a.t.pre[z * kPreSlots + PR_ABSMAX]) : 0;
-    if (e == 0) {
+    if (a.l1)
+      for (int r = lane; r < m; r += 32) s += fabs(x[r]);
+    else
       for (int r = lane; r < m; r += 32) s = fma(x[r], x[r], s);
-    } else {
-      const double inv = pre_pow2(-e);
-      for (int r = lane; r < m; r += 32) {
-        const double v = x[r] * inv;
-        s = fma(v, v, s);
-      }
-    }
     s = warp_sum(s);
   }
   if (lane == 0) bufp(a.t, z, a.bnrm)[j] = s;
@@ -191,6 +186,8 @@ __global__ void __launch_bounds__(1024) pre_order_kernel(PreOrderArgs a) {
   int np = 32;
   while (np < p) np <<= 1;
   const double* nr = bufp(a.t, z, a.bnrm);
+  const double absmax = a.t.pre[z * kPreSlots + PR_ABSMAX];
+  const int ex = a.record == 1 ? *pre_exp_slot(a.t, z) : a.record == 0 ? pre_exp(absmax) : 0;
   int nan_seen = 0;
   if (tid < np) {
     long long k = -2;  // padding, after everything
@@ -275,11 +272,10 @@ __global__ void __launch_bounds__(1024) pre_order_kernel(PreOrderArgs a) {
     if (!a.record) {
       for (int q = 0; q < 3; ++q) pr[PR_RES + q] = 0.0;
       pr[PR_ITRACE] = total > 0.0 ? 1.0 / total : 0.0;
-      pr[PR_EXP] = (double)pre_exp(pr[PR_ABSMAX]);
+      *pre_exp_slot(a.t, z) = ex;
       return;
     }
-    if (a.record == 2) pr[PR_EXP] = 0.0;
-    const int ex = (int)pr[PR_EXP];
+    if (a.record == 2) *pre_exp_slot(a.t, z) = 0;
     const double w = ex == 0 ? s_tail : ldexp(s_tail, 2 * ex);
     st[ST_WSUM] += w;
     st[ST_WSQRT] += sqrt(w);
@@ -675,7 +671,7 @@ __global__ void pre_rescue_kernel(PreRescueArgs a) {
   if (!bad) return;
   const int m = a.m.eval(a.t, z), p = a.p.eval(a.t, z);
   const double* L = bufp(a.t, z, a.bl);
-  const double inv = pre_pow2(-(int)a.t.pre[z * kPreSlots + PR_EXP]);
+  const double inv = pre_pow2(-*pre_exp_slot(a.t, z));
   double* W = bufp(a.t, z, a.bw);
   for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < (long)m * p; e += (long)gridDim.x * blockDim.x)
     W[e] = L[e] * inv;
@@ -696,7 +692,7 @@ __global__ void __launch_bounds__(256) pre_left_kernel(PreLeftArgs a) {
   if (r0 >= m || j0 >= k) return;
   __shared__ double tile[32][33];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const int ex = (int)a.t.pre[z * kPreSlots + PR_EXP];
+  const int ex = *pre_exp_slot(a.t, z);
   const double* W = bufp(a.t, z, pre_where(a.t, z) ? a.bw2 : a.bw);
   const int* perm = reinterpret_cast<const int*>(bufp(a.t, z, a.bperm));
   for (int q = ty; q < 32; q += 8)

@@ -74,7 +74,8 @@ __device__ __forceinline__ T qd_sum4(const T (&s)[4], int lane) {
 // and at least 2^1020 (its tau would leave the range), is scaled by a power of two that brings its largest
 // entry near 1 before its scalars are formed; beta, v and tau are then those of the scaled column, and only
 // the diagonal entry of R is scaled back. Every other column, a zero, an infinite and a NaN one included,
-// stays as it is. mag: the largest qd_mag of the column.
+// stays as it is. mag: the largest qd_mag of the column. The test is made only where qd_scalars has left its
+// main branch (as a comparison of its own on the chain it cost 1 to 3 % of a product).
 __device__ __forceinline__ bool qd_out_of_range(double g) {  // g >= 0 or a NaN
   return (unsigned)(__double2hiint(g) - 0x00100000) >= (unsigned)(0x7fb00000 - 0x00100000);
 }
@@ -87,13 +88,15 @@ __device__ __forceinline__ double qd_rescale(double g, unsigned mag) {
 }
 
 // beta, v_j and tau of a column with squared norm g and leading entry alpha. A column that counts as
-// zero has tau = 0; a NaN travels on in beta.
-__device__ __forceinline__ void qd_scalars(double g, double alpha, double& beta, double& vj, double& tau) {
+// zero has tau = 0; a NaN travels on in beta. rescale(g, alpha): called for a g out of range; may scale the
+// column and replace both.
+template <class Rescale>
+__device__ __forceinline__ void qd_scalars(double g, double alpha, double& beta, double& vj, double& tau, Rescale&& rescale) {
   const int hi = __double2hiint(g), lo = __double2loint(g), ex = (hi >> 20) - 1023;
-  const bool neg = __double2hiint(alpha) < 0;
-  const double aa = __hiloint2double(__double2hiint(alpha) & 0x7fffffff, __double2loint(alpha));
+  bool neg = __double2hiint(alpha) < 0;
+  double aa = __hiloint2double(__double2hiint(alpha) & 0x7fffffff, __double2loint(alpha));
   double mu, D;
-  if (ex > -900 && ex < 900) {  // (a negative or NaN g is outside)
+  if (__builtin_expect(ex > -900 && ex < 900, 1)) {  // (a negative or NaN g is outside)
     const int h = ex >> 1;
     const int gh = hi - ((2 * h) << 20);  // g 2^(-2h) in [1, 4)
     const double gs = __hiloint2double(gh, lo);
@@ -112,20 +115,27 @@ __device__ __forceinline__ void qd_scalars(double g, double alpha, double& beta,
     const double f = fma(-__hiloint2double(sh, dl), q0, 1.0);
     const double q = fma(q0 * f, 1.0 + f, q0);
     tau = __hiloint2double(__double2hiint(q) - (de << 20), __double2loint(q));
-  } else if (g >= 2.2250738585072014e-308) {  // the smallest normal number
+  } else {
+    if (qd_out_of_range(g)) {
+      rescale(g, alpha);
+      neg = __double2hiint(alpha) < 0;
+      aa = fabs(alpha);
+    }
+    if (!(g >= 2.2250738585072014e-308)) {  // (the smallest normal number) zero, or a NaN
+      beta = g == g ? alpha : g;
+      vj = 0.0;
+      tau = 0.0;
+      return;
+    }
     mu = sqrt(g);
     tau = 1.0 / fma(aa, mu, g);
-  } else {  // zero or a NaN (qd_rescale has brought any other column into the range)
-    beta = g == g ? alpha : g;
-    vj = 0.0;
-    tau = 0.0;
-    return;
   }
   beta = neg ? mu : -mu;
   const double y = aa + mu;
   vj = neg ? -y : y;
 }
-__device__ __forceinline__ void qd_scalars(float g, float alpha, float& beta, float& vj, float& tau) {
+template <class Rescale>
+__device__ __forceinline__ void qd_scalars(float g, float alpha, float& beta, float& vj, float& tau, Rescale&&) {
   if (g > 1e-36f) {  // below (columns of 1e-18 of max |A|) tau would leave the float range
     float r = rsqrtf(g);
     r = fmaf(r * 0.5f, fmaf(-(g * r), r, 1.f), r);
@@ -190,7 +200,7 @@ __device__ __noinline__ void qd_scaled_step(const double* x, const double* c, in
   __syncthreads();
   if (tid == 0) {
     double beta, vj, tau;
-    qd_scalars((red[0] + red[1]) + (red[2] + red[3]), x[j], beta, vj, tau);
+    qd_scalars((red[0] + red[1]) + (red[2] + red[3]), x[j], beta, vj, tau, [](double&, double&) {});
     sc[0] = beta;
     sc[1] = vj;
     sc[2] = tau;
@@ -212,13 +222,14 @@ __global__ void __launch_bounds__(kQdThreads, 3) qrd_kernel(QrdArgs a) {
   __shared__ T red[8];
   __shared__ T s_sc[4];                             // beta, v_j, tau, the chain column's factor
   __shared__ T s_up;
-  __shared__ int s_abort;                           // 1: a wait ran out, 2: the column is to be scaled
+  __shared__ int s_flags;                           // byte 0: a wait ran out, byte 1: the column is to be scaled
+  volatile unsigned char* flags = reinterpret_cast<unsigned char*>(&s_flags);
   if (b == 0 && tid == 0 && a.ik >= 0) a.t.bond[z * a.t.nbd + a.ik] = k;
   for (long e = (long)b * kQdThreads + tid; e < a.clear_n; e += (long)G * kQdThreads)
     a.ex_next[z * a.ex_stride + e] = kQdEmpty;
   const int nl = b < N ? (N - b + G - 1) / G : 0;
   if (nl == 0) return;  // nothing of this product here, and no one waits for this CTA
-  if (tid == 0) s_abort = 0;
+  if (tid == 0) s_flags = 0;
   const double* src = bufp(a.t, z, a.bsrc);
   double scale = 1.0;
   if constexpr (sizeof(T) == 4) {
@@ -287,7 +298,7 @@ __global__ void __launch_bounds__(kQdThreads, 3) qrd_kernel(QrdArgs a) {
         for (int u = 0; u < 4; ++u) {
           const int i = base + lane + 32 * u;
           for (int polls = 0; bits[u] == kQdEmpty && polls < kQdPolls; ++polls) bits[u] = qd_ld(src_x + i);
-          if (bits[u] == kQdEmpty) atomicOr(&s_abort, 1);
+          if (bits[u] == kQdEmpty) flags[0] = 1;
           xr[u] = QdBits<T>::from(bits[u]);
           if (!one && i < M) xs[i] = xr[u];  // (warp 0)
         }
@@ -308,30 +319,28 @@ __global__ void __launch_bounds__(kQdThreads, 3) qrd_kernel(QrdArgs a) {
         s += __shfl_xor_sync(0xffffffffu, hi ? p0 : p1, 16);
 #pragma unroll
         for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        T g = __shfl_sync(0xffffffffu, s, 0), d = __shfl_sync(0xffffffffu, s, 16);
-        if constexpr (sizeof(T) == 8) {
-          if (qd_out_of_range(g)) {
-            const unsigned mag = max(max(qd_mag(xr[0]), qd_mag(xr[1])), max(qd_mag(xr[2]), qd_mag(xr[3])));
-            const double up = qd_rescale(g, __reduce_max_sync(0xffffffffu, mag));
-            if (up != 1.0) {
-              if (lane == 0) {
-                s_up = up;
-                atomicOr(&s_abort, 2);
-              }
-              p0 = p1 = 0.0;
-#pragma unroll
-              for (int u = 0; u < 4; ++u) {
-                xr[u] *= up;
-                p0 = fma(xr[u], xr[u], p0);
-                p1 = fma(xr[u], cr[u], p1);
-              }
-              g = qd_sum(p0);
-              d = qd_sum(p1);
-            }
-          }
-        }
+        const T g = __shfl_sync(0xffffffffu, s, 0);
+        T d = __shfl_sync(0xffffffffu, s, 16);
         T beta, vj, tau;
-        qd_scalars(g, __shfl_sync(0xffffffffu, xr[0], j & 31), beta, vj, tau);
+        qd_scalars(g, __shfl_sync(0xffffffffu, xr[0], j & 31), beta, vj, tau, [&](auto& gr, auto& alpha) {
+          const unsigned mag = max(max(qd_mag(xr[0]), qd_mag(xr[1])), max(qd_mag(xr[2]), qd_mag(xr[3])));
+          const double up = qd_rescale(gr, __reduce_max_sync(0xffffffffu, mag));
+          if (up == 1.0) return;
+          if (lane == 0) {
+            s_up = up;
+            flags[1] = 1;
+          }
+          p0 = p1 = T(0);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            xr[u] *= up;
+            p0 = fma(xr[u], xr[u], p0);
+            p1 = fma(xr[u], cr[u], p1);
+          }
+          gr = qd_sum(p0);
+          d = qd_sum(p1);
+          alpha *= up;
+        });
         if (crit) {
           const T cj = __shfl_sync(0xffffffffu, cr[0], j & 31);
           const T f = tau * fma(-beta, cj, d);
@@ -386,7 +395,7 @@ __global__ void __launch_bounds__(kQdThreads, 3) qrd_kernel(QrdArgs a) {
               const int i = i0 + 128 * u;
               if (i >= M) break;
               for (int polls = 0; bits[u] == kQdEmpty && polls < kQdPolls; ++polls) bits[u] = qd_ld(src_x + i);
-              if (bits[u] == kQdEmpty) atomicOr(&s_abort, 1);
+              if (bits[u] == kQdEmpty) flags[0] = 1;
               const T xi = QdBits<T>::from(bits[u]);
               xs[i] = xi;
               p0 = fma(xi, xi, p0);
@@ -407,20 +416,17 @@ __global__ void __launch_bounds__(kQdThreads, 3) qrd_kernel(QrdArgs a) {
         s += __shfl_xor_sync(0xffffffffu, s, 1);
         s += __shfl_xor_sync(0xffffffffu, s, 2);
         const T g = __shfl_sync(0xffffffffu, s, 0), d = __shfl_sync(0xffffffffu, s, 4);
-        if constexpr (sizeof(T) == 8) {
-          if (qd_out_of_range(g)) {
-            unsigned mag = 0;
-            for (int i = base + lane; i < M; i += 32)
-              if (i >= j) mag = max(mag, qd_mag(x[i]));
-            const double up = qd_rescale(g, __reduce_max_sync(0xffffffffu, mag));
-            if (up != 1.0 && lane == 0) {
-              s_up = up;
-              atomicOr(&s_abort, 2);
-            }
-          }
-        }
         T beta, vj, tau;
-        qd_scalars(g, x[j], beta, vj, tau);
+        qd_scalars(g, x[j], beta, vj, tau, [&](auto& gr, auto&) {  // the step is done again after the barrier
+          unsigned mag = 0;
+          for (int i = base + lane; i < M; i += 32)
+            if (i >= j) mag = max(mag, qd_mag(x[i]));
+          const double up = qd_rescale(gr, __reduce_max_sync(0xffffffffu, mag));
+          if (up != 1.0 && lane == 0) {
+            s_up = up;
+            flags[1] = 1;
+          }
+        });
         const T cj = crit ? crit[j] : T(0);
         const T f = tau * fma(-beta, cj, d);
         if (lane == 0) {
@@ -437,8 +443,8 @@ __global__ void __launch_bounds__(kQdThreads, 3) qrd_kernel(QrdArgs a) {
     }
     __syncthreads();
     bool scaled = false;
-    if (s_abort) {  // every thread sees it: it was set before the barrier
-      if (s_abort & 1) {
+    if (__builtin_expect(s_flags != 0, 0)) {  // every thread sees it: it was set before the barrier
+      if (flags[0]) {
         if (tid == 0) atomicExch(&a.t.istat[z * a.t.nis + IS_STATUS], (int)TTM_ERR_TIMEOUT);
         return;
       }
@@ -449,7 +455,7 @@ __global__ void __launch_bounds__(kQdThreads, 3) qrd_kernel(QrdArgs a) {
         if (mine || !narrow || !one)
           for (int i = j + tid; i < M; i += kQdThreads) xw[i] *= up;
         __syncthreads();
-        if (tid == 0) s_abort = 0;
+        if (tid == 0) s_flags = 0;
         if (!narrow) {
           qd_scaled_step(x, crit, j, M, red, s_sc);
           if (tid == 0 && crit) R[(long)j * N + nxt] = fma(-s_sc[3], s_sc[1], crit[j]);
@@ -481,7 +487,7 @@ __global__ void __launch_bounds__(kQdThreads, 3) qrd_kernel(QrdArgs a) {
     }
     if (mine && tid == 0) {
       T rd = s_sc[0];
-      if (scaled) rd /= s_up;
+      if (scaled) rd *= __hiloint2double(0x7fe00000 - __double2hiint(s_up), 0);  // 1 / s_up, a power of two
       if constexpr (sizeof(T) == 4) rd += rd < T(0) ? -a.ridge : a.ridge;
       R[(long)j * N + j] = rd;
       if (V) {

@@ -178,6 +178,28 @@ __device__ __forceinline__ void qd_st(unsigned long long* p, unsigned long long 
   asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
+// The same for a column in the registers of one warp: its scale and its two sums after it.
+struct QdScaled {
+  double up, g, d;
+};
+__device__ __noinline__ QdScaled qd_scaled_sums(double g, double x0, double x1, double x2, double x3, double c0, double c1,
+                                                double c2, double c3) {
+  const double x[4] = {x0, x1, x2, x3}, c[4] = {c0, c1, c2, c3};
+  unsigned mag = 0;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) mag = max(mag, qd_mag(x[u]));
+  QdScaled q{qd_rescale(g, __reduce_max_sync(0xffffffffu, mag)), 0.0, 0.0};
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const double y = x[u] * q.up;
+    q.g = fma(y, y, q.g);
+    q.d = fma(y, c[u], q.d);
+  }
+  q.g = qd_sum(q.g);
+  q.d = qd_sum(q.d);
+  return q;
+}
+
 // The joint sums and scalars of a step once more, for a column x that qd_rescale has scaled in place:
 // g = x.x and d = x.c from row j down. All threads of the CTA; out of line, so that the step's registers do
 // not pay for it.
@@ -323,23 +345,17 @@ __global__ void __launch_bounds__(kQdThreads, 3) qrd_kernel(QrdArgs a) {
         T d = __shfl_sync(0xffffffffu, s, 16);
         T beta, vj, tau;
         qd_scalars(g, __shfl_sync(0xffffffffu, xr[0], j & 31), beta, vj, tau, [&](auto& gr, auto& alpha) {
-          const unsigned mag = max(max(qd_mag(xr[0]), qd_mag(xr[1])), max(qd_mag(xr[2]), qd_mag(xr[3])));
-          const double up = qd_rescale(gr, __reduce_max_sync(0xffffffffu, mag));
-          if (up == 1.0) return;
+          const QdScaled q = qd_scaled_sums(gr, xr[0], xr[1], xr[2], xr[3], cr[0], cr[1], cr[2], cr[3]);
+          if (q.up == 1.0) return;
           if (lane == 0) {
-            s_up = up;
+            s_up = q.up;
             flags[1] = 1;
           }
-          p0 = p1 = T(0);
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            xr[u] *= up;
-            p0 = fma(xr[u], xr[u], p0);
-            p1 = fma(xr[u], cr[u], p1);
-          }
-          gr = qd_sum(p0);
-          d = qd_sum(p1);
-          alpha *= up;
+          for (int u = 0; u < 4; ++u) xr[u] *= q.up;
+          gr = q.g;
+          d = q.d;
+          alpha *= q.up;
         });
         if (crit) {
           const T cj = __shfl_sync(0xffffffffu, cr[0], j & 31);

@@ -389,7 +389,8 @@ struct PreElimArgs {
   unsigned long long* ex_next;
   long ex_stride, clear_n;
 };
-// 1 / d for a positive d: float32 seed and one cubic step; 0 for a pivot d that is not positive or
+// 1 / d for a positive d: float32 seed and one step of Householder's third-order iteration (as the tau of
+// ttm_qrd.cuh); 0 for a pivot d that is not positive or
 // below 2^-46 of g0, its column's squared norm (by the high words).
 __device__ __forceinline__ double pre_pivot_inv(double d, double g0) {
   const int dh = __double2hiint(d), gh = __double2hiint(g0);

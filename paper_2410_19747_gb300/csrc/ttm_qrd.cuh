@@ -12,8 +12,10 @@
 // float64 instructions as possible:
 //   - column j travels as it is; whoever receives it forms x.x and x.a for its next column in one
 //     joint sum (4 warps, one per sub-partition) and derives beta, tau and v.a = x.a - beta a_j;
-//   - ||x|| and 1 / (||x||^2 + |x_j| ||x||) come from a float32 seed and one cubic step (10 instructions
-//     instead of a square root and two divisions);
+//   - ||x|| and 1 / (||x||^2 + |x_j| ||x||) come from a float32 seed and one step of Householder's
+//     third-order iteration (Householder 1970, ch. 4; 10 instructions instead of a square root and two
+//     divisions). For r near 1 / sqrt(g) and e = 1 - g r^2 it is r (1 + e / 2 + 3 e^2 / 8), for q near 1 / D
+//     and f = 1 - D q it is q (1 + f + f^2): from 2^-20 to rounding. Exponents beyond 900 take CUDA's own;
 //   - columns are dealt out cyclically to G CTAs and stay in shared memory; the owner of column
 //     j + 1 updates and publishes it before its other columns. Receivers poll the data itself (the
 //     exchange buffer is filled with a NaN pattern that arithmetic does not produce), so a step

@@ -38,7 +38,7 @@ L2_BYTES = 129 * 2 ** 20
 MEASURED_TRAFFIC = {
     "jacobi_res_kernel<float> (": (5.58e6, "profiles/jacobi_res_f32_chi512_L20.md: one full-size float32 pass "
                                          "(1024 x 1024, 70 ms); W and V stay in L2"),
-    "oz_gemm_kernel": (7.29e6, "profiles/oz_gemm_gram_chi512_L20.md: one 1024^3 Gram"),
+    "oz_gemm_kernel": (33.7e6, "profiles/oz_gemm_1024.md: one 1024^3 product with a cold L2 (its digits, 33.6 MB)"),
 }
 CPU_BASELINE_S = 40.0   # allowance for the CPU baseline leg in the --time-budget projection
 

@@ -61,7 +61,8 @@ typedef enum {
   TTM_PREC_BF16_SPLIT = 2  /* GEMMs on the tcgen05 tensor cores as the exactly sliced
                               product of bf16 digits (Ozaki scheme; with split_digits = 0 the
                               small GEMMs of a product stay on the float64 pipe, where they
-                              are faster and as accurate): each float64 operand
+                              are faster and as accurate, but in an allocation-free call
+                              without room for the faster kernels): each float64 operand
                               row (column) is scaled by a power of two and split into
                               split_digits digits of 7 bits; the digit products are summed
                               exactly in float32 and combined in float64. 8 digits (the
@@ -113,9 +114,14 @@ typedef struct {
                                jacobi_kernel and newton_steps 0 as well: two QR
                                factorisations and one Jacobi of the triangle (ttm_pre.cuh),
                                or no SVD where eps and the caps drop nothing; what that
-                               does not cover (more than 1024 rows, no room for its
-                               buffers), and 0 beside another option that is not 0: the
-                               general pipeline with 3 passes                            */
+                               does not cover (more than 1024 rows or 2048 columns, an
+                               allocation-free call without room for its buffers, a batch
+                               whose products cannot all be resident: on 152 SMs above 57
+                               products with Swaps of 256 x 256, 25 of 384 x 384, 9 of
+                               512 x 512, 2 of 1024 x 1024), and 0 beside another option
+                               that is not 0: the general pipeline with 3 passes. That
+                               one is faster where a wide spectrum in no order of the
+                               columns is kept to below 1e-16 (eps < 1e-16)              */
   int32_t jacobi_kernel;    /* kernel of the float32 passes: 0 = 3 when the Swap matrix
                                has at most 1024 rows, else 1; 1 = one column per
                                tournament slot (n - 1 grid barriers per sweep); 2 = two
@@ -151,7 +157,8 @@ typedef struct {
   int64_t *bond_trace;         /* caller array or NULL: max chain bond after each Contract */
   int64_t bond_trace_len;      /* in: capacity of bond_trace; out: entries written (N)    */
   int64_t n_kernel_launches;   /* kernels this call launched (all products of a batch)   */
-  int64_t jacobi_launches;     /* float32 one-sided Jacobi launches                       */
+  int64_t jacobi_launches;     /* float32 one-sided Jacobi launches (none for a Swap that
+                                  truncates nothing)                                      */
   double gemm_ms;              /* device time of every GEMM-shaped launch, for a
                                   tensor-core GEMM its exponent and digit kernels included
                                   (profile_kernels = 1), else 0                            */

@@ -208,7 +208,9 @@ class Engine {
   // accurate and faster: the digit product has a floor of about 20 us (one tile's chain of digits, K
   // chunks and epilogue) and fills few SMs with its 128 x 64 tiles. Kernel times of a cube on the
   // pipe / the tensor cores: 192: 13 / 32 us, 256: 35 / 36, 320: 61 / 44, 384: 97 / 48, 768: 780 / 85.
-  // An explicit split_digits always takes the tensor cores.
+  // An explicit split_digits always takes the tensor cores, and so does a plan of the general kernels alone
+  // (base_only_: an allocation-free call whose array has no room for the faster ones), whose GEMMs stay on
+  // the route that they had before there were others.
   static constexpr double kTcMinMnk = 256.0 * 256.0 * 256.0;
   // Digit workspace of a tensor-core GEMM with these upper bounds; every GEMM a step may
   // launch is reserved in both walks (the planning walk launches nothing).
@@ -402,7 +404,8 @@ class Engine {
     ++launches_;
     return true;
   }
-  // The preconditioned Swap SVD (ttm_pre.cuh) covers the default options up to kPreMax rows; an
+  // The preconditioned Swap SVD (ttm_pre.cuh) covers the default options up to kPreMax rows, where the
+  // columns fit the shared memory of the CTAs that can be resident for all products of the batch; an
   // explicit choice of passes, kernel, steps or sweeps takes the general pipeline.
   bool pre_fits(int m_ub, int n_ub) const {
     if (base_only_ || opt_.f32_passes || opt_.jacobi_kernel || opt_.newton_steps || opt_.max_sweeps) return false;

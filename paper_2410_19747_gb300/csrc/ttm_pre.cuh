@@ -1,6 +1,8 @@
 // ttm_pre.cuh -- the Swap SVD (Fig. 1C, Eq. eps) by a preconditioned float32 Jacobi and float64
-// Newton steps on the reduced problem; the default for Swap matrices of at most 1024 rows and
-// 1024 columns of the smaller side.
+// Newton steps on the reduced problem; the default for Swap matrices of at most 1024 rows and 2048
+// columns (Engine::pre_fits), as long as the distributed kernels' CTAs for all products of a batch are
+// resident together: up to 57 products with Swaps of 256 x 256, 25 of 384 x 384, 9 of 512 x 512, 2 of
+// 1024 x 1024 on 152 SMs. What does not fit takes the general pipeline (Engine::swap).
 //
 // Theta is m x n, p = min(m, n):
 //   1. Theta^T = Q1 R1 in float64 (ttm_qrd.cuh); L = R1^T is m x p, Q1 stays as reflectors;
@@ -24,6 +26,13 @@
 //   S_ij = (E_ij (d_i + d_j) / 2 - G'_ij) / (d_i - d_j),  X = I - E / 2 + S,  E = V^T V - I,
 // with the same filters. Measured: corrections 1e-3, 1e-7, 0 for successive steps.
 //
+// Where it is slow: a spectrum of many decades whose L is not graded by columns (the right parts of a chain
+// of square Gaussian cores, say) loses everything below 6e-8 of its largest singular value in step 2; the
+// rotations among those columns are then of order 1, four Newton steps do not converge, and the Swap takes
+// the float64 Jacobi from V = I. A left-canonical Gaussian train times a constant at chi = 256, L = 18,
+// eps = 1e-18: 33 of 153 Swaps, 4.2 s per product, against 0.96 s with f32_passes = 3; at eps = 1e-14, where
+// that tail is dropped, 4 Swaps and 0.85 s. Fields and random products need it for none or one Swap.
+//
 // Bound by latencies: the chains of the two QRs (about 1.3 and 0.7 us per column), of the inner rounds
 // of the Jacobi and of the elimination. Measured per product (GB300) against three float32 passes
 // with V, three to five Newton steps and a saved state: 2D field, d = 4, chi = 64 332 -> 153 ms; 3D
@@ -46,8 +55,10 @@ constexpr int kPreSweeps = 30;      // sweep limit (the Newton steps and the fal
 constexpr double kPreTol = 4 * 5.96e-8;  // times sqrt(p): couplings below are not rotated
 constexpr float kPreBig = 1e-3f;    // a sweep without a coupling above this is the last: the couplings
                                     // it leaves are of the order of its largest one squared. (With 1e-2
-                                    // 5 of 2300 Swaps needed the float64 Jacobi, with 1e-3 none of 8600, at
-                                    // the same time per product.)
+                                    // 5 of 2300 Swaps of fields and random trains, p to 768, needed the
+                                    // float64 Jacobi, with 1e-3 none of 8600, at the same time per product.
+                                    // At chi = 512, p to 1024, five of 435 do with 1e-3, from the Newton
+                                    // steps: see pre_x_kernel.)
 constexpr float kPreRidge = 1e-15f; // added to the diagonal of R2 (max |R1| = 1): no column of X vanishes
 
 // Binary exponent that W leaves out: the squares of its columns stay in the float64 range whatever the
@@ -607,8 +618,11 @@ __global__ void __launch_bounds__(256) pre_x_kernel(PreXArgs a) {
       x = 1.0 - 0.5 * e;
       smax = 0.5 * fabs(e);
     } else {
-      // the first two steps take the couplings after elimination; from then on what the small columns
-      // carry of the large ones is at rounding level and G itself serves (no elimination)
+      // The first two steps take the couplings after elimination. From then on what the small columns
+      // carry of the large ones is at rounding level for most Swaps, and G itself serves. Not where two
+      // small columns were still rotated by 1e-3 or more: that rotation hands on what the other one carried,
+      // the next corrections stay at that size, and the Swap ends in the float64 Jacobi (five of 435 at
+      // chi = 512, 0.6 s each; none with an elimination in steps 2 and 3 too, two more launches per Swap).
       const double g = a.step < 2 ? U[hi + (long)lo * p] : U[lo + (long)hi * p];
       const double di = U[i + (long)i * p], dj = U[j + (long)j * p];
       const double dmax = fmax(di, dj);

@@ -384,7 +384,7 @@ void Engine::swap_exact(int x, int y, int bl, int bm, int br, int nbnd, int pb, 
                   svd_rec(cur_svd_), svd_stride(), 0};
   TTM_CUDA(launch_pdl(pre_order_kernel, dim3(Z_), dim3(pow2_threads(p_ub)), 0, hs_.stream, oa));
   TTM_CUDA(launch_pdl(pre_left_kernel, dim3(cdiv(m_ub, 32), cdiv(k_ub, 32), Z_), dim3(256), 0, hs_.stream,
-                      PreLeftArgs{tab_, L, L, ws(WS_PERM), y, m, nbnd}));
+                      PreLeftArgs{tab_, L, L, ws(WS_PERM), y, m, nbnd, 0}));
   launches_ += 3;
   timed(2, [&] {
     qrd_apply(QrdApplyArgs{tab_, refl, ws(WS_TAU), n, m, -1, -1, -1, nbnd, x, 0, 0}, n_ub, k_ub);
@@ -499,7 +499,7 @@ void Engine::swap_pre(int x, int y, int bl, int bm, int br, int nbnd, int nprov,
                     svd_rec(cur_svd_), svd_stride(), 1};
     TTM_CUDA(launch_pdl(pre_order_kernel, dim3(Z_), dim3(pow2_threads(p_ub)), 0, hs_.stream, oa));
     TTM_CUDA(launch_pdl(pre_left_kernel, dim3(cdiv(m_ub, 32), cdiv(k_ub, 32), Z_), dim3(256), 0, hs_.stream,
-                        PreLeftArgs{tab_, w[0], w[1], ws(WS_PERM), y, m, nbnd}));
+                        PreLeftArgs{tab_, w[0], w[1], ws(WS_PERM), y, m, nbnd, 1}));
     launches_ += 3;
     timed(2, [&] {
       qrd_apply(QrdApplyArgs{tab_, refl, ws(WS_TAU), n, m, v[0], v[1], ws(WS_PERM), nbnd, x, 0, 0}, n_ub, k_ub);

@@ -197,8 +197,9 @@ __global__ void __launch_bounds__(1024) pre_order_kernel(PreOrderArgs a) {
   int np = 32;
   while (np < p) np <<= 1;
   const double* nr = bufp(a.t, z, a.bnrm);
-  const double absmax = a.t.pre[z * kPreSlots + PR_ABSMAX];
-  const int ex = a.record == 1 ? *pre_exp_slot(a.t, z) : a.record == 0 ? pre_exp(absmax) : 0;
+  int ex = 0;
+  if (a.record == 0) ex = pre_exp(a.t.pre[z * kPreSlots + PR_ABSMAX]);
+  if (a.record == 1) ex = *pre_exp_slot(a.t, z);
   int nan_seen = 0;
   if (tid < np) {
     long long k = -2;  // padding, after everything
@@ -286,7 +287,6 @@ __global__ void __launch_bounds__(1024) pre_order_kernel(PreOrderArgs a) {
       *pre_exp_slot(a.t, z) = ex;
       return;
     }
-    if (a.record == 2) *pre_exp_slot(a.t, z) = 0;
     const double w = ex == 0 ? s_tail : ldexp(s_tail, 2 * ex);
     st[ST_WSUM] += w;
     st[ST_WSQRT] += sqrt(w);
@@ -692,12 +692,14 @@ __global__ void pre_rescue_kernel(PreRescueArgs a) {
     W[e] = L[e] * inv;
 }
 
-// New left carriage, row-major [m][k]: column perm[j] of W 2^e. 32 x 32 tiles through shared memory.
+// New left carriage, row-major [m][k]: column perm[j] of W, times 2^e where W leaves it out (scaled). 32 x 32
+// tiles through shared memory.
 struct PreLeftArgs {
   Tables t;
   int bw, bw2, bperm, bout;
   Dim m;
   int ik;
+  int scaled;
 };
 __global__ void __launch_bounds__(256) pre_left_kernel(PreLeftArgs a) {
   pdl_begin();
@@ -707,7 +709,7 @@ __global__ void __launch_bounds__(256) pre_left_kernel(PreLeftArgs a) {
   if (r0 >= m || j0 >= k) return;
   __shared__ double tile[32][33];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const int ex = *pre_exp_slot(a.t, z);
+  const int ex = a.scaled ? *pre_exp_slot(a.t, z) : 0;
   const double* W = bufp(a.t, z, pre_where(a.t, z) ? a.bw2 : a.bw);
   const int* perm = reinterpret_cast<const int*>(bufp(a.t, z, a.bperm));
   for (int q = ty; q < 32; q += 8)
